@@ -143,48 +143,120 @@ void free_handle(sp_handle* h) {
   delete h;
 }
 
+// The pools as the sequence kernel's plan sees them: each column's smallest
+// and largest input, and, while every column's pool is strictly ascending (so
+// no input appears twice and a bitmap counts it once) and fits a 64 x 64 box
+// of the frame, the first frame row of its box.
+struct PoolScan {
+  std::vector<uint32_t> lo, hi, row;
+  bool boxes = true;
+};
+
+PoolScan scan_pools(uint32_t C, uint32_t S, uint32_t W, const uint32_t* idx) {
+  PoolScan p;
+  p.lo.resize(C);
+  p.hi.resize(C);
+  p.row.resize(C);
+  p.boxes = W % 32u == 0u && S <= 4096u;
+  for (uint32_t c = 0; c < C; ++c) {
+    const uint32_t* x = idx + (size_t)c * S;
+    uint32_t mn = x[0], mx = x[0];
+    if (p.boxes) {
+      // one division per row change: `base` is the current row's first input
+      uint32_t base = x[0] / W * W, x0 = x[0] - base, x1 = x0;
+      bool fit = true;
+      p.row[c] = base / W;
+      const uint64_t limit = (uint64_t)base + (uint64_t)64u * W;  // rows of the box
+      for (uint32_t s = 1; s < S && fit; ++s) {
+        fit = x[s] > x[s - 1] && x[s] < limit;
+        if (!fit) break;
+        if (x[s] - base >= W) base = x[s] / W * W;
+        const uint32_t px = x[s] - base;
+        x0 = std::min(x0, px);
+        x1 = std::max(x1, px);
+      }
+      fit = fit && x1 - x0 < 64u && x0 <= 0xffffu && p.row[c] <= 0xffffu;
+      p.boxes = fit;
+      if (fit) {
+        p.lo[c] = x[0];
+        p.hi[c] = x[S - 1];
+        continue;
+      }
+    }
+    for (uint32_t s = 1; s < S; ++s) {
+      mn = std::min(mn, x[s]);
+      mx = std::max(mx, x[s]);
+    }
+    p.lo[c] = mn;
+    p.hi[c] = mx;
+  }
+  return p;
+}
+
 // Decide whether whole frame sequences of this SP can run in one persistent
-// cluster launch: Q CTAs of Cq columns (a multiple of 32) must hold their
-// pools, permanences and input bands in shared memory, and the device must
+// cluster launch, and in which form: Q CTAs of Cq columns (a multiple of 32)
+// must hold their state and input bands in shared memory, and the device must
 // be able to schedule such a cluster.  Failure only disables the path.
 void plan_cluster_path(sp_handle* h, const uint32_t* idx) {
   h->seq_ok = false;
   if (h->cfg.inhibition == SP_INHIBIT_PAPER_LITERAL) return;  // per-frame kernel only
-  uint32_t Q = (h->C + 31u) / 32u;
-  if (Q > sp::kSeqMaxCluster) Q = sp::kSeqMaxCluster;
-  if (Q < 2u) Q = 2u;
+  const PoolScan p = scan_pools(h->C, h->S, h->cfg.input_w, idx);
+  uint32_t Q = std::min((h->C + 31u) / 32u, sp::kSeqMaxCluster);
+  // small SPs: one CTA counts them in less time than a cluster exchanges counts
+  if (h->C <= (uint32_t)sp::kSeqThreads && (uint64_t)h->C * h->S <= kSeqOneCtaSynapses) Q = 1u;
   const uint32_t Cq = (((h->C + Q - 1u) / Q) + 31u) & ~31u;
-  if (Cq > (uint32_t)sp::kSeqThreads) return;  // one column per thread in the decision
-  uint32_t band_max = 4u;
-  for (uint32_t q = 0; q < Q; ++q) {
-    const uint32_t c0 = q * Cq;
-    if (c0 >= h->C) break;
-    const uint32_t c1 = std::min(h->C, c0 + Cq);
-    uint32_t mn = 0xffffffffu, mx = 0u;
-    for (size_t e = (size_t)c0 * h->S; e < (size_t)c1 * h->S; ++e) {
-      mn = std::min(mn, idx[e]);
-      mx = std::max(mx, idx[e]);
+  if (Cq > (uint32_t)sp::kSeqThreads) return;  // a warp's columns are a 32-bit mask
+  const uint32_t wpr = h->cfg.input_w / 32u;
+  auto bytes = [&](uint32_t form, uint32_t* band) {
+    *band = 4u;
+    for (uint32_t c0 = 0; c0 < h->C; c0 += Cq) {
+      const uint32_t c1 = std::min(h->C, c0 + Cq);
+      uint64_t w_lo, w_hi;
+      if (form == sp::kSeqPools) {
+        const uint32_t mn = *std::min_element(p.lo.begin() + c0, p.lo.begin() + c1);
+        const uint32_t mx = *std::max_element(p.hi.begin() + c0, p.hi.begin() + c1);
+        w_lo = mn >> 5;
+        w_hi = (mx >> 5) + 1u;
+      } else {
+        // whole rows, padded to an odd number of words, 64 past the last box's
+        // first, and the word past the end that an unaligned segment reads
+        const uint64_t y0 = *std::min_element(p.row.begin() + c0, p.row.begin() + c1);
+        const uint64_t y1 = *std::max_element(p.row.begin() + c0, p.row.begin() + c1);
+        w_lo = y0 * (wpr | 1u);
+        w_hi = (y1 + 64u) * (wpr | 1u) + 4u;
+      }
+      if (w_hi - w_lo > (kSeqSmemLimit >> 2)) return (size_t)-1;
+      *band = std::max(*band, (uint32_t)((w_hi - w_lo + 3u) & ~uint64_t(3)));
     }
-    const uint32_t w_lo = (mn >> 5) & ~3u;
-    const uint32_t w_hi = ((mx >> 5) + 4u) & ~3u;
-    band_max = std::max(band_max, w_hi - w_lo);
+    return sp::seq_smem_bytes(form, Q, h->C, h->S, Cq, *band);
+  };
+  uint32_t band[3] = {0, 0, 0};
+  size_t smem[3] = {bytes(sp::kSeqPools, &band[0]), (size_t)-1, (size_t)-1};
+  if (p.boxes) {
+    smem[1] = bytes(sp::kSeqWindow, &band[1]);
+    smem[2] = bytes(sp::kSeqWindowL2, &band[2]);
   }
-  const size_t smem = sp::seq_smem_bytes(h->C, h->S, Cq, band_max);
-  if (smem > kSeqSmemLimit) return;
-  if (sp::seq_kernel_init(smem) != cudaSuccess) {
+  const uint32_t order[2][3] = {{sp::kSeqWindow, sp::kSeqWindowL2, sp::kSeqPools},
+                                {sp::kSeqPools, sp::kSeqWindow, sp::kSeqWindowL2}};
+  uint32_t form = 3u;
+  for (uint32_t f : order[h->S >= kSeqWindowSynapses ? 0 : 1])
+    if (form == 3u && smem[f] <= kSeqSmemLimit) form = f;
+  if (form == 3u) return;
+  if (sp::seq_kernel_init(form, kSeqSmemLimit) != cudaSuccess) {
     cudaGetLastError();
     return;
   }
   int clusters = 0;
-  if (sp::seq_max_active_clusters(Q, smem, &clusters) != cudaSuccess || clusters < 1) {
+  if (sp::seq_max_active_clusters(form, Q, smem[form], &clusters) != cudaSuccess || clusters < 1) {
     cudaGetLastError();
     return;
   }
   h->seq_ok = true;
+  h->seq_form = form;
   h->seq_Q = Q;
   h->seq_Cq = Cq;
-  h->seq_band_max = band_max;
-  h->seq_smem = smem;
+  h->seq_band_max = band[form];
+  h->seq_smem = smem[form];
 }
 
 // Allocate the device block, streams and events; copy idx/perm/boost.
@@ -234,8 +306,8 @@ sp_status init_handle(sp_handle* h, const sp_config* cfg, const uint32_t* idx, c
   h->d_duty = reinterpret_cast<float*>(b + off[9]);
   h->d_err = reinterpret_cast<uint32_t*>(b + off[10]);
   SP_CUDA(cudaMallocHost(&h->h_result, ((size_t)h->C + 1) * 4));
-  SP_CUDA(cudaMallocHost(&h->h_err, 4));
-  *h->h_err = 0u;
+  SP_CUDA(cudaMallocHost(&h->h_err, 8));
+  h->h_err[0] = h->h_err[1] = 0u;
   SP_CUDA(cudaStreamCreateWithFlags(&h->own_stream, cudaStreamNonBlocking));
   h->stream = h->own_stream;
   SP_CUDA(cudaEventCreateWithFlags(&h->ev_switch, cudaEventDisableTiming));
@@ -272,6 +344,10 @@ sp_status wait_handle(sp_handle* h) {
     if (e == cudaSuccess) {
       if (h->dense_used && *h->h_err != 0u)
         return fail(SP_ETIMEOUT, "a tensor-core kernel gave up waiting for its MMAs");
+      if (reinterpret_cast<volatile uint32_t*>(h->h_err)[1] != 0u) {
+        h->h_err[1] = 0u;
+        return fail(SP_ETIMEOUT, "a bounded device wait expired (the sequence stopped early)");
+      }
       return SP_OK;
     }
     if (e != cudaErrorNotReady)
@@ -508,8 +584,6 @@ sp_status run_sequence(sp_handle* h, const uint32_t* x_base, uint32_t n, uint64_
     a.mask_words = h->mask_words;
     a.Cq = h->seq_Cq;
     a.band_max = h->seq_band_max;
-    a.vec16 = (h->n_words % 4u == 0u && stride % 4u == 0u &&
-               reinterpret_cast<uintptr_t>(x_base) % 16u == 0u) ? 1u : 0u;
     a.thr = h->cfg.connect_threshold;
     a.inc = h->cfg.perm_inc;
     a.dec = h->cfg.perm_dec;
@@ -522,7 +596,10 @@ sp_status run_sequence(sp_handle* h, const uint32_t* x_base, uint32_t n, uint64_
     a.unit_boost = h->unit_boost ? 1u : 0u;
     a.duty = h->cfg.duty_period > 0.0f ? h->d_duty : nullptr;
     a.duty_period = h->cfg.duty_period;
-    SP_CUDA(sp::launch_seq(a, h->seq_Q, h->seq_smem, h->stream));
+    a.win_w = h->cfg.input_w;
+    a.wpr = h->cfg.input_w / 32u;
+    a.err = h->h_err + 1;  // pinned host memory, written by the device as it is
+    SP_CUDA(sp::launch_seq(a, h->seq_form, h->seq_Q, h->seq_smem, h->stream));
     h->pending = false;  // learning of every frame is already applied
     h->cur ^= 1;
     h->frames += n;

@@ -26,6 +26,14 @@ __device__ __forceinline__ float boosted(uint32_t raw, uint32_t min_overlap, flo
   return raw < min_overlap ? 0.0f : __fmul_rn(__uint2float_rn(raw), boost);
 }
 
+// Barrier of the NTHREADS threads that run one of the block-wide helpers below
+// (the whole block, or its compute warps where other warps help): its own
+// barrier number, so that other warps may wait at the block's.
+template <int NTHREADS>
+__device__ __forceinline__ void group_sync() {
+  asm volatile("bar.sync 1, %0;\n" ::"n"(NTHREADS) : "memory");
+}
+
 // Exclusive block-wide prefix sums of two per-thread counters, plus totals.
 // Every thread of the block must call it.  sh holds 2 * NW words.
 template <int NW>
@@ -47,7 +55,7 @@ __device__ __forceinline__ void block_scan2(uint32_t va, uint32_t vb, uint32_t& 
     sh[warp] = ia;
     sh[NW + warp] = ib;
   }
-  __syncthreads();
+  group_sync<32 * NW>();
   uint32_t wa = 0, wb = 0, sa = 0, sb = 0;
 #pragma unroll
   for (int w = 0; w < NW; ++w) {
@@ -63,7 +71,7 @@ __device__ __forceinline__ void block_scan2(uint32_t va, uint32_t vb, uint32_t& 
   ex_b = wb + ib - vb;
   tot_a = sa;
   tot_b = sb;
-  __syncthreads();
+  group_sync<32 * NW>();
 }
 
 // hist[bin] += 1 for every lane with `active`, one shared-memory atomic per
@@ -106,7 +114,7 @@ __device__ void select_threshold(const uint32_t* sv, uint32_t C, uint32_t k, uin
     const uint32_t nb = unit_S;  // bins 1..S hold the counts
     if (!ghist) {
       for (uint32_t b = t; b <= nb; b += NTHREADS) shist[b] = 0u;
-      __syncthreads();
+      group_sync<NTHREADS>();
       const uint32_t rounds = (C + NTHREADS - 1) / NTHREADS;
       for (uint32_t r = 0; r < rounds; ++r) {
         const uint32_t i = r * NTHREADS + t;
@@ -114,7 +122,7 @@ __device__ void select_threshold(const uint32_t* sv, uint32_t C, uint32_t k, uin
         // unit boosts: the overlap is an exact small integer
         warp_hist_add(shist, (uint32_t)__uint_as_float(v), v != 0u);
       }
-      __syncthreads();
+      group_sync<NTHREADS>();
     }
     const uint32_t* H = ghist ? ghist : shist;
     // thread t owns bins top = nb - t*pb down to top - cnt + 1 (descending)
@@ -137,10 +145,10 @@ __device__ void select_threshold(const uint32_t* sv, uint32_t C, uint32_t k, uin
         acc += hb;
       }
     }
-    __syncthreads();
+    group_sync<NTHREADS>();
     T = __float_as_uint(__uint2float_rn(s2[0]));
     need = k - s2[1];
-    __syncthreads();
+    group_sync<NTHREADS>();
     return;
   }
   // radix select, most significant byte first
@@ -148,13 +156,13 @@ __device__ void select_threshold(const uint32_t* sv, uint32_t C, uint32_t k, uin
   const uint32_t rounds = (C + NTHREADS - 1) / NTHREADS;
   for (int shift = 24; shift >= 0; shift -= 8) {
     for (uint32_t i = t; i < 256u; i += NTHREADS) shist[i] = 0u;
-    __syncthreads();
+    group_sync<NTHREADS>();
     for (uint32_t r = 0; r < rounds; ++r) {
       const uint32_t i = r * NTHREADS + t;
       const uint32_t v = i < C ? sv[i] : 0u;
       warp_hist_add(shist, (v >> shift) & 255u, v != 0u && (v & pmask) == prefix);
     }
-    __syncthreads();
+    group_sync<NTHREADS>();
     if (t < 32u) {
       // lane L scans digits 255-8L .. 248-8L (descending)
       uint32_t loc[8], sum = 0;
@@ -179,11 +187,11 @@ __device__ void select_threshold(const uint32_t* sv, uint32_t C, uint32_t k, uin
         above += loc[j];
       }
     }
-    __syncthreads();
+    group_sync<NTHREADS>();
     prefix |= s2[0] << shift;
     pmask |= 0xffu << shift;
     kk -= s2[1];
-    __syncthreads();
+    group_sync<NTHREADS>();
   }
   T = prefix;  // the k-th largest overlap (bit pattern)
   need = kk;   // how many columns equal to T still win
@@ -201,13 +209,13 @@ __device__ uint32_t kth_largest(const uint32_t* sv, uint32_t C, uint32_t k, uint
   const uint32_t rounds = (C + NTHREADS - 1) / NTHREADS;
   for (int shift = 24; shift >= 0; shift -= 8) {
     for (uint32_t i = t; i < 256u; i += NTHREADS) shist[i] = 0u;
-    __syncthreads();
+    group_sync<NTHREADS>();
     for (uint32_t r = 0; r < rounds; ++r) {
       const uint32_t i = r * NTHREADS + t;
       const uint32_t v = i < C ? sv[i] : 0u;
       warp_hist_add(shist, (v >> shift) & 255u, i < C && (v & pmask) == prefix);
     }
-    __syncthreads();
+    group_sync<NTHREADS>();
     if (t < 32u) {
       uint32_t loc[8], sum = 0;
 #pragma unroll
@@ -231,11 +239,11 @@ __device__ uint32_t kth_largest(const uint32_t* sv, uint32_t C, uint32_t k, uint
         above += loc[j];
       }
     }
-    __syncthreads();
+    group_sync<NTHREADS>();
     prefix |= s2[0] << shift;
     pmask |= 0xffu << shift;
     kk -= s2[1];
-    __syncthreads();
+    group_sync<NTHREADS>();
   }
   return prefix;
 }

@@ -85,7 +85,9 @@ constexpr uint32_t kChunkFrames = 32;  // frames per staged chunk in sp_compute_
 constexpr int kSlots = 2;
 constexpr uint32_t kGraphMinFrames = 4;  // shorter sequences are launched directly
 constexpr uint32_t kSeqMinFrames = 8;    // shorter sequences use the per-frame kernel
-constexpr size_t kSeqSmemLimit = 226u * 1024u;  // 227 KiB per CTA, less static shared memory
+constexpr uint64_t kSeqOneCtaSynapses = 16384;  // sequences of at most these run in one CTA
+constexpr uint32_t kSeqWindowSynapses = 96;  // pools of at least these count faster as bitmaps
+constexpr size_t kSeqSmemLimit = 231168u;  // 227 KiB per CTA, less 1.25 KiB of static shared memory
 
 inline bool seq_enabled() {
   const char* s = std::getenv("SP_DISABLE_CLUSTER");
@@ -166,7 +168,7 @@ struct sp_handle {
   uint32_t* d_hist = nullptr;  // [S + 1], used when every boost is 1
   float* d_duty = nullptr;     // [C] active-duty cycles (tracked when duty_period > 0)
   uint32_t* d_err = nullptr;   // set by a kernel whose bounded wait expired
-  uint32_t* h_err = nullptr;   // pinned copy of d_err
+  uint32_t* h_err = nullptr;   // pinned: [0] copy of d_err, [1] written by the sequence kernel
   // dense pools (every column sees the whole input): inference runs of frames
   // go through the tensor cores
   bool dense = false;
@@ -216,6 +218,6 @@ struct sp_handle {
   sp_batch* batch = nullptr;  // set while the handle is a member of a batch
   // persistent cluster path for frame sequences (state in shared memory)
   bool seq_ok = false;
-  uint32_t seq_Q = 0, seq_Cq = 0, seq_band_max = 0;
+  uint32_t seq_form = 0, seq_Q = 0, seq_Cq = 0, seq_band_max = 0;
   size_t seq_smem = 0;
 };

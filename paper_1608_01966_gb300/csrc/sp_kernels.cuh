@@ -208,8 +208,12 @@ struct LearnArgs {
 
 // A whole frame sequence of one SP in one persistent cluster launch
 // (sp_seq_cluster.cu): the state stays in the cluster's shared memory.
-constexpr int kSeqThreads = 512;
+constexpr int kSeqThreads = 512;  // compute threads of a CTA (helper warps come on top)
 constexpr uint32_t kSeqMaxCluster = 16;
+// Form of the state in shared memory: pools and permanences; connected
+// bitmaps, positions and permanences; connected bitmaps alone (pools and
+// permanences stay in global memory).
+enum : uint32_t { kSeqPools = 0u, kSeqWindow = 1u, kSeqWindowL2 = 2u };
 
 struct SeqArgs {
   const uint32_t* idx;        // [C][S]
@@ -229,18 +233,21 @@ struct SeqArgs {
   uint32_t C, S, n_words, mask_words;
   uint32_t Cq;                // columns per CTA (multiple of 32)
   uint32_t band_max;          // words of the largest per-CTA input band (multiple of 4)
-  uint32_t vec16;             // frames 16-byte aligned with stride, n_words % 4 == 0
   float thr, inc, dec;
   uint32_t min_overlap, k, inhibition, gw, gh, radius;
   uint32_t unit_boost;
   float* duty;                // [C] active-duty cycles, or nullptr
   float duty_period;
+  uint32_t win_w, wpr;        // window forms: input_w and its words per row
+  uint32_t* err;              // mapped host word, set to 1 if a bounded wait expired
 };
 
-size_t seq_smem_bytes(uint32_t C, uint32_t S, uint32_t Cq, uint32_t band_max);
-cudaError_t seq_kernel_init(size_t smem_bytes);
-cudaError_t seq_max_active_clusters(uint32_t Q, size_t smem_bytes, int* out);
-cudaError_t launch_seq(const SeqArgs& a, uint32_t Q, size_t smem_bytes, cudaStream_t stream);
+size_t seq_smem_bytes(uint32_t form, uint32_t Q, uint32_t C, uint32_t S, uint32_t Cq,
+                      uint32_t band_max);
+cudaError_t seq_kernel_init(uint32_t form, size_t smem_bytes);
+cudaError_t seq_max_active_clusters(uint32_t form, uint32_t Q, size_t smem_bytes, int* out);
+cudaError_t launch_seq(const SeqArgs& a, uint32_t form, uint32_t Q, size_t smem_bytes,
+                       cudaStream_t stream);
 
 // Dense pools on the tensor cores (sp_dense_tc.cu): the raw overlaps of a run
 // of frames without learning as one {0,1} matrix product.  Both operands are

@@ -1,42 +1,63 @@
 // Frame sequences of one Spatial Pooler in a single persistent launch: the
-// SP state lives in the distributed shared memory of one thread-block
-// cluster for the whole sequence.
+// SP state lives in the shared memory of one thread-block cluster for the
+// whole sequence.
 //
 // A sequence with learning is inherently serial (frame t+1 reads the
-// permanences frame t wrote), so one SP is latency-bound, not bandwidth-bound.
-// Instead of one kernel per frame reading the state from L2 each time, a
-// cluster of Q CTAs (Q = 16 for 1024 columns x 256 synapses) loads the state
-// once into shared memory -- CTA q owns columns [q*Cq, (q+1)*Cq) with their
-// pools, permanences and boosts -- and loops over the frames:
+// permanences frame t wrote), so one SP is bound by the latency of a frame's
+// chain, not by bandwidth.  A cluster of Q CTAs loads the state once -- CTA q
+// owns columns [q*Cq, (q+1)*Cq) -- and loops over the frames.  16 compute
+// warps walk the chain; four helper warps keep everything else off it (the
+// next frame's input band by cp.async into the other of two buffers, the
+// masks and overlap records, clearing what later frames count into).  A frame:
 //
-//   1. the input band its columns' pools cover (a contiguous word range of
-//      the packed frame) arrives in shared memory by cp.async, issued during
-//      the previous frame (double-buffered);
-//   2. Alg. 1 for its columns from shared memory, each warp counting four
-//      columns side by side; the boosted overlaps are published in shared
-//      memory;
-//   3. one cluster barrier (barrier.cluster arrive.release / wait.acquire);
-//   4. with global inhibition and unit boosts (counts are the overlaps),
-//      each CTA has published a count histogram of its columns in step 2;
-//      warp 0 of every CTA reads the cluster's histograms from the top, 32
-//      bins a round, until it reaches the k-th largest count, and decides its
-//      own columns; otherwise every CTA gathers all C overlaps through DSMEM
-//      and runs Alg. 2 on them (the same deterministic answer in every CTA),
-//      keeping the decisions for its own columns;
-//   5. learning (Section 1.1) of its winning columns in shared memory, with
-//      the frame band still resident.
+//   1. the band of input words the CTA's pools cover is waited for;
+//   2. Alg. 1, each warp its own columns; counts of at least min_overlap go to
+//      shared memory as 16-bit values; CTA barrier;
+//   3. the CTA pushes its counts to every other CTA of the cluster (st.async,
+//      completing on the receiver's mbarrier) and waits for theirs: one
+//      one-way trip, where a cluster barrier followed by reads of remote
+//      memory costs a barrier and a round trip;
+//   4. global inhibition: a histogram of all counts in shared memory, barrier,
+//      then every warp finds the k-th largest count (32 bins a step from the
+//      largest count down) and all winners of its CTA by itself; local
+//      inhibition: every column is ranked against its neighbours' counts by a
+//      few lanes of the warp that owns it, barrier;
+//   5. Section 1.1: the CTA's i-th winner is learnt by warp i % 16 (winners
+//      are neighbours, so dealing them out is what keeps one warp from doing
+//      them all), the frame's band still in place; barrier.
 //
-// Outputs per frame: this CTA's words of the active mask and, when asked
-// for, its columns' boosted overlaps; the last frame's list and overlaps.
+// A cluster of one CTA (small SPs) has no step 3: its warps add their counts
+// to the histogram as they publish them.
 //
-// The published overlaps are double-buffered by frame parity, so one
-// barrier per frame orders both the gather of frame t and the overwrite at
-// frame t+2.  Permanence rows that changed are written back at the end.
-// There is no software spin-wait anywhere: the cluster barrier and
-// cp.async.wait_all are hardware waits, and every CTA runs the same frame
-// loop, so every barrier is reached by all CTAs.
+// Three forms of the state:
+//   pools     input indices and fp32 permanences in shared memory; a column's
+//             pool is read four synapses per lane (S % 4 == 0), several
+//             columns side by side in a warp when pools are small;
+//   window    (frames a multiple of 32 pixels wide whose ascending pools fit
+//             64 x 64 boxes) a 64 x 64 bitmap of each column's connected
+//             synapses: a column is 64 row segments of funnel shift, AND and
+//             population count, whatever its pool's size.  Band rows are
+//             padded to an odd number of words, so that the 32 rows a warp
+//             reads lie in 32 banks.  Permanences and 16-bit positions of the
+//             synapses in their boxes are kept beside it in shared memory;
+//   windowL2  the same without them: learning reads the pools and permanences
+//             of the frame's winners from global memory (L2).
+//
+// Non-unit boosts make the overlaps fp32 values: then every CTA publishes its
+// boosted overlaps, a cluster barrier orders them, and every CTA gathers all
+// of them and runs Alg. 2 on its own.
+//
+// Counts are double-buffered by frame parity: a CTA sends frame t+2's counts
+// only after it has received frame t+1's from everyone, and those are sent
+// after the sender is done with frame t's.
+//
+// Waits are bounded (1 s of %globaltimer): when one expires, the CTA records
+// it, the loop ends at the next CTA barrier, and every CTA reaches the cluster
+// barrier at the end (the others after their own limit), so no CTA leaves
+// while another may still write to its shared memory.
 #include <cooperative_groups.h>
 
+#include <algorithm>
 #include <atomic>
 
 #include "../../include/sp.h"
@@ -54,392 +75,881 @@ namespace {
 using dev::kFull;
 using dev::learn_one;
 
-constexpr int kSeqWarps = kSeqThreads / 32;
-constexpr int kSeqCols = 4;  // columns a warp counts side by side
+constexpr uint32_t kSeqWarps = kSeqThreads / 32;   // compute warps
+constexpr uint32_t kSeqHelpers = 128;              // threads of the helper warps
+constexpr int kSeqCols = 4;   // window forms: columns a warp counts side by side
+constexpr unsigned long long kSeqWaitNs = 1000000000ull;
+constexpr uint32_t kBoxWords = 128;  // bitmap words of a 64 x 64 box
 
-__device__ __forceinline__ void cp_async4(uint32_t* smem_dst, const uint32_t* gmem_src) {
-  const uint32_t d = static_cast<uint32_t>(__cvta_generic_to_shared(smem_dst));
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(d), "l"(gmem_src) : "memory");
+__device__ __forceinline__ uint32_t smem_u32(const void* p) {
+  return static_cast<uint32_t>(__cvta_generic_to_shared(p));
 }
 
-__device__ __forceinline__ void cp_async16(uint32_t* smem_dst, const uint32_t* gmem_src) {
-  const uint32_t d = static_cast<uint32_t>(__cvta_generic_to_shared(smem_dst));
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(d), "l"(gmem_src) : "memory");
+__device__ __forceinline__ unsigned long long now_ns() {
+  unsigned long long t;
+  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+  return t;
 }
 
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
-__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }
+__device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count) {
+  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(smem_u32(bar)), "r"(count)
+               : "memory");
+}
 
-// Start copying words [w_lo, w_lo + nw) of one frame into a band buffer.
-__device__ __forceinline__ void issue_band(uint32_t* dst, const uint32_t* frame, uint32_t w_lo,
-                                           uint32_t nw, bool vec16) {
-  if (vec16) {
-    for (uint32_t i = threadIdx.x * 4u; i < nw; i += kSeqThreads * 4u)
-      cp_async16(dst + i, frame + w_lo + i);
-  } else {
-    for (uint32_t i = threadIdx.x; i < nw; i += kSeqThreads) cp_async4(dst + i, frame + w_lo + i);
+__device__ __forceinline__ void mbar_expect(uint64_t* bar, uint32_t bytes) {
+  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(smem_u32(bar)),
+               "r"(bytes)
+               : "memory");
+}
+
+// Wait (bounded) for the phase with this parity; with CLUSTER, what other CTAs
+// of the cluster sent with it is visible after.
+template <bool CLUSTER>
+__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity) {
+  unsigned long long t0 = 0;
+  for (uint32_t i = 0;; ++i) {
+    uint32_t ok;
+    if (CLUSTER)
+      asm volatile(
+          "{\n.reg .pred p;\n"
+          "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n"
+          "selp.b32 %0, 1, 0, p;\n}\n"
+          : "=r"(ok)
+          : "r"(smem_u32(bar)), "r"(parity)
+          : "memory");
+    else
+      asm volatile(
+          "{\n.reg .pred p;\n"
+          "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
+          "selp.b32 %0, 1, 0, p;\n}\n"
+          : "=r"(ok)
+          : "r"(smem_u32(bar)), "r"(parity)
+          : "memory");
+    if (ok) return true;
+    if ((i & 63u) == 0u) {
+      const unsigned long long t = now_ns();
+      if (i == 0u)
+        t0 = t;
+      else if (t - t0 > kSeqWaitNs)
+        return false;
+    }
   }
-  cp_async_commit();
 }
+
+// The shared::cluster address of `saddr` (this CTA's shared memory) in CTA `rank`.
+__device__ __forceinline__ uint32_t peer_addr(uint32_t saddr, uint32_t rank) {
+  uint32_t r;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;\n" : "=r"(r) : "r"(saddr), "r"(rank));
+  return r;
+}
+
+__device__ __forceinline__ void send16(uint32_t dst, const uint4& v, uint32_t bar) {
+  asm volatile(
+      "st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v4.b32 [%0], {%1, %2, %3, %4}, "
+      "[%5];\n" ::"r"(dst),
+      "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w), "r"(bar)
+      : "memory");
+}
+
+// This helper thread's share of copying `rows` rows of `len` consecutive words
+// from src to a band whose rows are `pitch` words apart; its arrival on bar
+// follows its copies.
+__device__ __forceinline__ void copy_band(uint32_t* dst, const uint32_t* src, uint32_t rows,
+                                          uint32_t len, uint32_t pitch, uint64_t* bar) {
+  const uint32_t h = threadIdx.x - kSeqThreads;
+  const uint32_t dr = kSeqHelpers / len, dx = kSeqHelpers - dr * len;
+  uint32_t r = h / len, x = h - r * len;
+  const uint32_t n = rows * len;
+  for (uint32_t i = h; i < n; i += kSeqHelpers) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(smem_u32(dst + r * pitch + x)),
+                 "l"(src + i)
+                 : "memory");
+    r += dr;
+    x += dx;
+    if (x >= len) {
+      x -= len;
+      ++r;
+    }
+  }
+  asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];\n" ::"r"(smem_u32(bar))
+               : "memory");
+}
+
+__device__ __forceinline__ void compute_sync() {
+  asm volatile("bar.sync 2, %0;\n" ::"n"(kSeqThreads) : "memory");
+}
+
+// Words of one frame's histogram: bins 0..S, bin 0 the largest count.
+__host__ __device__ __forceinline__ uint32_t hist_words(uint32_t S) { return (S + 4u) & ~3u; }
 
 // Shared-memory layout of one CTA (all offsets in 4-byte words).
 struct SeqLayout {
-  uint32_t idx, perm, boost, band, ov, raw, hstride, hpub, all, hist, mask, dirty, total;
-  __host__ __device__ SeqLayout(uint32_t Cq, uint32_t S, uint32_t band_max, uint32_t C) {
+  uint32_t bits, at, org, idx, perm, boost, band, cnt, hist, mask, dirty, ov, all, shist, smask, total;
+  __host__ __device__ SeqLayout(uint32_t form, uint32_t Q, uint32_t Cq, uint32_t S,
+                                uint32_t band_max, uint32_t C) {
     const uint32_t CqS = Cq * S;
-    idx = 0;
-    perm = idx + CqS;
-    boost = perm + CqS;
-    band = (boost + Cq + 3u) & ~3u;  // 16-byte aligned
-    ov = band + 2u * band_max;
-    raw = ov + 2u * Cq;
-    hstride = (S + 4u) & ~3u;         // bins 0..S, rounded up to whole 16-byte words
-    hpub = (raw + Cq + 3u) & ~3u;     // [2][hstride] published count histograms, bin 0 the max
-    all = hpub + 2u * hstride;
-    hist = all + C;
-    const uint32_t hw = (S + 1u) > 256u ? (S + 1u) : 256u;
-    mask = hist + hw;
-    dirty = mask + (C + 31u) / 32u;
-    total = dirty + Cq / 32u;
+    uint32_t o = 0;
+    auto part = [&](uint32_t words) {
+      const uint32_t at0 = o;
+      o += (words + 3u) & ~3u;  // 16-byte aligned parts
+      return at0;
+    };
+    const bool window = form != kSeqPools;
+    bits = part(window ? Cq * kBoxWords : 0u);
+    at = part(window ? Cq : 0u);
+    org = part(window ? Cq : 0u);
+    // pools: 32-bit indices; window: 16-bit positions in the box
+    idx = part(form == kSeqPools ? CqS : (form == kSeqWindow ? (CqS + 1u) / 2u : 0u));
+    perm = part(form != kSeqWindowL2 ? CqS : 0u);
+    boost = part(Cq);
+    band = part(2u * band_max);
+    mask = part(3u * (Cq / 32u));            // three frames' winner masks in turn
+    dirty = part(Cq / 32u);
+    const uint32_t rest = o;
+    cnt = part(2u * (Q * Cq / 2u));          // [2][Q * Cq] 16-bit counts
+    hist = part(3u * hist_words(S));         // three frames' histograms in turn
+    const uint32_t unit_end = o;
+    o = rest;  // non-unit boosts use the same memory for fp32 overlaps
+    ov = part(2u * Cq);
+    all = part(C);
+    shist = part((S + 1u) > 256u ? (S + 1u) : 256u);
+    smask = part((C + 31u) / 32u);
+    o = o > unit_end ? o : unit_end;
+    total = o;
   }
 };
 
-// Global inhibition with unit boosts, decided by warp 0 of each CTA for the
-// CTA's own columns from the count histograms the CTAs publish in shared
-// memory (hpub: bin b holds how many of the publishing CTA's columns count b;
-// bin 0 holds its largest count).  The warp reads the Q largest counts, then
-// gathers 32 bins at a time from the top (lane l: bin top - l, from every
-// CTA; usually one or two rounds reach the k-th largest count T), with one
-// warp scan per round for the columns above each bin, in the whole cluster
-// and in the lower-ranked CTAs.  That gives T, the ties at T that still win
-// (`need`) and the winners and ties of the lower-ranked CTAs.  The CTA's
-// columns (count in s_raw, 0 below min_overlap) are then decided 32 at a
-// time: a ballot ranks the ties in column order, another gives the mask
-// word.  When list != nullptr the winners' slots of the ascending list are
-// written.  Returns the cluster-wide number of winners (every lane gets it).
-template <typename Cluster>
-__device__ uint32_t decide_unit_global(const Cluster& cluster, const uint32_t* hpub,
-                                       const uint32_t* s_raw, uint32_t k, uint32_t q,
-                                       uint32_t c0, uint32_t nc, uint32_t* s_mask,
-                                       uint32_t* list) {
-  const uint32_t lane = threadIdx.x & 31u;
-  const uint32_t Q = cluster.num_blocks();
-  const uint32_t top0 = __reduce_max_sync(kFull, lane < Q ? cluster.map_shared_rank(hpub, lane)[0] : 0u);
-  // T: 0xffffffff nobody wins; 0 every counted column wins (at most k)
-  uint32_t T = 0xffffffffu, need = 0u, above_lower = 0u, ties_lower = 0u;
-  uint32_t acc_g = 0u, acc_p = 0u;  // columns above the current round's bins
-  if (k != 0u) {
-    T = 0u;                           // reaching bin 0: at most k counted columns
-    for (uint32_t top = top0; top >= 1u; top = top > 32u ? top - 32u : 0u) {
-      const uint32_t bin = top >= lane + 1u ? top - lane : 0u;  // 0: past the last bin
-      uint32_t v[kSeqMaxCluster];
-#pragma unroll
-      for (uint32_t r = 0; r < kSeqMaxCluster; ++r)
-        v[r] = (r < Q && bin != 0u) ? cluster.map_shared_rank(hpub, r)[bin] : 0u;
-      uint32_t g = 0u, p = 0u;
-#pragma unroll
-      for (uint32_t r = 0; r < kSeqMaxCluster; ++r) {
-        g += v[r];
-        p += r < q ? v[r] : 0u;
-      }
-      uint32_t ig = g, ip = p;  // inclusive sums from the top
-#pragma unroll
-      for (uint32_t o = 1; o < 32u; o <<= 1) {
-        const uint32_t yg = __shfl_up_sync(kFull, ig, o), yp = __shfl_up_sync(kFull, ip, o);
-        if (lane >= o) {
-          ig += yg;
-          ip += yp;
-        }
-      }
-      const uint32_t hit = __ballot_sync(kFull, acc_g + ig - g < k && acc_g + ig >= k);
-      if (hit) {
-        const int src = __ffs(hit) - 1;
-        T = __shfl_sync(kFull, bin, src);
-        need = k - (acc_g + __shfl_sync(kFull, ig - g, src));
-        above_lower = acc_p + __shfl_sync(kFull, ip - p, src);
-        ties_lower = __shfl_sync(kFull, p, src);
-        break;
-      }
-      acc_g += __shfl_sync(kFull, ig, 31);
-      acc_p += __shfl_sync(kFull, ip, 31);
-    }
-    if (T == 0u) above_lower = acc_p;  // every counted column of the lower CTAs wins
-  }
-  const bool real_T = T != 0u && T != 0xffffffffu;
-  const uint32_t base = above_lower + min(ties_lower, need);  // this CTA's first list slot
-  uint32_t ties_before = 0u, wins_before = 0u;
-  const uint32_t lt = (1u << lane) - 1u;
-  for (uint32_t j = 0; j < nc; j += 32u) {
-    const uint32_t r = j + lane < nc ? s_raw[j + lane] : 0u;
-    const bool tie = real_T && r == T;
-    const uint32_t tm = __ballot_sync(kFull, tie);
-    const bool win = r != 0u && T != 0xffffffffu &&
-                     (T == 0u || r > T ||
-                      (tie && ties_lower + ties_before + (uint32_t)__popc(tm & lt) < need));
-    const uint32_t wm = __ballot_sync(kFull, win);
-    if (lane == 0u) s_mask[(c0 >> 5) + (j >> 5)] = wm;
-    if (list && win) list[base + wins_before + (uint32_t)__popc(wm & lt)] = c0 + j + lane;
-    ties_before += (uint32_t)__popc(tm);
-    wins_before += (uint32_t)__popc(wm);
-  }
-  // T = 0: every counted column wins, acc_g of them (every bin was summed)
-  return T == 0xffffffffu ? 0u : (T == 0u ? acc_g : k);
-}
+template <int N>
+struct IntC {
+  static constexpr int value = N;
+};
 
-__global__ void __launch_bounds__(kSeqThreads, 1) sp_seq_cluster_kernel(const SeqArgs a) {
+template <uint32_t FORM>
+__global__ void __launch_bounds__(kSeqThreads + kSeqHelpers, 1) sp_seq_cluster_kernel(const SeqArgs a) {
+  constexpr bool kWindow = FORM != kSeqPools;
+  constexpr bool kPermSmem = FORM != kSeqWindowL2;
+  constexpr uint32_t kAll = kSeqThreads + kSeqHelpers;
   cg::cluster_group cluster = cg::this_cluster();
   extern __shared__ __align__(16) uint32_t sm[];
   __shared__ uint32_t sh[2 * kSeqWarps];
-  __shared__ uint32_t s2[8];
+  __shared__ uint32_t s2[2];
+  __shared__ uint32_t s_n;                 // winners listed in this frame
+  __shared__ uint16_t s_list[kSeqThreads];  // their columns in this CTA
+  __shared__ __align__(8) uint64_t s_band_bar[2], s_cnt_bar[2];
 
-  const uint32_t q = cluster.block_rank();
+  const uint32_t q = cluster.block_rank(), Q = cluster.num_blocks();
   const uint32_t t = threadIdx.x;
-  const int warp = t >> 5, lane = t & 31;
+  const uint32_t warp = t >> 5, lane = t & 31u;
+  const bool helper = t >= kSeqThreads;
   const uint32_t C = a.C, S = a.S, Cq = a.Cq;
   const uint32_t c0 = q * Cq;
   const uint32_t nc = C > c0 ? min(Cq, C - c0) : 0u;
-  const SeqLayout L(Cq, S, a.band_max, C);
+  const uint32_t mw = Cq / 32u;  // mask words of this CTA
+  const SeqLayout L(FORM, Q, Cq, S, a.band_max, C);
+  uint32_t* s_bits = sm + L.bits;
+  uint32_t* s_at = sm + L.at;
+  uint32_t* s_org = sm + L.org;
   uint32_t* s_idx = sm + L.idx;
+  uint16_t* s_pos = reinterpret_cast<uint16_t*>(sm + L.idx);
   float* s_perm = reinterpret_cast<float*>(sm + L.perm);
   float* s_boost = reinterpret_cast<float*>(sm + L.boost);
   uint32_t* s_band = sm + L.band;
-  float* s_ov = reinterpret_cast<float*>(sm + L.ov);
-  uint32_t* s_raw = sm + L.raw;
-  uint32_t* s_hpub = sm + L.hpub;
-  uint32_t* s_all = sm + L.all;
-  uint32_t* s_hist = sm + L.hist;
-  uint32_t* s_mask = sm + L.mask;
   uint32_t* s_dirty = sm + L.dirty;
-
-  // ---- load this CTA's state: pools, permanences, boosts -----------------
+  const uint32_t hw = hist_words(S);
+  const uint32_t cnt_words = Q * Cq / 2u;  // 32-bit words of one frame's counts
   const uint64_t g0 = (uint64_t)c0 * S;
-  const uint32_t nCS = nc * S;
-  if ((S & 3u) == 0u) {
-    const uint4* gi = reinterpret_cast<const uint4*>(a.idx + g0);
-    const uint4* gp = reinterpret_cast<const uint4*>(a.perm + g0);
-    for (uint32_t i = t; i < nCS / 4u; i += kSeqThreads) {
-      reinterpret_cast<uint4*>(s_idx)[i] = __ldg(gi + i);
-      reinterpret_cast<uint4*>(s_perm)[i] = gp[i];
-    }
-  } else {
-    for (uint32_t i = t; i < nCS; i += kSeqThreads) {
-      s_idx[i] = __ldg(a.idx + g0 + i);
-      s_perm[i] = a.perm[g0 + i];
-    }
+  const bool fast = a.unit_boost != 0u;  // counts are the overlaps
+  const bool global = a.inhibition == 0u;
+
+  // Column ownership of the count.  A warp counts P columns side by side,
+  // L32 = 32 / P lanes each (pools of a few synapses); its i-th own column is
+  //   lc = ((i / P) * kSeqWarps + warp) * P + i % P,   i < own.
+  uint32_t P = 1u;
+  if (!kWindow) {
+    const uint32_t units = (S & 3u) == 0u ? S >> 2 : S;  // lane loads of one pool
+    while (P < 8u && units * P * 2u <= 32u && kSeqWarps * P * 2u <= Cq) P <<= 1;
   }
-  for (uint32_t i = t; i < nc; i += kSeqThreads) s_boost[i] = __ldg(a.boost + c0 + i);
-  for (uint32_t i = t; i < Cq / 32u; i += kSeqThreads) s_dirty[i] = 0u;
-  for (uint32_t i = t; i < 2u * L.hstride; i += kSeqThreads) s_hpub[i] = 0u;
-  const bool fast = a.inhibition == 0u && a.unit_boost != 0u;
-  // input band of this CTA: the 16-byte aligned word range covering its pools
-  uint32_t mn = 0xffffffffu, mx = 0u;
-  for (uint32_t i = t; i < nCS; i += kSeqThreads) {
-    const uint32_t id = __ldg(a.idx + g0 + i);
-    mn = min(mn, id);
-    mx = max(mx, id);
+  const uint32_t L32 = 32u / P;
+  const uint32_t passes = (Cq + kSeqWarps * P - 1u) / (kSeqWarps * P);
+  const uint32_t own = passes * P;  // at most 32 (Cq <= kSeqThreads)
+  auto own_col = [&](uint32_t i) { return ((i / P) * kSeqWarps + warp) * P + i % P; };
+
+  // ---- prologue: barriers, this CTA's state and input band -------------------
+  if (t == 0) {
+    s_n = 0u;
+    mbar_init(&s_band_bar[0], kSeqHelpers);
+    mbar_init(&s_band_bar[1], kSeqHelpers);
+    mbar_init(&s_cnt_bar[0], 1);
+    mbar_init(&s_cnt_bar[1], 1);
+    asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
   }
-  mn = __reduce_min_sync(kFull, mn);
-  mx = __reduce_max_sync(kFull, mx);
-  if (lane == 0) {
-    sh[warp] = mn;
-    sh[kSeqWarps + warp] = mx;
+  for (uint32_t i = t; i < nc; i += kAll) s_boost[i] = __ldg(a.boost + c0 + i);
+  for (uint32_t i = t; i < mw; i += kAll) s_dirty[i] = 0u;
+  for (uint32_t i = t; i < 3u * hw; i += kAll) sm[L.hist + i] = 0u;
+  for (uint32_t i = t; i < 3u * mw; i += kAll) sm[L.mask + i] = 0u;
+  for (uint32_t i = t; i < 2u * cnt_words; i += kAll) sm[L.cnt + i] = 0u;
+  // band words no copy writes (rows past the frame, row padding) are read
+  // under empty bitmap bits only; they are set once all the same
+  for (uint32_t i = t; i < 2u * a.band_max; i += kAll) s_band[i] = 0u;
+  if (FORM == kSeqPools) {
+    const uint32_t nCS = nc * S;
+    if ((S & 3u) == 0u) {
+      const uint4* gi = reinterpret_cast<const uint4*>(a.idx + g0);
+      const uint4* gp = reinterpret_cast<const uint4*>(a.perm + g0);
+      for (uint32_t i = t; i < nCS / 4u; i += kAll) {
+        reinterpret_cast<uint4*>(s_idx)[i] = __ldg(gi + i);
+        reinterpret_cast<uint4*>(s_perm)[i] = gp[i];
+      }
+    } else {
+      for (uint32_t i = t; i < nCS; i += kAll) {
+        s_idx[i] = __ldg(a.idx + g0 + i);
+        s_perm[i] = a.perm[g0 + i];
+      }
+    }
   }
   __syncthreads();
-  if (t == 0) {
+  // exact quotient by the frame width from a float estimate
+  const float inv_w = kWindow ? 1.0f / (float)a.win_w : 0.0f;
+  auto row_of = [&](uint32_t id) {
+    uint32_t r = __float2uint_rz(__uint2float_rz(id) * inv_w);
+    while (r * a.win_w > id) --r;
+    while ((r + 1u) * a.win_w <= id) ++r;
+    return r;
+  };
+  // boxes of the columns, and the smallest and largest value that the CTA's
+  // band must cover (input indices; window forms: box rows)
+  if (!helper) {
+    uint32_t mn = 0xffffffffu, mx = 0u;
+    for (uint32_t i = 0; i < own; ++i) {
+      const uint32_t lc = own_col(i);
+      if (lc >= nc) continue;
+      const uint32_t* row = kWindow ? a.idx + g0 + (uint64_t)lc * S : s_idx + lc * S;
+      if (kWindow) {
+        uint32_t x0 = 0xffffffffu, y0 = 0xffffffffu;
+        for (uint32_t s = lane; s < S; s += 32u) {
+          const uint32_t id = __ldg(row + s), y = row_of(id);
+          x0 = min(x0, id - y * a.win_w);
+          y0 = min(y0, y);
+        }
+        x0 = __reduce_min_sync(kFull, x0);
+        y0 = __reduce_min_sync(kFull, y0);
+        if (lane == 0u) s_org[lc] = (y0 << 16) | x0;
+        mn = min(mn, y0);
+        mx = max(mx, y0 + 63u);
+      } else {
+        for (uint32_t s = lane; s < S; s += 32u) {
+          mn = min(mn, row[s]);
+          mx = max(mx, row[s]);
+        }
+      }
+    }
+    mn = __reduce_min_sync(kFull, mn);
+    mx = __reduce_max_sync(kFull, mx);
+    if (lane == 0u) {
+      sh[warp] = mn;
+      sh[kSeqWarps + warp] = mx;
+    }
+  }
+  __syncthreads();
+  // the band: brows rows of blen words from word w_lo of the frame, `pitch` apart
+  uint32_t w_lo = 0u, brows = 0u, blen = 1u, pitch = 1u, y_lo = 0u;
+  {
     uint32_t m0 = 0xffffffffu, m1 = 0u;
-    for (int w = 0; w < kSeqWarps; ++w) {
+    for (uint32_t w = 0; w < kSeqWarps; ++w) {
       m0 = min(m0, sh[w]);
       m1 = max(m1, sh[kSeqWarps + w]);
     }
-    if (m0 > m1) m0 = m1 = 0u;  // a CTA without columns
-    const uint32_t w_lo = (m0 >> 5) & ~3u;
-    uint32_t w_hi = ((m1 >> 5) + 4u) & ~3u;  // exclusive, multiple of 4
-    if (!a.vec16 && w_hi > a.n_words) w_hi = a.n_words;
-    s2[0] = w_lo;
-    s2[1] = min(w_hi - w_lo, a.band_max);
-  }
-  __syncthreads();
-  const uint32_t w_lo = s2[0], nbw = s2[1];
-  __syncthreads();
-
-  // ---- learning left pending by the previous call ------------------------
-  if (a.pend_mask) {
-    for (uint32_t lc = warp; lc < nc; lc += kSeqWarps) {
-      const uint32_t c = c0 + lc;
-      if (!((__ldg(a.pend_mask + (c >> 5)) >> (c & 31u)) & 1u)) continue;
-      for (uint32_t s = lane; s < S; s += 32) {
-        const uint32_t e = lc * S + s;
-        s_perm[e] = learn_one(s_perm[e], dev::input_bit(a.pend_x, s_idx[e]), a.inc, a.dec);
-      }
-      if (lane == 0) atomicOr(s_dirty + (lc >> 5), 1u << (lc & 31u));
+    if (m0 <= m1 && kWindow) {  // else a CTA without columns
+      y_lo = m0;
+      w_lo = m0 * a.wpr;
+      brows = min(m1 + 1u, a.n_words / a.wpr) - m0;
+      blen = a.wpr;
+      pitch = a.wpr | 1u;
+    } else if (m0 <= m1) {
+      w_lo = m0 >> 5;
+      brows = 1u;
+      blen = (m1 >> 5) + 1u - w_lo;
     }
   }
-  issue_band(s_band, a.frames, w_lo, nbw, a.vec16);
-
-  for (uint32_t f = 0; f < a.n_frames; ++f) {
-    const uint32_t par = f & 1u;
-    uint32_t* band = s_band + par * a.band_max;
-    float* ov_pub = s_ov + par * Cq;
-    cp_async_wait_all();
-    __syncthreads();  // band f visible; frame f-1 finished in this CTA
-    if (f + 1u < a.n_frames)
-      issue_band(s_band + (par ^ 1u) * a.band_max, a.frames + (uint64_t)(f + 1u) * a.stride,
-                 w_lo, nbw, a.vec16);
-
-    // ---- Alg. 1 for this CTA's columns --------------------------------------
-    // warp w counts columns w, w + 16, w + 32, w + 48 (kSeqCols of them) side
-    // by side, so the loads of all four are in flight together; lane j then
-    // publishes column j's count
-    uint32_t* hpub = s_hpub + par * L.hstride;
-    for (uint32_t lc0 = warp; lc0 < nc; lc0 += kSeqWarps * kSeqCols) {
-      uint32_t cnt[kSeqCols];
-#pragma unroll
-      for (int j = 0; j < kSeqCols; ++j) {
-        const uint32_t lc = lc0 + (uint32_t)j * kSeqWarps;
-        cnt[j] = 0u;
-        if (lc < nc) {
-          const uint32_t* ri = s_idx + lc * S;
-          const float* rp = s_perm + lc * S;
-#pragma unroll 8
-          for (uint32_t s = lane; s < S; s += 32) {
-            const uint32_t id = ri[s];
-            const uint32_t w = (id >> 5) - w_lo;
-            cnt[j] += (rp[s] >= a.thr) ? ((band[w] >> (id & 31u)) & 1u) : 0u;
+  // position of synapse id in its column's box: (bitmap word << 5) | bit
+  auto box_pos = [&](uint32_t id, uint32_t org) {
+    const uint32_t d = id - (org >> 16) * a.win_w;
+    const uint32_t r = row_of(d), jx = d - r * a.win_w - (org & 0xffffu);
+    return ((4u * (r & 31u) + 2u * (r >> 5) + (jx >> 5)) << 5) | (jx & 31u);
+  };
+  // ---- learning left pending by the previous call, then the bitmaps ----------
+  if (helper) {
+    copy_band(s_band, a.frames + w_lo, brows, blen, pitch, &s_band_bar[0]);
+  } else {
+    for (uint32_t i = 0; i < own; ++i) {
+      const uint32_t lc = own_col(i);
+      if (lc >= nc) continue;
+      const uint32_t c = c0 + lc;
+      const bool pend = a.pend_mask && ((__ldg(a.pend_mask + (c >> 5)) >> (c & 31u)) & 1u);
+      if (kWindow) {
+        const uint32_t org = s_org[lc];
+        uint32_t* wb = s_bits + lc * kBoxWords;
+        reinterpret_cast<uint4*>(wb)[lane] = make_uint4(0u, 0u, 0u, 0u);
+        if (lane == 0u)
+          s_at[lc] = ((((org >> 16) - y_lo) * pitch + ((org & 0xffffu) >> 5)) << 5) | (org & 31u);
+        __syncwarp();
+        for (uint32_t s = lane; s < S; s += 32u) {
+          const uint64_t e = g0 + (uint64_t)lc * S + s;
+          const uint32_t id = __ldg(a.idx + e), pos = box_pos(id, org);
+          float p = a.perm[e];
+          if (pend) p = learn_one(p, dev::input_bit(a.pend_x, id), a.inc, a.dec);
+          if (kPermSmem) {
+            s_pos[lc * S + s] = (uint16_t)pos;
+            s_perm[lc * S + s] = p;
+          } else if (pend) {
+            a.perm[e] = p;
           }
+          if (p >= a.thr) atomicOr(wb + (pos >> 5), 1u << (pos & 31u));
+        }
+      } else if (pend) {
+        for (uint32_t s = lane; s < S; s += 32u) {
+          const uint32_t e = lc * S + s;
+          s_perm[e] = learn_one(s_perm[e], dev::input_bit(a.pend_x, s_idx[e]), a.inc, a.dec);
         }
       }
-      uint32_t mine = 0u;
+      if (pend && kPermSmem && lane == 0u) atomicOr(s_dirty + (lc >> 5), 1u << (lc & 31u));
+    }
+  }
+  // barriers initialized, counts cleared and bitmaps built in every CTA
+  // before anyone sends
+  cluster.sync();
+
+  bool ok = true;  // this thread's waits so far
+  uint32_t f = 0;
+  if (helper) {
+    for (; f < a.n_frames; ++f) {
+      const uint32_t par = f & 1u;
+      if (__syncthreads_or(0)) {  // B1: frame f counted, frame f - 1 done with
+        ok = false;
+        if (fast) break;
+      }
+      const uint32_t h = t - kSeqThreads;
+      if (fast && Q > 1u && h == 0u) mbar_expect(&s_cnt_bar[par], (Q - 1u) * Cq * 2u);
+      if (f + 1u < a.n_frames)
+        copy_band(s_band + (par ^ 1u) * a.band_max, a.frames + (uint64_t)(f + 1u) * a.stride + w_lo,
+                  brows, blen, pitch, &s_band_bar[par ^ 1u]);
+      if (!fast) cluster.sync();  // every CTA's overlaps of frame f are published
+      // the masks of frame f - 1; the mask of frame f + 1 and the histogram of
+      // frame f + 2 cleared (their last readers passed B1)
+      const uint32_t* pm = sm + L.mask + ((f + 2u) % 3u) * mw;
+      uint32_t* zm = sm + L.mask + ((f + 1u) % 3u) * mw;
+      for (uint32_t i = h; i < mw; i += kSeqHelpers) {
+        if (f > 0u && a.masks_out && c0 / 32u + i < a.mask_words)
+          a.masks_out[(uint64_t)(f - 1u) * a.mask_words + c0 / 32u + i] = pm[i];
+        zm[i] = 0u;
+      }
+      if (fast && global) {
+        uint32_t* zh = sm + L.hist + ((f + 2u) % 3u) * hw;
+        for (uint32_t i = h; i < hw; i += kSeqHelpers) zh[i] = 0u;
+      }
+      if (a.ov_all) {
+        const uint16_t* cnt = reinterpret_cast<const uint16_t*>(sm + L.cnt + par * cnt_words) + c0;
+        const float* ov = reinterpret_cast<const float*>(sm + L.ov) + par * Cq;
+        for (uint32_t i = h; i < nc; i += kSeqHelpers)
+          a.ov_all[(uint64_t)f * C + c0 + i] = fast ? __uint2float_rn((uint32_t)cnt[i]) : ov[i];
+      }
+    }
+  } else {
+    // a warp's columns' bitmaps and band positions stay in registers when it
+    // has few columns
+    const bool reg_bits = kWindow && passes <= (uint32_t)kSeqCols;
+    const uint32_t row32 = 32u * pitch;
+    uint4 bm[kSeqCols];
+    uint32_t off[kSeqCols], shf[kSeqCols];
+    // column j past p0 of this warp (a valid one: results past nc are dropped)
+    auto col_at = [&](uint32_t p0, int j) {
+      return min((p0 + (uint32_t)j) * kSeqWarps + warp, nc - 1u);
+    };
+    auto load_bits = [&](uint32_t lc) {
+      return reinterpret_cast<const uint4*>(s_bits + lc * kBoxWords)[lane];
+    };
+    if (reg_bits && nc) {
 #pragma unroll
       for (int j = 0; j < kSeqCols; ++j) {
-        const uint32_t c = __reduce_add_sync(kFull, cnt[j]);
-        if (lane == (uint32_t)j) mine = c;
+        const uint32_t lc = col_at(0u, j), at = s_at[lc];
+        bm[j] = load_bits(lc);
+        off[j] = (at >> 5) + lane * pitch;
+        shf[j] = at & 31u;
       }
-      const uint32_t lc = lc0 + lane * kSeqWarps;
-      if (lane < (uint32_t)kSeqCols && lc < nc) {
-        const bool keep = mine >= a.min_overlap && mine != 0u;
-        s_raw[lc] = keep ? mine : 0u;
-        if (fast) {
-          if (keep) {
-            atomicAdd(hpub + mine, 1u);
-            atomicMax(hpub, mine);  // bin 0: this CTA's largest count
+    }
+    for (; f < a.n_frames; ++f) {
+      const uint32_t par = f & 1u, phase = (f >> 1) & 1u;
+      const uint32_t* band = s_band + par * a.band_max;
+      uint32_t* s_cnt32 = sm + L.cnt + par * cnt_words;
+      uint16_t* s_cnt = reinterpret_cast<uint16_t*>(s_cnt32);  // [Q * Cq], column order
+      uint32_t* hist = sm + L.hist + (f % 3u) * hw;
+      uint32_t* smask_f = sm + L.mask + (f % 3u) * mw;
+      float* ov_pub = reinterpret_cast<float*>(sm + L.ov) + par * Cq;
+      if (ok) ok = mbar_wait<false>(&s_band_bar[par], phase);
+
+      // ---- Alg. 1 for this warp's columns ---------------------------------------
+      // every load of a step is issued before its first use: no branch
+      // separates the columns a warp counts side by side
+      uint32_t top = 0u;  // largest count seen by this thread
+      auto publish = [&](uint32_t lc, uint32_t raw) {
+        const uint32_t v = raw >= a.min_overlap ? raw : 0u;
+        if (!fast) {
+          ov_pub[lc] = dev::boosted(raw, a.min_overlap, s_boost[lc]);
+          return;
+        }
+        s_cnt[c0 + lc] = (uint16_t)v;
+        if (Q == 1u && global && v != 0u) {
+          atomicAdd(hist + v, 1u);
+          top = max(top, v);
+        }
+      };
+      auto count_window = [&](uint32_t p0) {
+        uint32_t n[kSeqCols], a0[kSeqCols][3], a1[kSeqCols][3];
+        if (!reg_bits) {
+#pragma unroll
+          for (int j = 0; j < kSeqCols; ++j) {
+            const uint32_t lc = col_at(p0, j), at = s_at[lc];
+            bm[j] = load_bits(lc);
+            off[j] = (at >> 5) + lane * pitch;
+            shf[j] = at & 31u;
+          }
+        }
+#pragma unroll
+        for (int j = 0; j < kSeqCols; ++j) {
+          const uint32_t* p = band + off[j];
+#pragma unroll
+          for (int i = 0; i < 3; ++i) {
+            a0[j][i] = p[i];
+            a1[j][i] = p[row32 + i];
+          }
+        }
+#pragma unroll
+        for (int j = 0; j < kSeqCols; ++j)
+          n[j] = __popc(__funnelshift_r(a0[j][0], a0[j][1], shf[j]) & bm[j].x) +
+                 __popc(__funnelshift_r(a0[j][1], a0[j][2], shf[j]) & bm[j].y) +
+                 __popc(__funnelshift_r(a1[j][0], a1[j][1], shf[j]) & bm[j].z) +
+                 __popc(__funnelshift_r(a1[j][1], a1[j][2], shf[j]) & bm[j].w);
+        uint32_t mine = 0u;
+#pragma unroll
+        for (int j = 0; j < kSeqCols; ++j) {
+          const uint32_t r = __reduce_add_sync(kFull, n[j]);
+          mine = lane == (uint32_t)j ? r : mine;
+        }
+        const uint32_t lc = (p0 + lane) * kSeqWarps + warp;
+        if (lane < (uint32_t)kSeqCols && lc < nc) publish(lc, mine);
+      };
+      // U groups of P columns side by side
+      auto count_pools = [&](uint32_t p0, auto u) {
+        constexpr int U = decltype(u)::value;
+        uint32_t n[U], row[U];
+        const uint32_t sub = lane / L32, sl = lane % L32;
+#pragma unroll
+        for (int j = 0; j < U; ++j) {
+          n[j] = 0u;
+          row[j] = min(((p0 + j) * kSeqWarps + warp) * P + sub, nc - 1u) * S;
+        }
+        auto bit = [&](uint32_t w, uint32_t id, float p) {
+          return p >= a.thr ? (w >> (id & 31u)) & 1u : 0u;
+        };
+        if ((S & 3u) == 0u) {
+          for (uint32_t v = sl; v < (S >> 2); v += L32) {
+            uint4 id[U], w[U];
+            float4 pm[U];
+#pragma unroll
+            for (int j = 0; j < U; ++j) {
+              id[j] = reinterpret_cast<const uint4*>(s_idx + row[j])[v];
+              pm[j] = reinterpret_cast<const float4*>(s_perm + row[j])[v];
+            }
+#pragma unroll
+            for (int j = 0; j < U; ++j)
+              w[j] = make_uint4(band[(id[j].x >> 5) - w_lo], band[(id[j].y >> 5) - w_lo],
+                                band[(id[j].z >> 5) - w_lo], band[(id[j].w >> 5) - w_lo]);
+#pragma unroll
+            for (int j = 0; j < U; ++j)
+              n[j] += bit(w[j].x, id[j].x, pm[j].x) + bit(w[j].y, id[j].y, pm[j].y) +
+                      bit(w[j].z, id[j].z, pm[j].z) + bit(w[j].w, id[j].w, pm[j].w);
           }
         } else {
-          ov_pub[lc] = dev::boosted(mine, a.min_overlap, s_boost[lc]);
+          for (uint32_t s = sl; s < S; s += L32) {
+            uint32_t id[U], w[U];
+            float pm[U];
+#pragma unroll
+            for (int j = 0; j < U; ++j) {
+              id[j] = s_idx[row[j] + s];
+              pm[j] = s_perm[row[j] + s];
+            }
+#pragma unroll
+            for (int j = 0; j < U; ++j) w[j] = band[(id[j] >> 5) - w_lo];
+#pragma unroll
+            for (int j = 0; j < U; ++j) n[j] += bit(w[j], id[j], pm[j]);
+          }
+        }
+        if (P == 1u) {
+          uint32_t mine = 0u;
+#pragma unroll
+          for (int j = 0; j < U; ++j) {
+            const uint32_t r = __reduce_add_sync(kFull, n[j]);
+            mine = lane == (uint32_t)j ? r : mine;
+          }
+          const uint32_t lc = (p0 + lane) * kSeqWarps + warp;
+          if (lane < (uint32_t)U && lc < nc) publish(lc, mine);
+        } else {
+          for (uint32_t o = 1u; o < L32; o <<= 1) {
+#pragma unroll
+            for (int j = 0; j < U; ++j) n[j] += __shfl_xor_sync(kFull, n[j], o);
+          }
+          // lane j of a column's lanes publishes the j-th group's count
+          uint32_t mine = n[0];
+#pragma unroll
+          for (int j = 1; j < U; ++j) mine = sl == (uint32_t)j ? n[j] : mine;
+          const uint32_t lc = ((p0 + sl) * kSeqWarps + warp) * P + sub;
+          if (sl < (uint32_t)U && lc < nc) publish(lc, mine);
+        }
+      };
+      if (nc) {
+        if (kWindow) {
+          for (uint32_t p0 = 0; p0 < passes; p0 += kSeqCols) count_window(p0);
+        } else {
+          uint32_t p0 = 0;
+          for (; p0 + 3u <= passes; p0 += 4u) count_pools(p0, IntC<4>{});
+          for (; p0 < passes; p0 += 2u) count_pools(p0, IntC<2>{});
         }
       }
-    }
-    cluster.sync();  // every CTA's overlaps (or count histogram) of frame f are published
-    const bool last = f + 1u == a.n_frames;
-    uint32_t total;
-    if (fast) {
-      total = 0u;
-      if (warp == 0)
-        total = decide_unit_global(cluster, hpub, s_raw, a.k, q, c0, nc, s_mask,
-                                   last ? a.result + 1 : nullptr);
-      // the previous frame's published histogram is no longer read by anyone
-      for (uint32_t b = t; b < L.hstride; b += kSeqThreads) s_hpub[(par ^ 1u) * L.hstride + b] = 0u;
-    } else {
+      if (fast && global && Q == 1u) {
+        top = __reduce_max_sync(kFull, top);
+        if (lane == 0u && top) atomicMax(hist, top);
+      }
+      // B1: every warp's counts are in place
+      if (__syncthreads_or(!ok ? 1 : 0)) {
+        ok = false;
+        if (fast) break;  // else the cluster barriers below are still to be met
+      }
 
-    // ---- gather all overlaps through DSMEM -------------------------------------
-    {
-    uint32_t nz = 0;
+      if (fast) {
+        // ---- all counts to every CTA --------------------------------------------
+        if (Q > 1u) {
+          if (warp < Q && warp != q) {
+            const uint32_t dst = peer_addr(smem_u32(s_cnt + c0), warp);
+            const uint32_t bar = peer_addr(smem_u32(&s_cnt_bar[par]), warp);
+            for (uint32_t u = lane; u < Cq / 8u; u += 32u)
+              send16(dst + u * 16u, reinterpret_cast<const uint4*>(s_cnt + c0)[u], bar);
+          }
+          if (ok) ok = mbar_wait<true>(&s_cnt_bar[par], phase);
+        }
+        if (global) {
+          if (Q > 1u) {
+            for (uint32_t i = t; i < cnt_words; i += kSeqThreads) {
+              const uint32_t w = s_cnt32[i], v0 = w & 0xffffu, v1 = w >> 16;
+              if (v0) atomicAdd(hist + v0, 1u);
+              if (v1) atomicAdd(hist + v1, 1u);
+              top = max(top, max(v0, v1));
+            }
+            top = __reduce_max_sync(kFull, top);
+            if (lane == 0u && top) atomicMax(hist, top);
+            compute_sync();
+          }
+          // warp m decides the CTA's columns 32m .. 32m + 31
+          if (warp < mw) {
+            // T = the k-th largest count (0 when at most k columns count);
+            // `need` of the `ties` columns at it win, in column order
+            uint32_t T = 0xffffffffu, need = 0u, ties = 0u;
+            const uint32_t k = a.k, c = c0 + 32u * warp + lane, v = s_cnt[c];
+            if (k != 0u) {
+              T = 0u;
+              uint32_t acc = 0u;
+              for (uint32_t b0 = hist[0]; b0 >= 1u; b0 = b0 > 32u ? b0 - 32u : 0u) {
+                const uint32_t bin = b0 > lane ? b0 - lane : 0u;
+                const uint32_t h = bin ? hist[bin] : 0u;
+                uint32_t inc = h;
+#pragma unroll
+                for (uint32_t o = 1; o < 32u; o <<= 1) {
+                  const uint32_t y = __shfl_up_sync(kFull, inc, o);
+                  if (lane >= o) inc += y;
+                }
+                const uint32_t hit = __ballot_sync(kFull, acc + inc >= k);
+                if (hit) {
+                  const int src = __ffs(hit) - 1;
+                  T = b0 - (uint32_t)src;
+                  ties = __shfl_sync(kFull, h, src);
+                  need = k - (acc + __shfl_sync(kFull, inc, src) - ties);
+                  break;
+                }
+                acc += __shfl_sync(kFull, inc, 31);
+              }
+            }
+            const bool tie = T != 0u && v == T;
+            bool win = T != 0xffffffffu && v > T;
+            const uint32_t tw = __ballot_sync(kFull, tie);
+            if (tw) {
+              uint32_t before = 0u;  // tied columns below this warp's
+              if (ties > need) {
+                const uint4* cv = reinterpret_cast<const uint4*>(s_cnt);
+                const uint32_t lim = (c0 + 32u * warp) / 8u, TT = T | (T << 16);
+                auto eq2 = [&](uint32_t w) {
+                  const uint32_t x = w ^ TT;
+                  return ((x & 0xffffu) == 0u ? 1u : 0u) + ((x >> 16) == 0u ? 1u : 0u);
+                };
 #pragma unroll 4
-    for (uint32_t i = t; i < C; i += kSeqThreads) {
-      const uint32_t owner = i / Cq;
-      const float* src = cluster.map_shared_rank(ov_pub, owner);
-      const uint32_t v = __float_as_uint(src[i - owner * Cq]);
-      s_all[i] = v;
-      nz += v != 0u;
-    }
-    for (uint32_t i = t; i < a.mask_words; i += kSeqThreads) s_mask[i] = 0u;
-    if (a.inhibition == 0u) {
-      uint32_t e0, e1, nz_tot, z;
-      dev::block_scan2<kSeqWarps>(nz, 0u, e0, e1, nz_tot, z, sh);
-      uint32_t T, need;
-      dev::select_threshold<kSeqThreads>(s_all, C, a.k, nz_tot, nullptr,
-                                         a.unit_boost ? S : 0u, s_hist, sh, s2, T, need);
-      total = dev::mark_global<kSeqThreads>(s_all, C, T, need, s_mask,
-                                            (last && q == 0u) ? a.result + 1 : nullptr, sh);
-    } else {
-      __syncthreads();
-      // every CTA marks all columns: the list offsets then need no exchange
-      total = dev::mark_local<kSeqThreads>(s_all, 0u, C, a.gw, a.gh, a.radius, a.k, s_mask,
-                                           (last && q == 0u) ? a.result + 1 : nullptr, sh);
-    }
-    }
-    }
-    __syncthreads();
-    // ---- outputs: this CTA's mask words; the last frame's list and overlaps
-    const uint32_t mw0 = c0 / 32u, mw1 = min(a.mask_words, (c0 + nc + 31u) / 32u);
-    if (a.masks_out)
-      for (uint32_t i = mw0 + t; i < mw1; i += kSeqThreads)
-        a.masks_out[(uint64_t)f * a.mask_words + i] = s_mask[i];
-    if (a.ov_all)
-      for (uint32_t i = t; i < nc; i += kSeqThreads)
-        a.ov_all[(uint64_t)f * C + c0 + i] = fast ? __uint2float_rn(s_raw[i]) : ov_pub[i];
-    if (last) {
-      for (uint32_t i = mw0 + t; i < mw1; i += kSeqThreads) a.mask_last[i] = s_mask[i];
-      for (uint32_t i = t; i < nc; i += kSeqThreads)
-        a.ov_out[c0 + i] = fast ? __uint2float_rn(s_raw[i]) : ov_pub[i];
-      if (q == 0u && t == 0u) a.result[0] = total;
-    }
-
-    if (a.duty) {
-      for (uint32_t lc = t; lc < nc; lc += kSeqThreads) {
-        const uint32_t c = c0 + lc;
-        const float act = ((s_mask[c >> 5] >> (c & 31u)) & 1u) ? 1.0f : 0.0f;
-        const float d = a.duty[c];
-        a.duty[c] = __fadd_rn(d, __fdiv_rn(__fsub_rn(act, d), a.duty_period));
-      }
-    }
-
-    // ---- learning of this CTA's winners (frame band still resident) ---------
-    if (a.learn) {
-      for (uint32_t lc = warp; lc < nc; lc += kSeqWarps) {
-        const uint32_t c = c0 + lc;
-        if (!((s_mask[c >> 5] >> (c & 31u)) & 1u)) continue;
-        float* rp = s_perm + lc * S;
-        const uint32_t* ri = s_idx + lc * S;
-#pragma unroll 8
-        for (uint32_t s = lane; s < S; s += 32) {
-          const uint32_t id = ri[s];
-          const uint32_t bit = (band[(id >> 5) - w_lo] >> (id & 31u)) & 1u;
-          rp[s] = learn_one(rp[s], bit, a.inc, a.dec);
+                for (uint32_t i = lane; i < lim; i += 32u) {
+                  const uint4 w = cv[i];
+                  before += eq2(w.x) + eq2(w.y) + eq2(w.z) + eq2(w.w);
+                }
+                before = __reduce_add_sync(kFull, before);
+              }
+              win = win || (tie && before + __popc(tw & ((1u << lane) - 1u)) < need);
+            }
+            const uint32_t w = __ballot_sync(kFull, win);
+            if (lane == 0u) smask_f[warp] = w;
+          }
+        } else {
+          // local: G lanes share a column, each ranking it against every G-th
+          // row of its clipped (2r + 1)^2 neighbourhood.  A neighbour beats it
+          // with a higher count, or with an equal one and a lower index: rows
+          // above and columns to the left win ties
+          uint32_t n_own = 1u;
+          while (n_own < own) n_own <<= 1;
+          const uint32_t G = 32u / n_own, i = lane / G, g = lane % G;
+          const uint32_t lc = own_col(i), c = c0 + lc;
+          const uint32_t v = i < own && lc < nc ? s_cnt[c] : 0u;
+          uint32_t beaten = 0u;
+          if (v != 0u && a.k != 0u) {
+            const uint32_t x = c % a.gw, y = c / a.gw, r = a.radius;
+            const uint32_t x0 = x >= r ? x - r : 0u, x1 = min(a.gw - 1u, x + r);
+            const uint32_t y0 = y >= r ? y - r : 0u, y1 = min(a.gh - 1u, y + r);
+            // two columns a word: (count | 0x8000) - limit keeps its top bit
+            // where the count reaches the limit (counts are below 0x8000)
+            uint32_t two = 0u;  // a 16-bit sum per half
+            for (uint32_t jj = y0 + g; jj <= y1; jj += G) {
+              if (jj == y) {
+                for (uint32_t ii = x0; ii <= x1; ++ii)
+                  beaten += s_cnt[jj * a.gw + ii] >= (ii < x ? v : v + 1u) ? 1u : 0u;
+                continue;
+              }
+              const uint32_t lim = jj < y ? v : v + 1u, lim2 = lim | (lim << 16);
+              const uint32_t i0 = jj * a.gw + x0, i1 = jj * a.gw + x1;
+              const uint32_t w0 = i0 >> 1, w1 = i1 >> 1;
+              auto reach = [&](uint32_t w) {
+                return (((s_cnt32[w] | 0x80008000u) - lim2) >> 15) & 0x00010001u;
+              };
+              const uint32_t first = (i0 & 1u) ? 0x00010000u : 0x00010001u;
+              const uint32_t final = (i1 & 1u) ? 0x00010001u : 0x00000001u;
+              if (w0 == w1) {
+                two += reach(w0) & first & final;
+              } else {
+                two += (reach(w0) & first) + (reach(w1) & final);
+#pragma unroll 4
+                for (uint32_t w = w0 + 1u; w < w1; ++w) two += reach(w);
+              }
+            }
+            beaten += (two & 0xffffu) + (two >> 16);
+          }
+          for (uint32_t o = 1u; o < G; o <<= 1) beaten += __shfl_xor_sync(kFull, beaten, o);
+          if (g == 0u && v != 0u && beaten < a.k)
+            atomicOr(smask_f + (lc >> 5), 1u << (lc & 31u));
+          compute_sync();
         }
-        if (lane == 0) atomicOr(s_dirty + (lc >> 5), 1u << (lc & 31u));
+      } else {
+        // ---- non-unit boosts: gather all overlaps through DSMEM -------------------
+        cluster.sync();  // every CTA's overlaps of frame f are published
+        uint32_t* s_all = sm + L.all;
+        uint32_t* s_smask = sm + L.smask;
+        uint32_t nz = 0;
+#pragma unroll 4
+        for (uint32_t i = t; i < C; i += kSeqThreads) {
+          const uint32_t owner = i / Cq;
+          const float* src = cluster.map_shared_rank(ov_pub, owner);
+          const uint32_t v = __float_as_uint(src[i - owner * Cq]);
+          s_all[i] = v;
+          nz += v != 0u;
+        }
+        for (uint32_t i = t; i < a.mask_words; i += kSeqThreads) s_smask[i] = 0u;
+        if (global) {
+          uint32_t e0, e1, nz_tot, z, Tb, nd;
+          dev::block_scan2<kSeqWarps>(nz, 0u, e0, e1, nz_tot, z, sh);
+          dev::select_threshold<kSeqThreads>(s_all, C, a.k, nz_tot, nullptr, 0u, sm + L.shist, sh,
+                                             s2, Tb, nd);
+          dev::mark_global<kSeqThreads>(s_all, C, Tb, nd, s_smask, nullptr, sh);
+        } else {
+          compute_sync();
+          dev::mark_local<kSeqThreads>(s_all, 0u, C, a.gw, a.gh, a.radius, a.k, s_smask, nullptr,
+                                       sh);
+        }
+        compute_sync();
+        if (warp < mw && lane == 0u)
+          smask_f[warp] = c0 / 32u + warp < a.mask_words ? s_smask[c0 / 32u + warp] : 0u;
+      }
+
+      // ---- the winners' list (in no order), duty cycles ---------------------------
+      if (warp < mw) {
+        __syncwarp();
+        const uint32_t w = smask_f[warp], lc = 32u * warp + lane;
+        if (a.duty && lc < nc) {
+          const float d = a.duty[c0 + lc], act = (w >> lane) & 1u ? 1.0f : 0.0f;
+          a.duty[c0 + lc] = __fadd_rn(d, __fdiv_rn(__fsub_rn(act, d), a.duty_period));
+        }
+        if (a.learn && w != 0u) {
+          uint32_t at = 0u;
+          if (lane == 0u) at = atomicAdd(&s_n, (uint32_t)__popc(w));
+          at = __shfl_sync(kFull, at, 0) + __popc(w & ((1u << lane) - 1u));
+          if ((w >> lane) & 1u) s_list[at] = (uint16_t)lc;
+        }
+      }
+      if (!a.learn) continue;
+      compute_sync();
+      // ---- learning: the listed winners' synapses, 32 J of one column a unit,
+      // units dealt to the warps; a unit's loads are issued before the first is
+      // used.  Few winners: small units, so that their chains are short
+      const uint32_t n_win = s_n;
+      auto learn = [&](auto jc) {
+        constexpr int J = decltype(jc)::value;
+        const uint32_t parts = (S + 32u * J - 1u) / (32u * J), units = n_win * parts;
+        for (uint32_t u = warp; u < units; u += kSeqWarps) {
+          const uint32_t i = u / parts, s0 = (u - i * parts) * 32u * J + lane;
+          const uint32_t lc = s_list[i];
+          uint32_t* wb = s_bits + lc * kBoxWords;
+          uint32_t at = 0u, org = 0u;
+          if (kWindow) {
+            at = s_at[lc];
+            org = s_org[lc];
+          }
+          const uint64_t e0 = g0 + (uint64_t)lc * S;
+          uint32_t id[J], bit[J];
+          float p[J];
+#pragma unroll
+          for (int j = 0; j < J; ++j) {
+            const uint32_t s = min(s0 + 32u * j, S - 1u);
+            id[j] = FORM == kSeqPools ? s_idx[lc * S + s]
+                                      : (kPermSmem ? (uint32_t)s_pos[lc * S + s]
+                                                   : __ldg(a.idx + e0 + s));
+            p[j] = kPermSmem ? s_perm[lc * S + s] : __ldcg(a.perm + e0 + s);
+          }
+#pragma unroll
+          for (int j = 0; j < J; ++j) {
+            if (FORM == kSeqPools) {
+              bit[j] = (band[(id[j] >> 5) - w_lo] >> (id[j] & 31u)) & 1u;
+            } else {
+              if (!kPermSmem) id[j] = box_pos(id[j], org);
+              const uint32_t r = (id[j] >> 7) + ((id[j] & 64u) >> 1);
+              const uint32_t x = (at & 31u) + (id[j] & 63u);  // word parity and bit: the pixel
+              bit[j] = (band[(at >> 5) + r * pitch + (x >> 5)] >> (x & 31u)) & 1u;
+            }
+          }
+#pragma unroll
+          for (int j = 0; j < J; ++j) {
+            const uint32_t s = s0 + 32u * j;
+            const float np = learn_one(p[j], bit[j], a.inc, a.dec);
+            if (s < S) {
+              if (kPermSmem)
+                s_perm[lc * S + s] = np;
+              else
+                __stcg(a.perm + e0 + s, np);
+              if (kWindow && (np >= a.thr) != (p[j] >= a.thr))
+                atomicXor(wb + (id[j] >> 5), 1u << (id[j] & 31u));
+            }
+          }
+          if (kPermSmem && lane == 0u && s0 == 0u) atomicOr(s_dirty + (lc >> 5), 1u << (lc & 31u));
+        }
+      };
+      if (S <= 64u || n_win * S <= 2048u)
+        learn(IntC<2>{});
+      else
+        learn(IntC<kPermSmem ? 8 : 4>{});  // the box positions of 8 would spill
+      compute_sync();  // the next count reads what other warps learnt
+      if (t == 0u) s_n = 0u;
+      if (reg_bits && nc) {
+#pragma unroll
+        for (int j = 0; j < kSeqCols; ++j) {
+          const uint32_t lc = col_at(0u, j);
+          if ((smask_f[lc >> 5] >> (lc & 31u)) & 1u) bm[j] = load_bits(lc);
+        }
       }
     }
   }
-  cp_async_wait_all();
-  __syncthreads();
-  // ---- write back the permanence rows that changed ---------------------------
-  for (uint32_t lc = warp; lc < nc; lc += kSeqWarps) {
-    if (!((s_dirty[lc >> 5] >> (lc & 31u)) & 1u)) continue;
-    float* gp = a.perm + g0 + (uint64_t)lc * S;
-    for (uint32_t s = lane; s < S; s += 32) gp[s] = s_perm[lc * S + s];
+  if (!ok) {
+    // a wait gave up: report it, and wait (bounded) for what may still be on
+    // its way into this CTA's shared memory
+    if (a.err) atomicExch(a.err, 1u);
+    if (!helper && fast && Q > 1u && f < a.n_frames) {
+      if (t == 0) mbar_expect(&s_cnt_bar[f & 1u], (Q - 1u) * Cq * 2u);
+      mbar_wait<true>(&s_cnt_bar[f & 1u], (f >> 1) & 1u);
+    }
   }
-  // no CTA may exit while another can still read its shared memory
+  asm volatile("cp.async.wait_all;\n" ::: "memory");
+  __syncthreads();
+  // ---- the last frame's outputs, and the permanence rows that changed ------------
+  const uint32_t last = a.n_frames - 1u;
+  const uint32_t* lmask = sm + L.mask + (last % 3u) * mw;
+  for (uint32_t i = t; i < mw; i += kAll) {
+    const uint32_t w = c0 / 32u + i;
+    if (w < a.mask_words) {
+      if (a.masks_out) a.masks_out[(uint64_t)last * a.mask_words + w] = lmask[i];
+      a.mask_last[w] = lmask[i];
+    }
+  }
+  {
+    const uint16_t* cnt = reinterpret_cast<const uint16_t*>(sm + L.cnt + (last & 1u) * cnt_words);
+    const float* ov = reinterpret_cast<const float*>(sm + L.ov) + (last & 1u) * Cq;
+    for (uint32_t i = t; i < nc; i += kAll)
+      a.ov_out[c0 + i] = fast ? __uint2float_rn((uint32_t)cnt[c0 + i]) : ov[i];
+  }
+  if (kPermSmem) {
+    for (uint32_t lc = warp; lc < nc; lc += kAll / 32u) {
+      if (!((s_dirty[lc >> 5] >> (lc & 31u)) & 1u)) continue;
+      float* gp = a.perm + g0 + (uint64_t)lc * S;
+      for (uint32_t s = lane; s < S; s += 32) gp[s] = s_perm[lc * S + s];
+    }
+  }
+  cluster.sync();  // every CTA's mask of the last frame is final
+  if (q == 0u && warp == 0u) {
+    // ascending list of the last frame's winners, 32 mask words at a time
+    uint32_t total = 0u;
+    for (uint32_t b = 0; b < a.mask_words; b += 32u) {
+      const uint32_t w = b + lane, owner = w / mw;
+      uint32_t m = 0u;
+      if (w < a.mask_words) m = cluster.map_shared_rank(lmask, owner)[w - owner * mw];
+      const uint32_t n = __popc(m);
+      uint32_t inc = n;
+#pragma unroll
+      for (uint32_t o = 1; o < 32u; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(kFull, inc, o);
+        if (lane >= o) inc += y;
+      }
+      uint32_t pos = total + inc - n;
+      for (; m != 0u; m &= m - 1u) a.result[1 + pos++] = w * 32u + (uint32_t)(__ffs(m) - 1);
+      total += __shfl_sync(kFull, inc, 31);
+    }
+    if (lane == 0u) a.result[0] = total;
+  }
+  // no CTA may exit while another can still read or write its shared memory
   cluster.sync();
+}
+
+using SeqKernel = void (*)(const SeqArgs);
+
+SeqKernel seq_kernel(uint32_t form) {
+  return form == kSeqPools ? sp_seq_cluster_kernel<kSeqPools>
+                           : (form == kSeqWindow ? sp_seq_cluster_kernel<kSeqWindow>
+                                                 : sp_seq_cluster_kernel<kSeqWindowL2>);
 }
 
 }  // namespace
 
-size_t seq_smem_bytes(uint32_t C, uint32_t S, uint32_t Cq, uint32_t band_max) {
-  return (size_t)SeqLayout(Cq, S, band_max, C).total * 4u;
+size_t seq_smem_bytes(uint32_t form, uint32_t Q, uint32_t C, uint32_t S, uint32_t Cq,
+                      uint32_t band_max) {
+  return (size_t)SeqLayout(form, Q, Cq, S, band_max, C).total * 4u;
 }
 
-cudaError_t seq_kernel_init(size_t smem_bytes) {
-  cudaError_t e = cudaFuncSetAttribute(sp_seq_cluster_kernel,
-                                       cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+cudaError_t seq_kernel_init(uint32_t form, size_t smem_bytes) {
+  const SeqKernel k = seq_kernel(form);
+  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
   if (e != cudaSuccess) return e;
-  return cudaFuncSetAttribute(sp_seq_cluster_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              (int)smem_bytes);
+  return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes);
 }
 
-cudaError_t seq_max_active_clusters(uint32_t Q, size_t smem_bytes, int* out) {
+cudaError_t seq_max_active_clusters(uint32_t form, uint32_t Q, size_t smem_bytes, int* out) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(Q, 1, 1);
-  cfg.blockDim = dim3(kSeqThreads, 1, 1);
+  cfg.blockDim = dim3(kSeqThreads + kSeqHelpers, 1, 1);
   cfg.dynamicSmemBytes = smem_bytes;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -448,13 +958,14 @@ cudaError_t seq_max_active_clusters(uint32_t Q, size_t smem_bytes, int* out) {
   attr[0].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaOccupancyMaxActiveClusters(out, sp_seq_cluster_kernel, &cfg);
+  return cudaOccupancyMaxActiveClusters(out, seq_kernel(form), &cfg);
 }
 
-cudaError_t launch_seq(const SeqArgs& a, uint32_t Q, size_t smem_bytes, cudaStream_t stream) {
+cudaError_t launch_seq(const SeqArgs& a, uint32_t form, uint32_t Q, size_t smem_bytes,
+                       cudaStream_t stream) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(Q, 1, 1);
-  cfg.blockDim = dim3(kSeqThreads, 1, 1);
+  cfg.blockDim = dim3(kSeqThreads + kSeqHelpers, 1, 1);
   cfg.dynamicSmemBytes = smem_bytes;
   cfg.stream = stream;
   cudaLaunchAttribute attr[1];
@@ -464,7 +975,7 @@ cudaError_t launch_seq(const SeqArgs& a, uint32_t Q, size_t smem_bytes, cudaStre
   attr[0].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  const cudaError_t e = cudaLaunchKernelEx(&cfg, sp_seq_cluster_kernel, a);
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, seq_kernel(form), a);
   g_launches.fetch_add(1, std::memory_order_relaxed);
   return e;
 }
