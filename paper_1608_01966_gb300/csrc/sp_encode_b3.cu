@@ -1,0 +1,10 @@
+// Encoder kernels of window sizes 3 and 5 (a translation unit per pair, so
+// that they compile in parallel).
+#include "sp_encode_kernel.cuh"
+
+namespace sp {
+namespace enc {
+template cudaError_t launch_block<3>(const EncodeArgs&, bool, cudaStream_t);
+template cudaError_t launch_block<5>(const EncodeArgs&, bool, cudaStream_t);
+}  // namespace enc
+}  // namespace sp

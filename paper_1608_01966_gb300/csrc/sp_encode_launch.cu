@@ -1,0 +1,70 @@
+// Launch shape of the frame encoder: the reading mode, strips and row chunks.
+#include "sp_encode_kernel.cuh"
+
+#include <algorithm>
+#include <atomic>
+
+namespace sp {
+
+extern std::atomic<uint64_t> g_launches;
+
+cudaError_t launch_encode(EncodeArgs a, uint32_t block, cudaStream_t st) {
+  const bool a8 = reinterpret_cast<uintptr_t>(a.src) % 8u == 0u && a.src_stride % 8u == 0u &&
+                  (uint64_t)a.W * a.ch % 8u == 0u && a.Wr % 8u == 0u;
+  a.strips = (a.Wr + enc::kStrip - 1u) / enc::kStrip;
+  // Which kernel.  Blocks of 3 x 3 pixels and more: a strip's halo rows cost f
+  // times as many source rows each, so the band kernel, whose CTAs share them,
+  // reads less (128 frames of 960 x 540, f 4: 56 us against 136).  Below that a
+  // strip kernel's time goes with the strips walked, the band kernel's with
+  // the pixels, so strips have to be filled: to the percentage where the two
+  // meet, by how costly a strip's rows are to read (128 frames of 400 rows, us,
+  // strip / band: aligned f 1 RGB width 96 27 / 36, 48 31 / 25; aligned f 2 RGB
+  // 160 68 / 119, 96 87 / 64; unaligned f 1 RGB 321 74 / 103, 97 56 / 40, gray
+  // 250 56 / 83, 97 37 / 39; unaligned f 2 RGB 481 331 / 370, 250 240 / 201,
+  // gray 250 97 / 142, 97 73 / 62; full strips, 960 x 540, f 1 RGB: 84 / 211).
+  const uint32_t fill = a.f == 1u ? (a8 ? 40u : (a.ch == 1u ? 45u : 60u))
+                                  : (a.ch == 1u ? 50u : (a8 ? 60u : 75u));
+  if (a.f >= 3u || a.Wr < 8u || a.Wr * 100u < a.strips * enc::kStrip * fill)
+    return launch_encode_band(a, block, st);
+  // Rows per chunk: every chunk reads block - 1 rows besides its own, a chunk
+  // per warp; the fewest rows walked by the warps of a full machine in whole
+  // waves (16 warps resident per SM, at 128 registers a thread)
+  int dev = 0, sms = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  if (e != cudaSuccess) return e;
+  const uint64_t resident = 16ull * (uint64_t)std::max(1, sms);
+  uint64_t best = ~0ull;
+  a.rows = a.Hr;
+  for (uint32_t chunks = 1; chunks <= a.Hr; ++chunks) {
+    const uint32_t rows = (a.Hr + chunks - 1u) / chunks;
+    if (chunks > 1u && rows < 4u) break;
+    const uint64_t units = (uint64_t)a.n_frames * a.strips * ((a.Hr + rows - 1u) / rows);
+    const uint64_t cost = (units + resident - 1u) / resident * (rows + block + 3u);
+    if (cost < best) {
+      best = cost;
+      a.rows = rows;
+    }
+  }
+  a.chunks = (a.Hr + a.rows - 1u) / a.rows;
+  const uint64_t units = (uint64_t)a.n_frames * a.strips * a.chunks;
+  if (units > 0x7fffffffull) return cudaErrorInvalidValue;
+  a.units = (uint32_t)units;
+  if (a.Wr % 8u != 0u) {
+    // rows that start inside a byte are OR'ed into words
+    e = cudaMemset2DAsync(a.out, a.out_stride * 4u, 0, (size_t)a.n_words * 4u, a.n_frames, st);
+    if (e != cudaSuccess) return e;
+  }
+  switch (block) {
+    case 3: e = enc::launch_block<3>(a, a8, st); break;
+    case 5: e = enc::launch_block<5>(a, a8, st); break;
+    case 7: e = enc::launch_block<7>(a, a8, st); break;
+    case 9: e = enc::launch_block<9>(a, a8, st); break;
+    case 11: e = enc::launch_block<11>(a, a8, st); break;
+    default: e = enc::launch_block<13>(a, a8, st); break;
+  }
+  g_launches.fetch_add(1, std::memory_order_relaxed);
+  return e;
+}
+
+}  // namespace sp
