@@ -143,67 +143,21 @@ void free_handle(sp_handle* h) {
   delete h;
 }
 
-// The pools as the sequence kernel's plan sees them: each column's smallest
-// and largest input, and, while every column's pool is strictly ascending (so
-// no input appears twice and a bitmap counts it once) and fits a 64 x 64 box
-// of the frame, the first frame row of its box.
-struct PoolScan {
-  std::vector<uint32_t> lo, hi, row;
-  bool boxes = true;
-};
-
-PoolScan scan_pools(uint32_t C, uint32_t S, uint32_t W, const uint32_t* idx) {
-  PoolScan p;
-  p.lo.resize(C);
-  p.hi.resize(C);
-  p.row.resize(C);
-  p.boxes = W % 32u == 0u && S <= 4096u;
-  for (uint32_t c = 0; c < C; ++c) {
-    const uint32_t* x = idx + (size_t)c * S;
-    uint32_t mn = x[0], mx = x[0];
-    if (p.boxes) {
-      // one division per row change: `base` is the current row's first input
-      uint32_t base = x[0] / W * W, x0 = x[0] - base, x1 = x0;
-      bool fit = true;
-      p.row[c] = base / W;
-      const uint64_t limit = (uint64_t)base + (uint64_t)64u * W;  // rows of the box
-      for (uint32_t s = 1; s < S && fit; ++s) {
-        fit = x[s] > x[s - 1] && x[s] < limit;
-        if (!fit) break;
-        if (x[s] - base >= W) base = x[s] / W * W;
-        const uint32_t px = x[s] - base;
-        x0 = std::min(x0, px);
-        x1 = std::max(x1, px);
-      }
-      fit = fit && x1 - x0 < 64u && x0 <= 0xffffu && p.row[c] <= 0xffffu;
-      p.boxes = fit;
-      if (fit) {
-        p.lo[c] = x[0];
-        p.hi[c] = x[S - 1];
-        continue;
-      }
-    }
-    for (uint32_t s = 1; s < S; ++s) {
-      mn = std::min(mn, x[s]);
-      mx = std::max(mx, x[s]);
-    }
-    p.lo[c] = mn;
-    p.hi[c] = mx;
-  }
-  return p;
-}
-
 // Decide whether whole frame sequences of this SP can run in one persistent
 // cluster launch, and in which form: Q CTAs of Cq columns (a multiple of 32)
 // must hold their state and input bands in shared memory, and the device must
-// be able to schedule such a cluster.  Failure only disables the path.
-void plan_cluster_path(sp_handle* h, const uint32_t* idx) {
+// be able to schedule such a cluster.  scan: launch_pool_scan's results.
+// Failure only disables the path.
+void plan_cluster_path(sp_handle* h, const uint32_t* scan) {
   h->seq_ok = false;
   if (h->cfg.inhibition == SP_INHIBIT_PAPER_LITERAL) return;  // per-frame kernel only
-  const PoolScan p = scan_pools(h->C, h->S, h->cfg.input_w, idx);
+  const uint32_t *lo = scan, *hi = scan + h->C, *row = scan + 2u * h->C;
+  const bool boxes = std::find(row, row + h->C, 0xffffffffu) == row + h->C;
   uint32_t Q = std::min((h->C + 31u) / 32u, sp::kSeqMaxCluster);
   // small SPs: one CTA counts them in less time than a cluster exchanges counts
-  if (h->C <= (uint32_t)sp::kSeqThreads && (uint64_t)h->C * h->S <= kSeqOneCtaSynapses) Q = 1u;
+  if (h->C <= (uint32_t)sp::kSeqThreads && (uint64_t)h->C * h->S <= kSeqOneCtaSynapses &&
+      h->n_words <= kSeqOneCtaWords)
+    Q = 1u;
   const uint32_t Cq = (((h->C + Q - 1u) / Q) + 31u) & ~31u;
   if (Cq > (uint32_t)sp::kSeqThreads) return;  // a warp's columns are a 32-bit mask
   const uint32_t wpr = h->cfg.input_w / 32u;
@@ -213,15 +167,15 @@ void plan_cluster_path(sp_handle* h, const uint32_t* idx) {
       const uint32_t c1 = std::min(h->C, c0 + Cq);
       uint64_t w_lo, w_hi;
       if (form == sp::kSeqPools) {
-        const uint32_t mn = *std::min_element(p.lo.begin() + c0, p.lo.begin() + c1);
-        const uint32_t mx = *std::max_element(p.hi.begin() + c0, p.hi.begin() + c1);
+        const uint32_t mn = *std::min_element(lo + c0, lo + c1);
+        const uint32_t mx = *std::max_element(hi + c0, hi + c1);
         w_lo = mn >> 5;
         w_hi = (mx >> 5) + 1u;
       } else {
         // whole rows, padded to an odd number of words, 64 past the last box's
         // first, and the word past the end that an unaligned segment reads
-        const uint64_t y0 = *std::min_element(p.row.begin() + c0, p.row.begin() + c1);
-        const uint64_t y1 = *std::max_element(p.row.begin() + c0, p.row.begin() + c1);
+        const uint64_t y0 = *std::min_element(row + c0, row + c1);
+        const uint64_t y1 = *std::max_element(row + c0, row + c1);
         w_lo = y0 * (wpr | 1u);
         w_hi = (y1 + 64u) * (wpr | 1u) + 4u;
       }
@@ -232,7 +186,7 @@ void plan_cluster_path(sp_handle* h, const uint32_t* idx) {
   };
   uint32_t band[3] = {0, 0, 0};
   size_t smem[3] = {bytes(sp::kSeqPools, &band[0]), (size_t)-1, (size_t)-1};
-  if (p.boxes) {
+  if (boxes) {
     smem[1] = bytes(sp::kSeqWindow, &band[1]);
     smem[2] = bytes(sp::kSeqWindowL2, &band[2]);
   }
@@ -305,7 +259,7 @@ sp_status init_handle(sp_handle* h, const sp_config* cfg, const uint32_t* idx, c
   h->d_hist = reinterpret_cast<uint32_t*>(b + off[8]);
   h->d_duty = reinterpret_cast<float*>(b + off[9]);
   h->d_err = reinterpret_cast<uint32_t*>(b + off[10]);
-  SP_CUDA(cudaMallocHost(&h->h_result, ((size_t)h->C + 1) * 4));
+  SP_CUDA(cudaMallocHost(&h->h_result, std::max((size_t)h->C + 1, (size_t)h->C * 3) * 4));
   SP_CUDA(cudaMallocHost(&h->h_err, 8));
   h->h_err[0] = h->h_err[1] = 0u;
   SP_CUDA(cudaStreamCreateWithFlags(&h->own_stream, cudaStreamNonBlocking));
@@ -324,6 +278,9 @@ sp_status init_handle(sp_handle* h, const sp_config* cfg, const uint32_t* idx, c
   h->dense = h->S == h->n_in;
   for (size_t e = 0; h->dense && e < CS; ++e) h->dense = idx[e] == (uint32_t)(e % h->S);
   SP_CUDA(cudaMemcpyAsync(h->d_boost, boost, (size_t)h->C * 4, cudaMemcpyHostToDevice, h->stream));
+  // the pools' extents for the sequence plan, into pinned memory (h_result
+  // holds nothing before the first frame)
+  SP_CUDA(sp::launch_pool_scan(h->d_idx, h->C, h->S, cfg->input_w, h->h_result, h->stream));
   SP_CUDA(cudaStreamSynchronize(h->stream));
   h->grid = sp::step_grid(h->C);
   plan_cluster_path(h, idx);

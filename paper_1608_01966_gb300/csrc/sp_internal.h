@@ -85,8 +85,18 @@ constexpr uint32_t kChunkFrames = 32;  // frames per staged chunk in sp_compute_
 constexpr int kSlots = 2;
 constexpr uint32_t kGraphMinFrames = 4;  // shorter sequences are launched directly
 constexpr uint32_t kSeqMinFrames = 8;    // shorter sequences use the per-frame kernel
-constexpr uint64_t kSeqOneCtaSynapses = 16384;  // sequences of at most these run in one CTA
-constexpr uint32_t kSeqWindowSynapses = 96;  // pools of at least these count faster as bitmaps
+// Sequences of SPs of at most so many synapses, on frames of at most so many
+// words, run in one CTA instead of a cluster, us per frame: 256 x 16 2.02
+// against 2.56, 512 x 16 2.51 / 2.65, 256 x 32 2.62 / 2.74, but 256 x 64 3.66 /
+// 2.75; and a lone CTA that must copy all 16,200 words of a 960 x 540 frame
+// takes 4.2 where a cluster, a band each, takes 2.8 (256 x 32).
+constexpr uint64_t kSeqOneCtaSynapses = 8192;
+constexpr uint32_t kSeqOneCtaWords = 2048;
+// Pools of at least so many synapses count faster as bitmaps (the pools' cost
+// grows with S, the bitmaps' does not), us per frame: 1024 columns S 64 3.00
+// against 3.09, S 192 3.21 / 3.85; 2025 columns S 64 3.88 / 3.64, S 96 3.88 /
+// 4.20; 4096 columns S 64 5.66 / 5.07.
+constexpr uint32_t kSeqWindowSynapses = 96;
 constexpr size_t kSeqSmemLimit = 231168u;  // 227 KiB per CTA, less 1.25 KiB of static shared memory
 
 inline bool seq_enabled() {

@@ -248,6 +248,13 @@ cudaError_t seq_kernel_init(uint32_t form, size_t smem_bytes);
 cudaError_t seq_max_active_clusters(uint32_t form, uint32_t Q, size_t smem_bytes, int* out);
 cudaError_t launch_seq(const SeqArgs& a, uint32_t form, uint32_t Q, size_t smem_bytes,
                        cudaStream_t stream);
+// What the plan of a sequence needs to know of the pools, per column: out[0][c]
+// and out[1][c] its smallest and largest input, out[2][c] the frame row of its
+// smallest, or 0xffffffff where a 64 x 64 bitmap cannot stand for the pool: it
+// is not strictly ascending (a synapse listed twice counts twice), does not fit
+// a 64 x 64 box, or the frame is not a multiple of 32 pixels wide.
+cudaError_t launch_pool_scan(const uint32_t* idx, uint32_t C, uint32_t S, uint32_t W,
+                             uint32_t* out, cudaStream_t stream);
 
 // Dense pools on the tensor cores (sp_dense_tc.cu): the raw overlaps of a run
 // of frames without learning as one {0,1} matrix product.  Both operands are

@@ -924,6 +924,41 @@ __global__ void __launch_bounds__(kSeqThreads + kSeqHelpers, 1) sp_seq_cluster_k
   cluster.sync();
 }
 
+// One warp per column.
+__global__ void __launch_bounds__(256) sp_pool_scan_kernel(const uint32_t* idx, uint32_t C,
+                                                           uint32_t S, uint32_t W, uint32_t* out) {
+  const uint32_t c = blockIdx.x * 8u + (threadIdx.x >> 5), lane = threadIdx.x & 31u;
+  if (c >= C) return;
+  const uint32_t* p = idx + (uint64_t)c * S;
+  const bool box = W % 32u == 0u && S <= 4096u;
+  uint32_t lo = 0xffffffffu, hi = 0u, x0 = 0xffffffffu, x1 = 0u;
+  bool ascending = true;
+  for (uint32_t s = lane; s < S; s += 32u) {
+    const uint32_t id = p[s];
+    lo = min(lo, id);
+    hi = max(hi, id);
+    if (s + 1u < S) ascending = ascending && p[s + 1u] > id;
+    if (box) {
+      const uint32_t x = id % W;
+      x0 = min(x0, x);
+      x1 = max(x1, x);
+    }
+  }
+  lo = __reduce_min_sync(kFull, lo);
+  hi = __reduce_max_sync(kFull, hi);
+  x0 = __reduce_min_sync(kFull, x0);
+  x1 = __reduce_max_sync(kFull, x1);
+  ascending = __all_sync(kFull, ascending);
+  if (lane == 0u) {
+    const uint32_t y0 = lo / W, y1 = hi / W;
+    const bool fits = box && ascending && x1 - x0 < 64u && y1 - y0 < 64u && x0 <= 0xffffu &&
+                      y0 <= 0xffffu;
+    out[c] = lo;
+    out[C + c] = hi;
+    out[2u * C + c] = fits ? y0 : 0xffffffffu;
+  }
+}
+
 using SeqKernel = void (*)(const SeqArgs);
 
 SeqKernel seq_kernel(uint32_t form) {
@@ -933,6 +968,13 @@ SeqKernel seq_kernel(uint32_t form) {
 }
 
 }  // namespace
+
+cudaError_t launch_pool_scan(const uint32_t* idx, uint32_t C, uint32_t S, uint32_t W,
+                             uint32_t* out, cudaStream_t stream) {
+  sp_pool_scan_kernel<<<(C + 7u) / 8u, 256, 0, stream>>>(idx, C, S, W, out);
+  g_launches.fetch_add(1, std::memory_order_relaxed);
+  return cudaGetLastError();
+}
 
 size_t seq_smem_bytes(uint32_t form, uint32_t Q, uint32_t C, uint32_t S, uint32_t Cq,
                       uint32_t band_max) {
