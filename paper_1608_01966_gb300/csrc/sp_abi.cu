@@ -1256,7 +1256,8 @@ struct sp_batch {
   uint32_t n_ctas_sparse = 0, max_C_sparse = 0;
   std::vector<sp::BatchDesc> h_desc;  // host copy of the descriptors
   void* d_sync = nullptr;             // persistent launches: work counter, abort, done[n]
-  std::vector<uint32_t> member_cpw;   // columns per warp of each member (0: batch_ctas' default)
+  std::vector<uint32_t> member_cpw;   // columns per warp of each member (0: the default)
+  uint32_t default_cpw = 0;           // the batch's default columns per warp (default_split)
   uint32_t sched = 0;                 // compiled schedule of the persistent pass (0: default)
   uint32_t stage_cap = 0;             // shared memory for staging state by bulk copy
   uint32_t xspan_cap = 0;             // shared memory for each CTA's input words
@@ -1310,6 +1311,24 @@ uint32_t batch_ctas(uint32_t C, uint32_t S, uint32_t cols_per_warp) {
 
 // Dynamic shared memory a batch launch offers for staging each CTA's
 // pools and permanences by bulk copy (0: the CTAs stream them from global
+// Columns per warp of a batch whose members together have `columns` columns,
+// the largest `largest`.  A frame of an SP is a chain (band or pools, count,
+// ticket, Alg. 2), and a warp's columns a chain inside it, so a warp gets the
+// fewest that keep a frame's items at most about twice the resident CTAs: with
+// more, each takes its ticket for too little work.  us per frame by columns per
+// warp 2 / 4 / 8 / 16 / 32: 8 SPs of 1024 x 256 16.5 16.4 17.6 19.9 25.5; 32: 19.6
+// 18.6 20.2 24.1 31.3; 64: 38 22.2 21.8 26.7 34.1; 128: 75 43 29.0 27.0 35.2; 200: 120
+// 70 46 34.6 39.2; 256: 159 93 61 44.9 43.3.  Where sizes are uneven the largest
+// SP's chain is the longest, and half as many items again pay: 64 SPs of 128 to
+// 4096 columns 91 54 41.9 45.5 59.7 (60.5 with 32, 16 or 8 by the synapses).
+uint32_t default_split(uint64_t columns, uint32_t members, uint32_t largest, int sms) {
+  uint64_t items = 22ull * (uint64_t)sms;  // 10 CTAs resident per SM
+  if ((uint64_t)largest * members * 2u >= columns * 3u) items += items / 2u;
+  uint32_t cpw = 2u;
+  while (cpw < 32u && columns > items * (uint64_t)(sp::kStepWarps * cpw)) cpw *= 2u;
+  return cpw;
+}
+
 // memory into registers).  Off unless SP_BATCH_STAGE_KB (1..64) allows it:
 // on 256 SPs of 1024x256 the staged form measured 0.29-0.47 of HBM peak
 // against 0.63 for the streamed one, since a CTA waits for all of its state
@@ -1606,12 +1625,23 @@ SP_API sp_status sp_batch_create(sp_handle* const* members, uint32_t n, sp_batch
   }
   std::vector<sp::BatchDesc> desc(n);
   std::vector<uint32_t> cta_inst;
+  uint64_t columns = 0;
+  uint32_t largest = 0;
+  for (uint32_t i = 0; i < n; ++i) {
+    columns += members[i]->C;
+    largest = std::max(largest, members[i]->C);
+  }
+  int sms = 0;
+  if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, b->device) != cudaSuccess || sms < 1)
+    sms = 1;
+  if (!std::getenv("SP_BATCH_COLS_PER_WARP"))
+    b->default_cpw = default_split(columns, n, largest, sms);
   uint64_t foff = 0, moff = 0, ooff = 0;
   for (uint32_t i = 0; i < n; ++i) {
     sp_handle* h = members[i];
     sp::BatchDesc& d = desc[i];
     uint32_t wb = 0;
-    fill_desc(h, &d, 0, &wb);
+    fill_desc(h, &d, b->default_cpw, &wb);
     b->win_cap = std::max(b->win_cap, wb);
     d.frame_off = foff;
     d.mask_off = moff;
@@ -2047,7 +2077,7 @@ sp_status batch_relayout(sp_batch* b, const std::vector<uint32_t>& cols_per_warp
   for (size_t i = 0; i < b->members.size(); ++i) {
     sp_handle* h = b->members[i];
     sp::BatchDesc& d = b->h_desc[i];
-    d.n_ctas = batch_ctas(h->C, h->S, cols_per_warp[i]);
+    d.n_ctas = batch_ctas(h->C, h->S, cols_per_warp[i] ? cols_per_warp[i] : b->default_cpw);
     d.cta_first = (uint32_t)cta_inst.size();
     d.xspan = batch_xspan_cap() > 0u ? handle_xspan(h, d.n_ctas) : nullptr;
     uint32_t wb = 0;
