@@ -283,7 +283,7 @@ sp_status init_handle(sp_handle* h, const sp_config* cfg, const uint32_t* idx, c
   SP_CUDA(sp::launch_pool_scan(h->d_idx, h->C, h->S, cfg->input_w, h->h_result, h->stream));
   SP_CUDA(cudaStreamSynchronize(h->stream));
   h->grid = sp::step_grid(h->C);
-  plan_cluster_path(h, idx);
+  plan_cluster_path(h, h->h_result);
   return SP_OK;
 }
 
@@ -337,7 +337,8 @@ sp::StepArgs base_args(const sp_handle* h) {
   a.ov = h->d_ov;
   a.result = h->d_result;
   a.counter = h->d_counter;
-  a.hist = (h->unit_boost && h->cfg.inhibition == SP_INHIBIT_GLOBAL) ? h->d_hist : nullptr;
+  a.unit = (h->unit_boost && h->cfg.inhibition == SP_INHIBIT_GLOBAL) ? 1u : 0u;
+  a.hist = a.unit && h->S > sp::kStepBins ? h->d_hist : nullptr;
   a.duty = h->cfg.duty_period > 0.0f ? h->d_duty : nullptr;
   a.duty_period = h->cfg.duty_period;
   a.C = h->C;
@@ -809,7 +810,8 @@ void fill_desc(sp_handle* h, sp::BatchDesc* d, uint32_t cols_per_warp, uint32_t*
   d->mask1 = h->d_mask[1];
   d->result = h->d_result;
   d->counter = h->d_counter;
-  d->hist = (h->unit_boost && h->cfg.inhibition == SP_INHIBIT_GLOBAL) ? h->d_hist : nullptr;
+  d->unit = (h->unit_boost && h->cfg.inhibition == SP_INHIBIT_GLOBAL) ? 1u : 0u;
+  d->hist = d->unit && h->S > sp::kStepBins ? h->d_hist : nullptr;
   d->duty = h->cfg.duty_period > 0.0f ? h->d_duty : nullptr;
   d->duty_period = h->cfg.duty_period;
   d->C = h->C;
@@ -1249,7 +1251,7 @@ struct sp_batch {
   void* d_block = nullptr;  // descriptors + CTA map
   sp::BatchDesc* d_desc = nullptr;
   uint32_t* d_cta_inst = nullptr;
-  uint32_t n_ctas = 0, max_C = 0;
+  uint32_t n_ctas = 0, max_C = 0, max_S = 0;  // max_S: of the members with S <= kStepBins
   // inference of a batch that mixes dense members (tensor cores) with others:
   // the CTA map of the others alone, for their persistent launch
   uint32_t* d_cta_sparse = nullptr;
@@ -1296,8 +1298,8 @@ namespace sp {
 namespace rt {
 
 // CTAs given to one SP in a batch launch: every warp takes several columns
-// so each CTA streams a few tens of KB of state (fewer, fatter CTAs keep the
-// per-CTA ticket and fence cost small).  SP_BATCH_COLS_PER_WARP overrides.
+// (fewer, fatter CTAs keep the per-CTA ticket and fence cost small).
+// SP_BATCH_COLS_PER_WARP overrides.
 uint32_t batch_ctas(uint32_t C, uint32_t S, uint32_t cols_per_warp) {
   uint32_t cpw = S >= 128u ? 32u : (S >= 32u ? 8u : 16u);
   if (const char* e = std::getenv("SP_BATCH_COLS_PER_WARP")) {
@@ -1309,8 +1311,6 @@ uint32_t batch_ctas(uint32_t C, uint32_t S, uint32_t cols_per_warp) {
   return (C + per_cta - 1u) / per_cta;
 }
 
-// Dynamic shared memory a batch launch offers for staging each CTA's
-// pools and permanences by bulk copy (0: the CTAs stream them from global
 // Columns per warp of a batch whose members together have `columns` columns,
 // the largest `largest`.  A frame of an SP is a chain (band or pools, count,
 // ticket, Alg. 2), and a warp's columns a chain inside it, so a warp gets the
@@ -1329,6 +1329,8 @@ uint32_t default_split(uint64_t columns, uint32_t members, uint32_t largest, int
   return cpw;
 }
 
+// Dynamic shared memory a batch launch offers for staging each CTA's
+// pools and permanences by bulk copy (0: the CTAs stream them from global
 // memory into registers).  Off unless SP_BATCH_STAGE_KB (1..64) allows it:
 // on 256 SPs of 1024x256 the staged form measured 0.29-0.47 of HBM peak
 // against 0.63 for the streamed one, since a CTA waits for all of its state
@@ -1489,7 +1491,7 @@ sp_status batch_enqueue(sp_batch* b, cudaStream_t st, const uint32_t* x_base, ui
     a.xspan_cap = b->xspan_cap;
     a.win_cap = b->win_cap;
     a.err = b->d_err;
-    SP_CUDA(sp::launch_batch_step(a, b->n_ctas, b->max_C, st));
+    SP_CUDA(sp::launch_batch_step(a, b->n_ctas, b->max_C, b->max_S, st));
     b->pending = learn != 0;
     b->cur ^= 1;
   }
@@ -1535,7 +1537,7 @@ sp_status batch_run(sp_batch* b, const uint32_t* x_base, uint32_t n, uint64_t st
     // counter, abort word and done flags start at 0 in every launch, so a
     // launch recorded into a graph and replayed sees no stale flags
     SP_CUDA(cudaMemsetAsync(b->d_sync, 0, 16 + b->members.size() * 4, b->stream));
-    SP_CUDA(sp::launch_batch_run(r, b->max_C, b->sched, b->stream));
+    SP_CUDA(sp::launch_batch_run(r, b->max_C, b->max_S, b->sched, b->stream));
     b->pending = learn != 0;
     b->cur ^= (int)(n & 1u);
     b->frames += n;
@@ -1623,8 +1625,6 @@ SP_API sp_status sp_batch_create(sp_handle* const* members, uint32_t n, sp_batch
       return s;
     }
   }
-  std::vector<sp::BatchDesc> desc(n);
-  std::vector<uint32_t> cta_inst;
   uint64_t columns = 0;
   uint32_t largest = 0;
   for (uint32_t i = 0; i < n; ++i) {
@@ -1636,6 +1636,8 @@ SP_API sp_status sp_batch_create(sp_handle* const* members, uint32_t n, sp_batch
     sms = 1;
   if (!std::getenv("SP_BATCH_COLS_PER_WARP"))
     b->default_cpw = default_split(columns, n, largest, sms);
+  std::vector<sp::BatchDesc> desc(n);
+  std::vector<uint32_t> cta_inst;
   uint64_t foff = 0, moff = 0, ooff = 0;
   for (uint32_t i = 0; i < n; ++i) {
     sp_handle* h = members[i];
@@ -1655,6 +1657,7 @@ SP_API sp_status sp_batch_create(sp_handle* const* members, uint32_t n, sp_batch
     foff += ((uint64_t)h->n_words + 3u) & ~uint64_t(3);  // 16-byte aligned members
     moff += h->mask_words;
     b->max_C = std::max(b->max_C, h->C);
+    if (h->S <= sp::kStepBins) b->max_S = std::max(b->max_S, h->S);
     b->stage_cap = std::max(b->stage_cap, sp::batch_stage_bytes(h->C, h->S, d.n_ctas));
   }
   b->stage_cap = batch_stage_cap(b->stage_cap);
@@ -1907,7 +1910,7 @@ SP_API sp_status sp_batch_infer_overlaps_device(sp_batch* b, const uint32_t* d_f
     r.win_cap = b->win_cap;
     r.wait_ns = b->wait_ns;
     SP_CUDA(cudaMemsetAsync(b->d_sync, 0, 16 + b->members.size() * 4, b->stream));
-    SP_CUDA(sp::launch_batch_run(r, b->max_C_sparse, b->sched, b->stream));
+    SP_CUDA(sp::launch_batch_run(r, b->max_C_sparse, b->max_S, b->sched, b->stream));
   }
   if (n == 0) {
     b->cur ^= (int)(n_frames & 1u);
@@ -2205,7 +2208,7 @@ SP_API sp_status sp_batch_autotune(sp_batch* b, const uint32_t* d_frames, uint32
         r.wait_ns = b->wait_ns;
         if (e == cudaSuccess)
           e = cudaMemsetAsync(b->d_sync, 0, 16 + b->members.size() * 4, b->stream);
-        if (e == cudaSuccess) e = sp::launch_batch_run(r, b->max_C, b->sched, b->stream);
+        if (e == cudaSuccess) e = sp::launch_batch_run(r, b->max_C, b->max_S, b->sched, b->stream);
       } else {
         for (uint32_t t = 0; t < n_frames && e == cudaSuccess; ++t) {
           sp::BatchArgs a{};
@@ -2217,7 +2220,7 @@ SP_API sp_status sp_batch_autotune(sp_batch* b, const uint32_t* d_frames, uint32
           a.xspan_cap = b->xspan_cap;
           a.win_cap = b->win_cap;
           a.err = b->d_err;
-          e = sp::launch_batch_step(a, b->n_ctas, b->max_C, b->stream);
+          e = sp::launch_batch_step(a, b->n_ctas, b->max_C, b->max_S, b->stream);
         }
       }
       if (e == cudaSuccess) e = cudaEventRecord(e1, b->stream);

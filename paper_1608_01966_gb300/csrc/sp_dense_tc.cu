@@ -363,7 +363,8 @@ __global__ void __launch_bounds__(kStepThreads) sp_frame_inhibit_kernel(const In
   __shared__ uint32_t s2[2];
   uint32_t* sv = dyn;
   uint32_t* smask = dyn + a.C;
-  uint32_t* shist = smask + a.mask_words;
+  uint32_t* stie = smask + a.mask_words;
+  uint32_t* shist = stie + a.mask_words;
   const uint32_t f = blockIdx.x, t = threadIdx.x;
   const float* ov = a.ov + (uint64_t)f * a.C;
   uint32_t nz = 0, vmax = 0;
@@ -390,7 +391,7 @@ __global__ void __launch_bounds__(kStepThreads) sp_frame_inhibit_kernel(const In
     uint32_t T, need;
     dev::select_threshold<kStepThreads>(sv, a.C, a.k, nz_tot, nullptr, unit_S ? unit_S : 0u,
                                         shist, sh, s2, T, need);
-    total = dev::mark_global<kStepThreads>(sv, a.C, T, need, smask, list, sh);
+    total = dev::mark_global<kStepThreads>(sv, a.C, T, need, smask, stie, list);
   } else if (a.inhibition == 1u) {
     __syncthreads();
     total = dev::mark_local<kStepThreads>(sv, 0u, a.C, a.gw, a.gh, a.radius, a.k, smask, list, sh);
@@ -789,7 +790,7 @@ cudaError_t launch_dense_overlap_many(const DenseArgs* args, uint32_t n, uint32_
 
 size_t frame_inhibit_smem(uint32_t C, uint32_t unit_S) {
   const uint32_t hist = unit_S + 1u > 256u ? unit_S + 1u : 256u;
-  return ((size_t)C + (C + 31u) / 32u + hist) * 4u;
+  return ((size_t)C + 2u * ((C + 31u) / 32u) + hist) * 4u;
 }
 
 size_t frame_inhibit_smem_limit() { return 226u * 1024u; }

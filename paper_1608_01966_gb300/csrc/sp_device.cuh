@@ -285,40 +285,102 @@ __device__ uint32_t mark_paper_literal(const uint32_t* sv, uint32_t C, uint32_t 
   return tot;
 }
 
-// Winner flags of global inhibition for all C columns, given (T, need):
-// sets bits of smask (zeroed by the caller) and, if list != nullptr, writes
-// the ascending winner list there.  Returns the number of winners.
+// The k-th largest of the counts in a histogram (hist[v] columns count v, v >=
+// 1; hist[0] is the largest count), by one warp: 32 bins a step from the
+// largest down.  T = 0 when at most k columns count (all of them win),
+// 0xffffffff when k is 0; else `need` of the columns at T win.
+__device__ __forceinline__ void warp_kth_count(const uint32_t* hist, uint32_t k, uint32_t& T,
+                                               uint32_t& need) {
+  const uint32_t lane = threadIdx.x & 31u;
+  T = 0xffffffffu;
+  need = 0u;
+  if (k == 0u) return;
+  T = 0u;
+  uint32_t acc = 0u;
+  for (uint32_t b0 = hist[0]; b0 >= 1u; b0 = b0 > 32u ? b0 - 32u : 0u) {
+    const uint32_t bin = b0 > lane ? b0 - lane : 0u;
+    const uint32_t h = bin ? hist[bin] : 0u;
+    uint32_t inc = h;
+#pragma unroll
+    for (uint32_t o = 1; o < 32u; o <<= 1) {
+      const uint32_t y = __shfl_up_sync(kFull, inc, o);
+      if (lane >= o) inc += y;
+    }
+    const uint32_t hit = __ballot_sync(kFull, acc + inc >= k);
+    if (hit) {
+      const int src = __ffs(hit) - 1;
+      T = b0 - (uint32_t)src;
+      need = k - (acc + __shfl_sync(kFull, inc - h, src));
+      return;
+    }
+    acc += __shfl_sync(kFull, inc, 31);
+  }
+}
+
+// Winner mask of global inhibition for all C columns, given (T, need): every
+// warp takes 32 columns a step (a ballot is a mask word); warp 0 then gives
+// the `need` lowest tied columns their bits, 32 words a step, and writes the
+// words to smask and, if list != nullptr, the ascending winner list.  stie
+// holds ceil(C / 32) words.  Returns the number of winners in warp 0's
+// threads.  Every thread of the block must call it; smask is visible to the
+// caller's other warps after its next barrier.
 template <int NTHREADS>
 __device__ uint32_t mark_global(const uint32_t* sv, uint32_t C, uint32_t T, uint32_t need,
-                                uint32_t* smask, uint32_t* list, uint32_t* sh) {
-  constexpr int NW = NTHREADS / 32;
-  const uint32_t t = threadIdx.x;
-  const uint32_t per = (C + NTHREADS - 1) / NTHREADS;  // contiguous chunks keep index order
-  const uint32_t lo = min(C, t * per), hi = min(C, lo + per);
-  uint32_t gt = 0, eq = 0;
-  for (uint32_t i = lo; i < hi; ++i) {
-    const uint32_t v = sv[i];
-    gt += v > T;
-    eq += (need != 0u) & (v == T);
-  }
-  uint32_t gt_ex, eq_ex, gt_tot, eq_tot;
-  block_scan2<NW>(gt, eq, gt_ex, eq_ex, gt_tot, eq_tot, sh);
-  uint32_t pos = gt_ex + min(eq_ex, need);
-  uint32_t e = eq_ex;
-  for (uint32_t i = lo; i < hi; ++i) {
-    const uint32_t v = sv[i];
-    bool w = v > T;
-    if (!w && need != 0u && v == T) {
-      w = e < need;
-      ++e;
-    }
-    if (w) {
-      if (list) list[pos] = i;
-      ++pos;
-      atomicOr(smask + (i >> 5), 1u << (i & 31u));
+                                uint32_t* smask, uint32_t* stie, uint32_t* list) {
+  constexpr uint32_t NW = NTHREADS / 32;
+  const uint32_t warp = threadIdx.x >> 5, lane = threadIdx.x & 31u;
+  const uint32_t words = (C + 31u) / 32u;
+  for (uint32_t w = warp; w < words; w += NW) {
+    const uint32_t i = 32u * w + lane, v = i < C ? sv[i] : 0u;
+    const uint32_t g = __ballot_sync(kFull, v > T);
+    const uint32_t e = __ballot_sync(kFull, i < C && v == T);
+    if (lane == 0u) {
+      smask[w] = g;
+      stie[w] = e;
     }
   }
-  return gt_tot + min(eq_tot, need);
+  group_sync<NTHREADS>();
+  if (warp != 0u) return 0u;
+  uint32_t seen = 0u, total = 0u;
+  for (uint32_t b = 0; b < words; b += 32u) {
+    const uint32_t w = b + lane;
+    uint32_t m = w < words ? smask[w] : 0u;
+    if (need != 0u) {
+      uint32_t e = w < words ? stie[w] : 0u;
+      const uint32_t ce = __popc(e);
+      uint32_t inc = ce;
+#pragma unroll
+      for (uint32_t o = 1; o < 32u; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(kFull, inc, o);
+        if (lane >= o) inc += y;
+      }
+      const uint32_t before = seen + inc - ce;
+      seen += __shfl_sync(kFull, inc, 31);
+      uint32_t take = need > before ? min(need - before, ce) : 0u;
+      if (take == ce) {
+        m |= e;
+      } else {
+        for (; take != 0u; --take) {  // the lowest tied columns
+          m |= e & (0u - e);
+          e &= e - 1u;
+        }
+      }
+      if (w < words) smask[w] = m;
+    }
+    const uint32_t c = __popc(m);
+    uint32_t inc = c;
+#pragma unroll
+    for (uint32_t o = 1; o < 32u; o <<= 1) {
+      const uint32_t y = __shfl_up_sync(kFull, inc, o);
+      if (lane >= o) inc += y;
+    }
+    if (list) {
+      uint32_t pos = total + inc - c;
+      for (uint32_t r = m; r != 0u; r &= r - 1u) list[pos++] = 32u * w + (uint32_t)(__ffs(r) - 1);
+    }
+    total += __shfl_sync(kFull, inc, 31);
+  }
+  return total;
 }
 
 // Does column c win its clipped (2r+1)^2 neighbourhood?  sv holds the fp32

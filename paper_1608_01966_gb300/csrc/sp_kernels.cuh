@@ -14,6 +14,10 @@ namespace sp {
 
 constexpr int kStepThreads = 128;  // 4 warps: one column per warp at a time
 constexpr int kStepWarps = kStepThreads / 32;
+// SPs of at most so many synapses per column: the last CTA counts the overlaps
+// of unit boosts into a histogram in its shared memory (up to 4 KB); of more,
+// every CTA adds its counts to one in global memory
+constexpr uint32_t kStepBins = 1022;
 
 // Everything one frame of one SP needs.  Passed by value.
 struct StepArgs {
@@ -31,7 +35,8 @@ struct StepArgs {
   uint32_t* counter;         // last-CTA ticket, 0 between launches
   uint32_t* hist;            // [S + 1] counts of surviving raw overlaps, 0 between
                              // launches; used (global inhibition) when every boost
-                             // is exactly 1, else nullptr (radix select instead)
+                             // is exactly 1 and S > kStepBins, else nullptr
+  uint32_t unit;             // every boost is exactly 1 (global inhibition)
   uint32_t* result_copy;     // optional second copy of result[0..n] (serving), or nullptr
   float* ov_copy;            // optional copy of this frame's boosted overlaps [C] (a
                              // caller's per-frame overlap record), or nullptr
@@ -69,7 +74,8 @@ struct BatchDesc {
   uint32_t *xsave0, *xsave1, *mask0, *mask1;
   uint32_t* result;
   uint32_t* counter;
-  uint32_t* hist;       // nullptr unless global inhibition with unit boosts
+  uint32_t* hist;       // as in StepArgs
+  uint32_t unit;
   float* duty;          // nullptr unless duty cycles are tracked
   float duty_period;
   const uint32_t* xspan;  // per CTA of this SP: [lo, hi) input words read (nullable)
@@ -143,13 +149,13 @@ struct BatchArgs {
   uint32_t* err;                // set to 1 if a bounded wait expired (nullable)
 };
 
-cudaError_t launch_batch_step(const BatchArgs& a, uint32_t n_ctas, uint32_t max_C,
+cudaError_t launch_batch_step(const BatchArgs& a, uint32_t n_ctas, uint32_t max_C, uint32_t max_S,
                               cudaStream_t stream);
 // One persistent launch over r.n_frames batch frames (grid sized to the
 // resident CTAs) with compiled schedule `schedule` (0: the default; out of
 // range: the default); r.work and r.abort must be 0.
-cudaError_t launch_batch_run(const BatchRunArgs& r, uint32_t max_C, uint32_t schedule,
-                             cudaStream_t stream);
+cudaError_t launch_batch_run(const BatchRunArgs& r, uint32_t max_C, uint32_t max_S,
+                             uint32_t schedule, cudaStream_t stream);
 // The compiled schedules of the persistent batch pass: how many, and the
 // resident CTAs per SM and columns per warp in flight of schedule i (false
 // when i is out of range).
@@ -242,12 +248,6 @@ struct SeqArgs {
   uint32_t* err;              // mapped host word, set to 1 if a bounded wait expired
 };
 
-size_t seq_smem_bytes(uint32_t form, uint32_t Q, uint32_t C, uint32_t S, uint32_t Cq,
-                      uint32_t band_max);
-cudaError_t seq_kernel_init(uint32_t form, size_t smem_bytes);
-cudaError_t seq_max_active_clusters(uint32_t form, uint32_t Q, size_t smem_bytes, int* out);
-cudaError_t launch_seq(const SeqArgs& a, uint32_t form, uint32_t Q, size_t smem_bytes,
-                       cudaStream_t stream);
 // What the plan of a sequence needs to know of the pools, per column: out[0][c]
 // and out[1][c] its smallest and largest input, out[2][c] the frame row of its
 // smallest, or 0xffffffff where a 64 x 64 bitmap cannot stand for the pool: it
@@ -255,6 +255,12 @@ cudaError_t launch_seq(const SeqArgs& a, uint32_t form, uint32_t Q, size_t smem_
 // a 64 x 64 box, or the frame is not a multiple of 32 pixels wide.
 cudaError_t launch_pool_scan(const uint32_t* idx, uint32_t C, uint32_t S, uint32_t W,
                              uint32_t* out, cudaStream_t stream);
+size_t seq_smem_bytes(uint32_t form, uint32_t Q, uint32_t C, uint32_t S, uint32_t Cq,
+                      uint32_t band_max);
+cudaError_t seq_kernel_init(uint32_t form, size_t smem_bytes);
+cudaError_t seq_max_active_clusters(uint32_t form, uint32_t Q, size_t smem_bytes, int* out);
+cudaError_t launch_seq(const SeqArgs& a, uint32_t form, uint32_t Q, size_t smem_bytes,
+                       cudaStream_t stream);
 
 // Dense pools on the tensor cores (sp_dense_tc.cu): the raw overlaps of a run
 // of frames without learning as one {0,1} matrix product.  Both operands are
@@ -320,8 +326,9 @@ cudaError_t launch_frame_inhibit_many(const FrameInhibitArgs* args, uint32_t n, 
 cudaError_t launch_duty_run(const uint32_t* masks, uint32_t n_frames, uint32_t mask_words,
                             uint32_t C, float* duty, float period, cudaStream_t stream);
 
-// Dynamic shared memory of the fused kernel for C columns.
-size_t step_smem_bytes(uint32_t C);
+// Dynamic shared memory of the fused kernel for C columns of S synapses (of a
+// launch of several SPs: the largest C and the largest S up to kStepBins).
+size_t step_smem_bytes(uint32_t C, uint32_t S);
 
 // Launch the fused step on `stream`.  Returns the launch error.
 cudaError_t launch_step(const StepArgs& a, int grid, cudaStream_t stream);

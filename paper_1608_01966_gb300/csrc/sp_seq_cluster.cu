@@ -213,7 +213,7 @@ struct SeqLayout {
     ov = part(2u * Cq);
     all = part(C);
     shist = part((S + 1u) > 256u ? (S + 1u) : 256u);
-    smask = part((C + 31u) / 32u);
+    smask = part(2u * ((C + 31u) / 32u));    // mask words, and tied columns
     o = o > unit_end ? o : unit_end;
     total = o;
   }
@@ -768,7 +768,7 @@ __global__ void __launch_bounds__(kSeqThreads + kSeqHelpers, 1) sp_seq_cluster_k
           dev::block_scan2<kSeqWarps>(nz, 0u, e0, e1, nz_tot, z, sh);
           dev::select_threshold<kSeqThreads>(s_all, C, a.k, nz_tot, nullptr, 0u, sm + L.shist, sh,
                                              s2, Tb, nd);
-          dev::mark_global<kSeqThreads>(s_all, C, Tb, nd, s_smask, nullptr, sh);
+          dev::mark_global<kSeqThreads>(s_all, C, Tb, nd, s_smask, s_smask + a.mask_words, nullptr);
         } else {
           compute_sync();
           dev::mark_local<kSeqThreads>(s_all, 0u, C, a.gw, a.gh, a.radius, a.k, s_smask, nullptr,

@@ -222,9 +222,11 @@ sp_status start_launch(sp_server* s, LaunchSlot& L, const LaunchSlot& other) {
   a.cta_inst = L.d_cta;
   a.tick = L.d_table;
   a.results_out = L.d_results;
-  uint32_t max_C = 1, stage = 0, win = 0;
+  uint32_t max_C = 1, max_S = 0, stage = 0, win = 0;
   for (auto& m : L.members) {
     max_C = std::max(max_C, s->streams[m.first].h->C);
+    if (s->streams[m.first].h->S <= sp::kStepBins)
+      max_S = std::max(max_S, s->streams[m.first].h->S);
     stage = std::max(stage, s->streams[m.first].stage_bytes);
     win = std::max(win, s->streams[m.first].win_bytes);
   }
@@ -232,7 +234,7 @@ sp_status start_launch(sp_server* s, LaunchSlot& L, const LaunchSlot& other) {
   a.xspan_cap = batch_xspan_cap();
   a.win_cap = win;
   a.err = L.d_err;
-  SP_CUDA(sp::launch_batch_step(a, ctas, max_C, L.st));
+  SP_CUDA(sp::launch_batch_step(a, ctas, max_C, max_S, L.st));
   SP_CUDA(cudaMemcpyAsync(L.h_results, L.d_results, (size_t)count * row * 4,
                           cudaMemcpyDeviceToHost, L.st));
   SP_CUDA(cudaEventRecord(L.done, L.st));

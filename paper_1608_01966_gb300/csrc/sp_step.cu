@@ -11,12 +11,11 @@
 //   phase 2 (last CTA)  Alg. 2 over all C overlaps held in shared memory:
 //                       global = find the k-th largest overlap, then ties at
 //                       that value go to the lowest indices through one
-//                       block scan.  With unit boosts the overlap is the raw
-//                       count itself, so phase 1 builds a histogram of the
-//                       surviving counts (global atomics) and the k-th value
-//                       is read off it in one scan; otherwise a radix select
-//                       runs four 8-bit passes over the fp32 bit patterns
-//                       (which order like the values, overlaps being >= 0).
+//                       scan.  Where the overlaps are counts (unit boosts) the
+//                       k-th value is read off their histogram; otherwise a
+//                       radix select runs four 8-bit passes over the fp32 bit
+//                       patterns (which order like the values, overlaps being
+//                       >= 0).
 //                       Local = rank count over the clipped (2r+1)^2 window.
 //                       Output: ascending winner list and winner bitmask.
 //
@@ -238,38 +237,92 @@ __device__ __forceinline__ uint32_t column_overlap(const StepArgs& a, uint32_t c
   return __reduce_add_sync(kFull, cnt);
 }
 
-// Alg. 2 over all overlaps, run by the last CTA.
-__device__ void last_cta_inhibit(const StepArgs& a, uint32_t* sv, uint32_t* smask) {
+// Alg. 2 over all overlaps, run by the last CTA.  This is the tail of every
+// frame's chain, so it makes one pass over the overlaps in L2 (kSelLoads of a
+// thread's loads in flight).  Where the overlaps are counts (unit boosts, or
+// found to be whole numbers up to S) they are counted into a histogram in
+// shared memory as they arrive, and every warp reads the k-th largest off it:
+// four barriers in all.  dyn: C overlaps, two sets of mask words, and S + 2
+// bins where S <= kStepBins.
+constexpr int kSelLoads = 8;
+
+__device__ void last_cta_inhibit(const StepArgs& a, uint32_t* dyn) {
   __shared__ uint32_t shist[256];
   __shared__ uint32_t sh[2 * kStepWarps];
   __shared__ uint32_t s2[2];
+  __shared__ uint32_t s_total;
   const uint32_t C = a.C;
   const uint32_t t = threadIdx.x;
-  uint32_t nz = 0;
-  for (uint32_t i = t; i < C; i += kStepThreads) {
-    const uint32_t v = __float_as_uint(__ldcg(a.ov + i));
-    sv[i] = v;
-    nz += v != 0u;
+  uint32_t* sv = dyn;
+  uint32_t* smask = sv + C;
+  uint32_t* stie = smask + a.mask_words;
+  uint32_t* bins = stie + a.mask_words;
+  const bool binned = a.inhibition == 0u && a.S <= kStepBins && !a.hist;
+  if (binned) {
+    for (uint32_t b = t; b <= a.S; b += kStepThreads) bins[b] = 0u;
+    __syncthreads();
   }
-  for (uint32_t i = t; i < a.mask_words; i += kStepThreads) smask[i] = 0u;
+  uint32_t nz = 0u, top = 0u;
+  bool whole = true;  // every overlap of this thread is a count of at most S
+  for (uint32_t i0 = t; i0 < C; i0 += kStepThreads * kSelLoads) {
+    uint32_t v[kSelLoads];
+#pragma unroll
+    for (int j = 0; j < kSelLoads; ++j) {
+      const uint32_t i = i0 + (uint32_t)j * kStepThreads;
+      v[j] = i < C ? __float_as_uint(__ldcg(a.ov + i)) : 0u;
+    }
+#pragma unroll
+    for (int j = 0; j < kSelLoads; ++j) {
+      const uint32_t i = i0 + (uint32_t)j * kStepThreads;
+      if (i < C) sv[i] = v[j];
+      if (v[j] != 0u) {
+        ++nz;
+        if (binned) {
+          const float f = __uint_as_float(v[j]);
+          const uint32_t n = f <= (float)a.S ? __float2uint_rz(f) : 0u;
+          if (n != 0u && __uint2float_rn(n) == f) {
+            atomicAdd(bins + n, 1u);
+            top = max(top, n);
+          } else {
+            whole = false;
+          }
+        }
+      }
+    }
+  }
   uint32_t total;
   if (a.inhibition == 0u) {
-    uint32_t e0, e1, nz_tot, z;
-    dev::block_scan2<kStepWarps>(nz, 0u, e0, e1, nz_tot, z, sh);  // also publishes sv
     uint32_t T, need;
-    dev::select_threshold<kStepThreads>(sv, C, a.k, nz_tot, a.hist, a.hist ? a.S : 0u, shist,
-                                        sh, s2, T, need);
-    total = dev::mark_global<kStepThreads>(sv, C, T, need, smask, a.result + 1, sh);
+    bool counts = false;
+    if (binned) {
+      top = __reduce_max_sync(kFull, top);
+      if ((t & 31u) == 0u && top) atomicMax(bins, top);
+      counts = a.unit ? (__syncthreads(), true) : __syncthreads_and(whole ? 1 : 0) != 0;
+    }
+    if (counts) {
+      dev::warp_kth_count(bins, a.k, T, need);
+      if (T != 0xffffffffu) T = __float_as_uint(__uint2float_rn(T));
+    } else {
+      uint32_t e0, e1, nz_tot, z;
+      dev::block_scan2<kStepWarps>(nz, 0u, e0, e1, nz_tot, z, sh);  // also publishes sv
+      dev::select_threshold<kStepThreads>(sv, C, a.k, nz_tot, a.hist, a.hist ? a.S : 0u, shist,
+                                          sh, s2, T, need);
+    }
+    total = dev::mark_global<kStepThreads>(sv, C, T, need, smask, stie, a.result + 1);
+    if (t == 0u) s_total = total;
   } else if (a.inhibition == 1u) {
+    for (uint32_t i = t; i < a.mask_words; i += kStepThreads) smask[i] = 0u;
     __syncthreads();
     total = dev::mark_local<kStepThreads>(sv, 0u, C, a.gw, a.gh, a.radius, a.k, smask,
                                           a.result + 1, sh);
   } else {
+    for (uint32_t i = t; i < a.mask_words; i += kStepThreads) smask[i] = 0u;
     __syncthreads();
     total = dev::mark_paper_literal<kStepThreads>(sv, C, a.k, smask, a.result + 1, shist, sh,
                                                   s2);
   }
   __syncthreads();
+  if (a.inhibition == 0u) total = s_total;
   if (t == 0u) a.result[0] = total;
   if (a.learn_next) {
     // the SP's next frame learns these winners first thing: ask L2 for their
@@ -360,12 +413,13 @@ __host__ __device__ __forceinline__ uint32_t stage_ring_bytes(uint32_t S) {
 }
 
 // Alg. 1's tail for column c with raw count `raw` (one lane): the boosted
-// overlap to the SP's overlaps (and the caller's record), and, with unit
-// boosts, the count into the histogram the last CTA selects from.
+// overlap to the SP's overlaps (and the caller's record), and, for SPs of more
+// than kStepBins synapses with unit boosts, the count into the histogram the
+// last CTA selects from (it counts smaller ones itself).
 __device__ __forceinline__ void publish_overlap(const StepArgs& a, uint32_t c, uint32_t raw) {
-  // a histogram is kept only when every boost is exactly 1, and then the
-  // product is the count itself: no load stalls the warp here
-  const float v = dev::boosted(raw, a.min_overlap, a.hist ? 1.0f : __ldg(a.boost + c));
+  // where every boost is exactly 1 the product is the count itself: no load
+  // stalls the warp here
+  const float v = dev::boosted(raw, a.min_overlap, a.unit ? 1.0f : __ldg(a.boost + c));
   a.ov[c] = v;
   if (a.ov_copy) a.ov_copy[c] = v;
   if (a.hist && raw >= a.min_overlap && raw != 0u) atomicAdd(a.hist + raw, 1u);
@@ -878,7 +932,7 @@ __device__ __forceinline__ void step_body(const StepArgs& a, uint32_t bid, uint3
   __syncthreads();
   if (s_ticket != nb - 1u) return;
   __threadfence();
-  last_cta_inhibit(a, dyn_smem, dyn_smem + a.C);
+  last_cta_inhibit(a, dyn_smem);
   if (threadIdx.x == 0) atomicExch(a.counter, 0u);
   if (done) {
     // release this frame's results (mask, list, reset counter and
@@ -945,6 +999,7 @@ __global__ void __launch_bounds__(kStepThreads, SP_BATCH_MIN_BLOCKS) sp_batch_st
     a.x_prev = !pending ? nullptr
                : (ba.prev_frames ? ba.prev_frames + d.frame_off : (cur ? d.xsave0 : d.xsave1));
   }
+  a.unit = d.unit;
   a.mask_prev = pending ? (cur ? d.mask0 : d.mask1) : nullptr;
   a.x_save = (learn && save) ? (cur ? d.xsave1 : d.xsave0) : nullptr;
   a.mask_out = cur ? d.mask1 : d.mask0;
@@ -999,7 +1054,10 @@ __global__ void __launch_bounds__(kStepThreads) sp_learn_kernel(const LearnArgs 
 
 }  // namespace
 
-size_t step_smem_bytes(uint32_t C) { return ((size_t)C + (C + 31u) / 32u) * sizeof(uint32_t); }
+size_t step_smem_bytes(uint32_t C, uint32_t S) {
+  const uint32_t bins = S <= kStepBins ? S + 2u : 0u;
+  return ((size_t)C + 2u * ((C + 31u) / 32u) + bins) * sizeof(uint32_t);
+}
 
 int step_grid(uint32_t C) { return (int)((C + kStepWarps - 1) / kStepWarps); }
 
@@ -1069,6 +1127,7 @@ __global__ void __launch_bounds__(kStepThreads, MINB) sp_batch_run_kernel(const 
     }
     StepArgs a;
     a.learn_next = r.learn;
+    a.unit = d.unit;
     const uint32_t cur = r.cur0 ^ (t & 1u);
     const uint32_t pending = t > 0u ? r.learn : r.pending0;
     const uint32_t save = t + 1u == r.n_frames ? 1u : 0u;
@@ -1152,7 +1211,7 @@ bool batch_schedule(uint32_t i, uint32_t* ctas_per_sm, uint32_t* cols_in_flight)
 }
 
 cudaError_t kernels_init() {
-  const int bytes = (int)step_smem_bytes(SP_MAX_COLUMNS);
+  const int bytes = (int)step_smem_bytes(SP_MAX_COLUMNS, kStepBins);
   cudaError_t e = cudaFuncSetAttribute(sp_step_kernel<4>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
   if (e != cudaSuccess) return e;
@@ -1331,10 +1390,10 @@ cudaError_t launch_xspan(const uint32_t* idx, uint32_t C, uint32_t S, uint32_t n
   return cudaGetLastError();
 }
 
-cudaError_t launch_batch_run(const BatchRunArgs& r, uint32_t max_C, uint32_t schedule,
-                             cudaStream_t stream) {
+cudaError_t launch_batch_run(const BatchRunArgs& r, uint32_t max_C, uint32_t max_S,
+                             uint32_t schedule, cudaStream_t stream) {
   const RunSchedule& rs = kRunSchedules[schedule < kNumRunSchedules ? schedule : 0u];
-  const size_t smem = std::max<size_t>(step_smem_bytes(max_C),
+  const size_t smem = std::max<size_t>(step_smem_bytes(max_C, max_S),
                                        std::max(std::max(r.stage_cap, r.xspan_cap), r.win_cap));
   int dev = 0, sms = 0, per_sm = 0;
   cudaError_t e = cudaGetDevice(&dev);
@@ -1357,9 +1416,9 @@ uint32_t batch_stage_bytes(uint32_t C, uint32_t S, uint32_t n_ctas) {
   return kStepWarps * stage_ring_bytes(S);
 }
 
-cudaError_t launch_batch_step(const BatchArgs& a, uint32_t n_ctas, uint32_t max_C,
+cudaError_t launch_batch_step(const BatchArgs& a, uint32_t n_ctas, uint32_t max_C, uint32_t max_S,
                               cudaStream_t stream) {
-  const size_t smem = std::max<size_t>(step_smem_bytes(max_C),
+  const size_t smem = std::max<size_t>(step_smem_bytes(max_C, max_S),
                                        std::max(std::max(a.stage_cap, a.xspan_cap), a.win_cap));
   static const bool pdl = [] {
     const char* e = std::getenv("SP_DISABLE_PDL");
@@ -1381,7 +1440,7 @@ cudaError_t launch_batch_step(const BatchArgs& a, uint32_t n_ctas, uint32_t max_
 }
 
 cudaError_t launch_step(const StepArgs& a, int grid, cudaStream_t stream) {
-  const size_t smem = step_smem_bytes(a.C);
+  const size_t smem = step_smem_bytes(a.C, a.S);
   if (a.S % 4u == 0u)
     sp_step_kernel<4><<<grid, kStepThreads, smem, stream>>>(a);
   else
