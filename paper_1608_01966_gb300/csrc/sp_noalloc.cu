@@ -17,6 +17,8 @@
 // holds it until the process exits) and is shared by every call.
 #include <cuda_runtime.h>
 
+#include <atomic>
+
 #include "../../include/sp.h"
 #include "sp_internal.h"
 #include "sp_kernels.cuh"
@@ -24,9 +26,15 @@
 namespace {
 
 // [0, SP_NOALLOC_MAX_COLUMNS): boosted overlaps of the current call;
-// [SP_NOALLOC_MAX_COLUMNS]: the last-CTA ticket counter (cleared every call).
+// [SP_NOALLOC_MAX_COLUMNS .. + 1]: two last-CTA ticket counters, used by calls
+// in turn.  A call leaves its own at zero and its kernel clears the other one
+// first, so that a counter left wrong by calls that raced does not last; with
+// one counter, clearing it took a memset node of 1.5 us before every kernel.
 constexpr uint32_t kScratchWords = SP_NOALLOC_MAX_COLUMNS + 64u;
 static __device__ __align__(256) uint32_t g_noalloc_scratch[kScratchWords];
+std::atomic<uint32_t> g_turn{0};
+
+constexpr size_t kPlainSmem = 44u << 10;  // less the step kernel's static shared memory
 
 sp_status noalloc_fail(sp_status s, const char* msg) {
   sp::set_last_error("sp_step_noalloc: %s", msg);
@@ -39,8 +47,10 @@ sp_status noalloc_fail(sp_status s, const char* msg) {
 // up on every call (a lookup, no allocation): a context that was destroyed
 // and created again -- a device reset between calls -- loads the library's
 // device code again, possibly at another address, so a remembered address
-// could be stale.  The kernels' attributes are set again for the same reason.
-sp_status scratch_address(uint32_t** out) {
+// could be stale.  The kernels' attributes are set again for the same reason,
+// where the launch needs them: kernels take up to 48 KB of shared memory
+// without (setting all of them costs 5 us of host time a call).
+sp_status scratch_address(uint32_t** out, size_t smem) {
   void* p = nullptr;
   const cudaError_t e = cudaGetSymbolAddress(&p, g_noalloc_scratch);
   if (e != cudaSuccess || !p) {
@@ -48,7 +58,7 @@ sp_status scratch_address(uint32_t** out) {
                        cudaGetErrorString(e));
     return SP_ECUDA;
   }
-  if (sp::kernels_init() != cudaSuccess)
+  if (smem > kPlainSmem && sp::kernels_init() != cudaSuccess)
     return noalloc_fail(SP_ECUDA, "kernel attribute set-up failed");
   *out = static_cast<uint32_t*>(p);
   return SP_OK;
@@ -78,13 +88,11 @@ SP_API sp_status sp_step_noalloc(const sp_config* cfg, const uint32_t* d_idx, fl
     return noalloc_fail(SP_EINVAL, "device pointers misaligned (16 bytes for idx/perm when S % 4 == 0)");
 
   uint32_t* scratch = nullptr;
-  sp_status s = scratch_address(&scratch);
+  sp_status s = scratch_address(&scratch, sp::step_smem_bytes(C, S));
   if (s != SP_OK) return s;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  uint32_t* counter = scratch + SP_NOALLOC_MAX_COLUMNS;
-  // the ticket counter must start at zero; the overlaps are fully rewritten
-  if (cudaMemsetAsync(counter, 0, sizeof(uint32_t), st) != cudaSuccess)
-    return noalloc_fail(SP_ECUDA, "clearing the scratch counter failed");
+  const uint32_t turn = g_turn.fetch_add(1, std::memory_order_relaxed) & 1u;
+  uint32_t* counter = scratch + SP_NOALLOC_MAX_COLUMNS + turn;
 
   sp::StepArgs a{};
   a.idx = d_idx;
@@ -95,6 +103,7 @@ SP_API sp_status sp_step_noalloc(const sp_config* cfg, const uint32_t* d_idx, fl
   a.mask_out = d_active_mask;
   a.result = d_active_list;
   a.counter = counter;
+  a.counter_clear = scratch + SP_NOALLOC_MAX_COLUMNS + (turn ^ 1u);
   a.C = C;
   a.S = S;
   a.n_words = (uint32_t)((n_in + 31) / 32);

@@ -948,6 +948,7 @@ __device__ __forceinline__ void step_body(const StepArgs& a, uint32_t bid, uint3
 template <int VEC>
 __global__ void __launch_bounds__(kStepThreads) sp_step_kernel(const StepArgs a) {
   extern __shared__ __align__(128) uint32_t dyn_smem[];
+  if (a.counter_clear && blockIdx.x == 0u && threadIdx.x == 0u) *a.counter_clear = 0u;
   step_body<VEC, false>(a, blockIdx.x, gridDim.x, dyn_smem);
 }
 
