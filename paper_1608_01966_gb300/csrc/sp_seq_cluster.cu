@@ -264,15 +264,17 @@ __global__ void __launch_bounds__(kSeqThreads + kSeqHelpers, 1) sp_seq_cluster_k
   // Column ownership of the count.  A warp counts P columns side by side,
   // L32 = 32 / P lanes each (pools of a few synapses); its i-th own column is
   //   lc = ((i / P) * kSeqWarps + warp) * P + i % P,   i < own.
-  uint32_t P = 1u;
+  uint32_t lp = 0u;  // log2 P
   if (!kWindow) {
     const uint32_t units = (S & 3u) == 0u ? S >> 2 : S;  // lane loads of one pool
-    while (P < 8u && units * P * 2u <= 32u && kSeqWarps * P * 2u <= Cq) P <<= 1;
+    while (lp < 3u && (units << (lp + 1u)) <= 32u && (kSeqWarps << (lp + 1u)) <= Cq) ++lp;
   }
-  const uint32_t L32 = 32u / P;
-  const uint32_t passes = (Cq + kSeqWarps * P - 1u) / (kSeqWarps * P);
-  const uint32_t own = passes * P;  // at most 32 (Cq <= kSeqThreads)
-  auto own_col = [&](uint32_t i) { return ((i / P) * kSeqWarps + warp) * P + i % P; };
+  const uint32_t P = 1u << lp, ll = 5u - lp, L32 = 1u << ll;
+  const uint32_t passes = (Cq + (kSeqWarps << lp) - 1u) / (kSeqWarps << lp);
+  const uint32_t own = passes << lp;  // at most 32 (Cq <= kSeqThreads)
+  auto own_col = [&](uint32_t i) {
+    return (((i >> lp) * kSeqWarps + warp) << lp) + (i & (P - 1u));
+  };
 
   // ---- prologue: barriers, this CTA's state and input band -------------------
   if (t == 0) {
@@ -308,13 +310,12 @@ __global__ void __launch_bounds__(kSeqThreads + kSeqHelpers, 1) sp_seq_cluster_k
     }
   }
   __syncthreads();
-  // exact quotient by the frame width from a float estimate
-  const float inv_w = kWindow ? 1.0f / (float)a.win_w : 0.0f;
+  // exact quotient by the frame width: with m = ceil(2^32 / W) the estimate
+  // floor(id m / 2^32) is the quotient or one more (id < 2^32, m W - 2^32 < W)
+  const uint32_t inv_w = kWindow ? 0xffffffffu / a.win_w + 1u : 0u;
   auto row_of = [&](uint32_t id) {
-    uint32_t r = __float2uint_rz(__uint2float_rz(id) * inv_w);
-    while (r * a.win_w > id) --r;
-    while ((r + 1u) * a.win_w <= id) ++r;
-    return r;
+    const uint32_t r = __umulhi(id, inv_w);
+    return r * a.win_w > id ? r - 1u : r;
   };
   // boxes of the columns, and the smallest and largest value that the CTA's
   // band must cover (input indices; window forms: box rows)
@@ -477,13 +478,32 @@ __global__ void __launch_bounds__(kSeqThreads + kSeqHelpers, 1) sp_seq_cluster_k
         shf[j] = at & 31u;
       }
     }
-    for (; f < a.n_frames; ++f) {
+    // what does not change from frame to frame: the CTA this warp sends to, and
+    // in local inhibition the lane's column and its clipped window
+    uint32_t peer_cnt = 0u, peer_bar = 0u;
+    if (Q > 1u && warp < Q) {
+      peer_cnt = peer_addr(smem_u32(reinterpret_cast<uint16_t*>(sm + L.cnt) + c0), warp);
+      peer_bar = peer_addr(smem_u32(&s_cnt_bar[0]), warp);
+    }
+    uint32_t lg = 5u;  // log2 of the lanes that share a column
+    for (uint32_t n_own = 1u; n_own < own; n_own <<= 1) --lg;
+    const uint32_t loc_i = lane >> lg, loc_g = lane & ((1u << lg) - 1u), loc_lc = own_col(loc_i);
+    const bool loc_ok = !global && loc_i < own && loc_lc < nc;
+    uint32_t loc_x = 0u, loc_y = 0u;
+    if (loc_ok) {
+      loc_y = (c0 + loc_lc) / a.gw;
+      loc_x = c0 + loc_lc - loc_y * a.gw;
+    }
+    const uint32_t parts2 = (S + 63u) / 64u;
+    const float inv_parts2 = 1.0f / (float)parts2;
+    uint32_t slot = 0u;  // f % 3
+    for (; f < a.n_frames; ++f, slot = slot == 2u ? 0u : slot + 1u) {
       const uint32_t par = f & 1u, phase = (f >> 1) & 1u;
       const uint32_t* band = s_band + par * a.band_max;
       uint32_t* s_cnt32 = sm + L.cnt + par * cnt_words;
       uint16_t* s_cnt = reinterpret_cast<uint16_t*>(s_cnt32);  // [Q * Cq], column order
-      uint32_t* hist = sm + L.hist + (f % 3u) * hw;
-      uint32_t* smask_f = sm + L.mask + (f % 3u) * mw;
+      uint32_t* hist = sm + L.hist + slot * hw;
+      uint32_t* smask_f = sm + L.mask + slot * mw;
       float* ov_pub = reinterpret_cast<float*>(sm + L.ov) + par * Cq;
       if (ok) ok = mbar_wait<false>(&s_band_bar[par], phase);
 
@@ -542,11 +562,11 @@ __global__ void __launch_bounds__(kSeqThreads + kSeqHelpers, 1) sp_seq_cluster_k
       auto count_pools = [&](uint32_t p0, auto u) {
         constexpr int U = decltype(u)::value;
         uint32_t n[U], row[U];
-        const uint32_t sub = lane / L32, sl = lane % L32;
+        const uint32_t sub = lane >> ll, sl = lane & (L32 - 1u);
 #pragma unroll
         for (int j = 0; j < U; ++j) {
           n[j] = 0u;
-          row[j] = min(((p0 + j) * kSeqWarps + warp) * P + sub, nc - 1u) * S;
+          row[j] = min((((p0 + j) * kSeqWarps + warp) << lp) + sub, nc - 1u) * S;
         }
         auto bit = [&](uint32_t w, uint32_t id, float p) {
           return p >= a.thr ? (w >> (id & 31u)) & 1u : 0u;
@@ -602,7 +622,7 @@ __global__ void __launch_bounds__(kSeqThreads + kSeqHelpers, 1) sp_seq_cluster_k
           uint32_t mine = n[0];
 #pragma unroll
           for (int j = 1; j < U; ++j) mine = sl == (uint32_t)j ? n[j] : mine;
-          const uint32_t lc = ((p0 + sl) * kSeqWarps + warp) * P + sub;
+          const uint32_t lc = (((p0 + sl) * kSeqWarps + warp) << lp) + sub;
           if (sl < (uint32_t)U && lc < nc) publish(lc, mine);
         }
       };
@@ -629,8 +649,7 @@ __global__ void __launch_bounds__(kSeqThreads + kSeqHelpers, 1) sp_seq_cluster_k
         // ---- all counts to every CTA --------------------------------------------
         if (Q > 1u) {
           if (warp < Q && warp != q) {
-            const uint32_t dst = peer_addr(smem_u32(s_cnt + c0), warp);
-            const uint32_t bar = peer_addr(smem_u32(&s_cnt_bar[par]), warp);
+            const uint32_t dst = peer_cnt + par * cnt_words * 4u, bar = peer_bar + par * 8u;
             for (uint32_t u = lane; u < Cq / 8u; u += 32u)
               send16(dst + u * 16u, reinterpret_cast<const uint4*>(s_cnt + c0)[u], bar);
           }
@@ -706,14 +725,11 @@ __global__ void __launch_bounds__(kSeqThreads + kSeqHelpers, 1) sp_seq_cluster_k
           // row of its clipped (2r + 1)^2 neighbourhood.  A neighbour beats it
           // with a higher count, or with an equal one and a lower index: rows
           // above and columns to the left win ties
-          uint32_t n_own = 1u;
-          while (n_own < own) n_own <<= 1;
-          const uint32_t G = 32u / n_own, i = lane / G, g = lane % G;
-          const uint32_t lc = own_col(i), c = c0 + lc;
-          const uint32_t v = i < own && lc < nc ? s_cnt[c] : 0u;
+          const uint32_t lc = loc_lc, c = c0 + lc, G = 1u << lg, g = loc_g;
+          const uint32_t v = loc_ok ? s_cnt[c] : 0u;
           uint32_t beaten = 0u;
           if (v != 0u && a.k != 0u) {
-            const uint32_t x = c % a.gw, y = c / a.gw, r = a.radius;
+            const uint32_t x = loc_x, y = loc_y, r = a.radius;
             const uint32_t x0 = x >= r ? x - r : 0u, x1 = min(a.gw - 1u, x + r);
             const uint32_t y0 = y >= r ? y - r : 0u, y1 = min(a.gh - 1u, y + r);
             // two columns a word: (count | 0x8000) - limit keeps its top bit
@@ -800,11 +816,13 @@ __global__ void __launch_bounds__(kSeqThreads + kSeqHelpers, 1) sp_seq_cluster_k
       // units dealt to the warps; a unit's loads are issued before the first is
       // used.  Few winners: small units, so that their chains are short
       const uint32_t n_win = s_n;
-      auto learn = [&](auto jc) {
+      auto learn = [&](auto jc, uint32_t parts, float inv_parts) {
         constexpr int J = decltype(jc)::value;
-        const uint32_t parts = (S + 32u * J - 1u) / (32u * J), units = n_win * parts;
+        const uint32_t units = n_win * parts;
         for (uint32_t u = warp; u < units; u += kSeqWarps) {
-          const uint32_t i = u / parts, s0 = (u - i * parts) * 32u * J + lane;
+          // u / parts: both below 2^16, half a unit from the next quotient
+          const uint32_t i = __float2uint_rz(((float)u + 0.5f) * inv_parts);
+          const uint32_t s0 = (u - i * parts) * 32u * J + lane;
           const uint32_t lc = s_list[i];
           uint32_t* wb = s_bits + lc * kBoxWords;
           uint32_t at = 0u, org = 0u;
@@ -850,10 +868,13 @@ __global__ void __launch_bounds__(kSeqThreads + kSeqHelpers, 1) sp_seq_cluster_k
           if (kPermSmem && lane == 0u && s0 == 0u) atomicOr(s_dirty + (lc >> 5), 1u << (lc & 31u));
         }
       };
-      if (S <= 64u || n_win * S <= 2048u)
-        learn(IntC<2>{});
-      else
-        learn(IntC<kPermSmem ? 8 : 4>{});  // the box positions of 8 would spill
+      if (parts2 == 1u || n_win * S <= 2048u) {
+        learn(IntC<2>{}, parts2, inv_parts2);
+      } else {
+        constexpr int J = kPermSmem ? 8 : 4;  // the box positions of 8 would spill
+        const uint32_t parts = (S + 32u * J - 1u) / (32u * J);
+        learn(IntC<J>{}, parts, 1.0f / (float)parts);
+      }
       compute_sync();  // the next count reads what other warps learnt
       if (t == 0u) s_n = 0u;
       if (reg_bits && nc) {
