@@ -128,6 +128,17 @@ struct TickMember {
   uint32_t out_off;    // words: its [count, list...] in results_out
   uint32_t pad;
 };
+// One member of a serving launch as the host lists it (pinned memory, read by
+// the device): its TickMember, its CTAs, and where its frame waits on the host
+// (nullptr: it is on the device already).
+struct TickItem {
+  TickMember tm;
+  const uint32_t* src;  // pinned; copied to tm.x
+  uint32_t words;
+  uint32_t stream;      // index of tm in the launch's table
+  uint32_t n_ctas;
+  uint32_t pad;
+};
 enum : uint32_t { kTickCur = 1u, kTickPending = 2u, kTickLearn = 4u, kTickSave = 8u };
 
 // One frame for every SP of a batch.  All members share the buffer parity
@@ -150,6 +161,10 @@ struct BatchArgs {
   uint32_t* err;                // set to 1 if a bounded wait expired (nullable)
 };
 
+// Prepare a serving launch on the device from its `count` pinned items: copy
+// the frames in, fill table[stream] and the CTA map.
+cudaError_t launch_tick_gather(const TickItem* items, uint32_t count, TickMember* table,
+                               uint32_t* cta_inst, cudaStream_t stream);
 cudaError_t launch_batch_step(const BatchArgs& a, uint32_t n_ctas, uint32_t max_C, uint32_t max_S,
                               cudaStream_t stream);
 // One persistent launch over r.n_frames batch frames (grid sized to the

@@ -1,15 +1,15 @@
 // Serving many streams with continuous batching (include/sp.h, sp_server_*).
 //
 // Client threads submit frames: each frame is copied into its stream's pinned
-// ring slot and its host-to-device copy is enqueued at once on the server's
-// copy stream.  One worker thread forms launches: every open stream with a
+// ring slot.  One worker thread forms launches: every open stream with a
 // frame waiting and none in flight joins the next launch, which steps that
 // subset of SPs with the batch kernel (a per-launch member table gives each
-// SP its frame, buffer parity, pending-learning flag and CTA range).  Two
-// launch slots, each with its own CUDA stream, let a new launch start while
-// the previous one runs.  Results (count + ascending list per SP) come back
-// into pinned memory; the worker records each request's latency and hands
-// the results to sp_server_poll.
+// SP its frame, buffer parity, pending-learning flag and CTA range).  A launch
+// is two kernels and no copies: the first reads the members' items and frames
+// from pinned memory, the second steps them and writes the results (count +
+// ascending list per SP) to pinned memory.  Two launch slots, each with its own
+// CUDA stream, let a new launch start while the previous one runs; the worker
+// records each request's latency and hands the results to sp_server_poll.
 #include <algorithm>
 #include <atomic>
 #include <chrono>
@@ -30,6 +30,7 @@ namespace {
 
 constexpr int kLaunchSlots = 2;
 constexpr uint32_t kServeColsPerWarp = 4;
+constexpr auto kSpin = std::chrono::microseconds(100);  // a sleep and wake-up cost tens
 constexpr uint32_t kMaxServerStreams = 4096;
 
 struct Request {
@@ -71,15 +72,12 @@ struct LaunchSlot {
   bool busy = false;
   cudaStream_t st = nullptr;
   cudaEvent_t done = nullptr;
-  sp::TickMember* h_table = nullptr;  // pinned [max_streams]
-  uint32_t* h_cta = nullptr;          // pinned [max_ctas]
-  uint32_t* h_results = nullptr;      // pinned [max_streams][1 + max_active]
-  sp::TickMember* d_table = nullptr;
-  uint32_t* d_cta = nullptr;
-  uint32_t* d_results = nullptr;
+  sp::TickItem* h_items = nullptr;    // pinned [max_streams], read by the device
+  uint32_t* h_results = nullptr;      // pinned [max_streams][1 + max_active], written by the device
+  sp::TickMember* d_table = nullptr;  // [max_streams]
+  uint32_t* d_cta = nullptr;          // [max_ctas]
   uint32_t* h_err = nullptr;          // mapped host word: a bounded wait expired
   uint32_t* d_err = nullptr;
-  cudaEvent_t copies = nullptr;       // host frame copies issued before this launch
   uint64_t launch_no = 0;             // order of the launches (results are delivered in it)
   std::vector<std::pair<uint32_t, Request>> members;  // (slot, request)
 };
@@ -93,6 +91,9 @@ struct sp_server {
   std::condition_variable cv_work, cv_done;
   std::thread worker;
   std::atomic<bool> stop{false};
+  // requests published and results delivered so far: what the worker and a
+  // waiting poll watch for a moment before they sleep
+  std::atomic<uint64_t> published{0}, delivered{0};
   std::vector<Stream> streams;
   sp::BatchDesc* d_desc = nullptr;
   cudaStream_t copy_stream = nullptr;
@@ -107,6 +108,13 @@ struct sp_server {
 };
 
 namespace {
+
+// Yield until `counter` leaves `seen` or kSpin has passed.
+void spin_while(const std::atomic<uint64_t>& counter, uint64_t seen) {
+  const auto end = Clock::now() + kSpin;
+  while (counter.load(std::memory_order_acquire) == seen && Clock::now() < end)
+    std::this_thread::yield();
+}
 
 uint64_t estimate_bytes(const sp_config* c, uint32_t depth, uint32_t words) {
   const uint64_t C = c->num_columns, S = c->synapses_per_column;
@@ -146,13 +154,14 @@ void finish_launch(sp_server* s, LaunchSlot& L, sp_status st) {
   }
   L.members.clear();
   L.busy = false;
+  s->delivered.fetch_add(pos, std::memory_order_release);
 }
 
 // Form and enqueue one launch from the waiting streams (caller holds mu).  A
 // stream whose previous frame is still in the other slot's launch may take
 // part: this launch then waits on the GPU for that one.
 sp_status start_launch(sp_server* s, LaunchSlot& L, const LaunchSlot& other) {
-  bool chained = false, host_copies = false;
+  bool chained = false;
   const uint32_t n = (uint32_t)s->streams.size();
   const uint32_t row = 1u + s->cfg.max_active;
   uint32_t ctas = 0, count = 0;
@@ -174,6 +183,7 @@ sp_status start_launch(sp_server* s, LaunchSlot& L, const LaunchSlot& other) {
       S.launch_seq += 1;
       S.outstanding -= 1;
       ++s->completed;
+      s->delivered.fetch_add(1, std::memory_order_release);
     }
     // requests launch in sequence order; one still being copied holds back
     // the ones after it
@@ -183,13 +193,16 @@ sp_status start_launch(sp_server* s, LaunchSlot& L, const LaunchSlot& other) {
     Request r = S.queue.front();
     S.queue.pop_front();
     S.launch_seq += 1;
-    sp::TickMember& tm = L.h_table[i];
-    tm.x = S.d_ring + (size_t)r.ring * S.input_words;
-    tm.flags = (S.cur ? sp::kTickCur : 0u) | (S.pending ? sp::kTickPending : 0u) |
-               (r.learn ? sp::kTickLearn : 0u) | sp::kTickSave;
-    tm.cta_first = ctas;
-    tm.out_off = count * row;
-    for (uint32_t c = 0; c < S.n_ctas; ++c) L.h_cta[ctas + c] = i;
+    sp::TickItem& it = L.h_items[count];
+    it.tm.x = S.d_ring + (size_t)r.ring * S.input_words;
+    it.tm.flags = (S.cur ? sp::kTickCur : 0u) | (S.pending ? sp::kTickPending : 0u) |
+                  (r.learn ? sp::kTickLearn : 0u) | sp::kTickSave;
+    it.tm.cta_first = ctas;
+    it.tm.out_off = count * row;
+    it.src = r.device ? nullptr : S.h_ring + (size_t)r.ring * S.input_words;
+    it.words = S.input_words;
+    it.stream = i;
+    it.n_ctas = S.n_ctas;
     ctas += S.n_ctas;
     chained = chained || S.in_flight > 0u;
     S.in_flight += 1;
@@ -198,30 +211,18 @@ sp_status start_launch(sp_server* s, LaunchSlot& L, const LaunchSlot& other) {
     S.cur ^= 1;
     L.members.emplace_back(i, r);
     ++count;
-    // the launch waits for this frame's copy: frames copied on a caller's
-    // stream one by one, host frames all at once below
-    if (r.device)
-      SP_CUDA(cudaStreamWaitEvent(L.st, S.ev_h2d[r.ring], 0));
-    else
-      host_copies = true;
+    // a frame copied on a caller's stream: the launch waits for that copy
+    if (r.device) SP_CUDA(cudaStreamWaitEvent(L.st, S.ev_h2d[r.ring], 0));
   }
   if (count == 0) return SP_OK;
-  if (host_copies) {
-    // every published host frame's copy was issued on the copy stream before
-    // its request was published
-    SP_CUDA(cudaEventRecord(L.copies, s->copy_stream));
-    SP_CUDA(cudaStreamWaitEvent(L.st, L.copies, 0));
-  }
   if (chained) SP_CUDA(cudaStreamWaitEvent(L.st, other.done, 0));
   s->rr = (s->rr + 1) % n;
-  SP_CUDA(cudaMemcpyAsync(L.d_table, L.h_table, sizeof(sp::TickMember) * n,
-                          cudaMemcpyHostToDevice, L.st));
-  SP_CUDA(cudaMemcpyAsync(L.d_cta, L.h_cta, (size_t)ctas * 4, cudaMemcpyHostToDevice, L.st));
+  SP_CUDA(sp::launch_tick_gather(L.h_items, count, L.d_table, L.d_cta, L.st));
   sp::BatchArgs a{};
   a.desc = s->d_desc;
   a.cta_inst = L.d_cta;
   a.tick = L.d_table;
-  a.results_out = L.d_results;
+  a.results_out = L.h_results;
   uint32_t max_C = 1, max_S = 0, stage = 0, win = 0;
   for (auto& m : L.members) {
     max_C = std::max(max_C, s->streams[m.first].h->C);
@@ -235,8 +236,6 @@ sp_status start_launch(sp_server* s, LaunchSlot& L, const LaunchSlot& other) {
   a.win_cap = win;
   a.err = L.d_err;
   SP_CUDA(sp::launch_batch_step(a, ctas, max_C, max_S, L.st));
-  SP_CUDA(cudaMemcpyAsync(L.h_results, L.d_results, (size_t)count * row * 4,
-                          cudaMemcpyDeviceToHost, L.st));
   SP_CUDA(cudaEventRecord(L.done, L.st));
   L.busy = true;
   L.launch_no = ++s->launches;
@@ -295,7 +294,12 @@ void worker_main(sp_server* s) {
       lk.lock();
     } else {
       idle_spins = 0;
-      s->cv_work.wait_for(lk, std::chrono::milliseconds(5));
+      const uint64_t seen = s->published.load(std::memory_order_acquire);
+      lk.unlock();
+      spin_while(s->published, seen);
+      lk.lock();
+      if (s->published.load(std::memory_order_acquire) == seen)
+        s->cv_work.wait_for(lk, std::chrono::milliseconds(5));
     }
   }
 }
@@ -325,14 +329,11 @@ void free_server(sp_server* s) {
     if (L.st) cudaStreamSynchronize(L.st);
     if (L.done) cudaEventDestroy(L.done);
     if (L.st) cudaStreamDestroy(L.st);
-    if (L.h_table) cudaFreeHost(L.h_table);
-    if (L.h_cta) cudaFreeHost(L.h_cta);
+    if (L.h_items) cudaFreeHost(L.h_items);
     if (L.h_results) cudaFreeHost(L.h_results);
     if (L.h_err) cudaFreeHost(L.h_err);
-    if (L.copies) cudaEventDestroy(L.copies);
     if (L.d_table) cudaFree(L.d_table);
     if (L.d_cta) cudaFree(L.d_cta);
-    if (L.d_results) cudaFree(L.d_results);
   }
   if (s->copy_stream) cudaStreamSynchronize(s->copy_stream);
   for (auto& S : s->streams) {
@@ -457,13 +458,10 @@ SP_API sp_status sp_server_create(const sp_server_config* cfg, sp_server** out) 
   for (auto& L : s->slots) {
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&L.st, cudaStreamNonBlocking);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&L.done, cudaEventDisableTiming);
-    if (e == cudaSuccess) e = cudaMallocHost(&L.h_table, sizeof(sp::TickMember) * cfg->max_streams);
-    if (e == cudaSuccess) e = cudaMallocHost(&L.h_cta, (size_t)s->max_ctas * 4);
+    if (e == cudaSuccess) e = cudaMallocHost(&L.h_items, sizeof(sp::TickItem) * cfg->max_streams);
     if (e == cudaSuccess) e = cudaMallocHost(&L.h_results, (size_t)cfg->max_streams * row * 4);
     if (e == cudaSuccess) e = device_malloc((void**)&L.d_table, sizeof(sp::TickMember) * cfg->max_streams);
     if (e == cudaSuccess) e = device_malloc((void**)&L.d_cta, (size_t)s->max_ctas * 4);
-    if (e == cudaSuccess) e = device_malloc((void**)&L.d_results, (size_t)cfg->max_streams * row * 4);
-    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&L.copies, cudaEventDisableTiming);
     if (e == cudaSuccess) e = cudaHostAlloc((void**)&L.h_err, 4, cudaHostAllocMapped);
     if (e == cudaSuccess) {
       *L.h_err = 0u;
@@ -546,6 +544,7 @@ void publish(sp_server* s, const std::vector<Pending>& ps, const std::vector<boo
     ++s->submitted;
     if (request_ids) request_ids[ps[k].entry] = r.id;
   }
+  s->published.fetch_add(ps.size(), std::memory_order_release);
 }
 
 }  // namespace
@@ -567,7 +566,7 @@ SP_API sp_status sp_server_submit(sp_server* s, uint32_t id, const uint32_t* bit
 
 namespace {
 
-// Reserve, copy (host frames through the pinned ring on the copy stream, or
+// Reserve, copy (host frames into the pinned ring, which the launch reads, or
 // device frames on the caller's stream), publish.
 sp_status submit_impl(sp_server* s, uint32_t n, const uint32_t* ids,
                       const uint32_t* const* frames, const int* learn, uint64_t* request_ids,
@@ -603,16 +602,14 @@ sp_status submit_impl(sp_server* s, uint32_t n, const uint32_t* ids,
     // the stream cannot close while it has a reserved slot (outstanding > 0)
     Stream& S = s->streams[ps[k].stream];
     uint32_t* dst = S.d_ring + (size_t)ps[k].ring * S.input_words;
-    cudaError_t e;
+    cudaError_t e = cudaSuccess;
     if (device) {
       e = cudaMemcpyAsync(dst, frames[ps[k].entry], (size_t)S.input_words * 4,
                           cudaMemcpyDeviceToDevice, cst);
       if (e == cudaSuccess) e = cudaEventRecord(S.ev_h2d[ps[k].ring], cst);
     } else {
-      uint32_t* hs = S.h_ring + (size_t)ps[k].ring * S.input_words;
-      std::memcpy(hs, frames[ps[k].entry], (size_t)S.input_words * 4);
-      e = cudaMemcpyAsync(dst, hs, (size_t)S.input_words * 4, cudaMemcpyHostToDevice,
-                          s->copy_stream);
+      std::memcpy(S.h_ring + (size_t)ps[k].ring * S.input_words, frames[ps[k].entry],
+                  (size_t)S.input_words * 4);
     }
     if (e != cudaSuccess) {
       copied[k] = false;
@@ -646,6 +643,12 @@ SP_API sp_status sp_server_poll(sp_server* s, sp_server_result* results, uint32_
   if (!s || !n_results || (!results && max_results)) return fail(SP_EINVAL, "NULL argument");
   *n_results = 0;
   std::unique_lock<std::mutex> lk(s->mu);
+  if (s->done.empty() && wait_ms) {
+    const uint64_t seen = s->delivered.load(std::memory_order_acquire);
+    lk.unlock();
+    spin_while(s->delivered, seen);
+    lk.lock();
+  }
   if (s->done.empty() && wait_ms)
     s->cv_done.wait_for(lk, std::chrono::milliseconds(wait_ms), [&] { return !s->done.empty(); });
   uint32_t used = 0, n = 0;

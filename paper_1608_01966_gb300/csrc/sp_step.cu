@@ -1417,6 +1417,44 @@ uint32_t batch_stage_bytes(uint32_t C, uint32_t S, uint32_t n_ctas) {
   return kStepWarps * stage_ring_bytes(S);
 }
 
+// The start of a serving launch: kGatherParts CTAs per member read its item and
+// its frame straight from the host's pinned memory.  One launch in place of a
+// copy per frame and two for the tables: 32 streams' frames (1.1 MB) took 70 us
+// of host time to enqueue; what bounds this is two trips over the host link.
+constexpr uint32_t kGatherParts = 8;
+
+__global__ void __launch_bounds__(256) sp_tick_gather_kernel(const TickItem* items,
+                                                             TickMember* table,
+                                                             uint32_t* cta_inst) {
+  const TickItem& it = items[blockIdx.x / kGatherParts];
+  const uint32_t part = blockIdx.x % kGatherParts, t = threadIdx.x;
+  if (part == 0u) {
+    if (t == 0u) table[it.stream] = it.tm;
+    for (uint32_t c = t; c < it.n_ctas; c += 256u) cta_inst[it.tm.cta_first + c] = it.stream;
+  }
+  const uint32_t* src = it.src;
+  if (!src) return;
+  uint32_t* dst = const_cast<uint32_t*>(it.tm.x);
+  const uint32_t words = it.words;
+  if (((reinterpret_cast<uintptr_t>(src) | reinterpret_cast<uintptr_t>(dst)) & 15u) == 0u) {
+    const uint32_t n = words >> 2;
+#pragma unroll 4
+    for (uint32_t i = part * 256u + t; i < n; i += kGatherParts * 256u)
+      reinterpret_cast<uint4*>(dst)[i] = __ldcs(reinterpret_cast<const uint4*>(src) + i);
+    if (part == 0u && t < (words & 3u)) dst[(n << 2) + t] = __ldcs(src + (n << 2) + t);
+  } else {
+#pragma unroll 4
+    for (uint32_t i = part * 256u + t; i < words; i += kGatherParts * 256u) dst[i] = __ldcs(src + i);
+  }
+}
+
+cudaError_t launch_tick_gather(const TickItem* items, uint32_t count, TickMember* table,
+                               uint32_t* cta_inst, cudaStream_t stream) {
+  sp_tick_gather_kernel<<<count * kGatherParts, 256, 0, stream>>>(items, table, cta_inst);
+  g_launches.fetch_add(1, std::memory_order_relaxed);
+  return cudaGetLastError();
+}
+
 cudaError_t launch_batch_step(const BatchArgs& a, uint32_t n_ctas, uint32_t max_C, uint32_t max_S,
                               cudaStream_t stream) {
   const size_t smem = std::max<size_t>(step_smem_bytes(max_C, max_S),
