@@ -361,9 +361,13 @@ sp::StepArgs base_args(const sp_handle* h) {
 // frame's (used iff learning is pending); x_save, if set, receives a copy of
 // x for the next frame's learning.
 sp_status enqueue_frame(sp_handle* h, cudaStream_t st, const uint32_t* x, const uint32_t* x_prev,
-                        uint32_t* x_save, int learn, uint32_t* mask_copy, float* ov_copy = nullptr) {
+                        uint32_t* x_save, int learn, uint32_t* mask_copy, float* ov_copy = nullptr,
+                        bool host_result = false) {
   sp::StepArgs a = base_args(h);
   a.ov_copy = ov_copy;
+  // pinned memory, written by the kernel: sp_active_columns needs no copy
+  a.result_copy = host_result ? h->h_result : nullptr;
+  h->host_result = host_result;
   const int cur = h->cur;
   a.x = x;
   if (h->pending) {
@@ -515,6 +519,7 @@ sp_status run_dense(sp_handle* h, const uint32_t* x_base, uint32_t n, uint64_t s
 
 sp_status run_sequence(sp_handle* h, const uint32_t* x_base, uint32_t n, uint64_t stride,
                        int learn, uint32_t* masks, float* ovs = nullptr) {
+  h->host_result = false;
   if (learn) h->bimg_stale = true;
   if (!learn && h->dense && n >= kDenseMinFrames && dense_enabled())
     return run_dense(h, x_base, n, stride, masks, ovs);
@@ -961,7 +966,8 @@ SP_API sp_status sp_compute(sp_handle* h, const uint32_t* input_bits, int learn)
   uint32_t* dst = h->d_xsave[h->cur];
   SP_CUDA(cudaMemcpyAsync(dst, input_bits, (size_t)h->n_words * 4, cudaMemcpyHostToDevice,
                           h->stream));
-  return enqueue_frame(h, h->stream, dst, h->d_xsave[h->cur ^ 1], nullptr, learn, nullptr);
+  return enqueue_frame(h, h->stream, dst, h->d_xsave[h->cur ^ 1], nullptr, learn, nullptr, nullptr,
+                       true);
 }
 
 SP_API sp_status sp_compute_device(sp_handle* h, const uint32_t* d_bits, int learn, void* stream) {
@@ -1058,8 +1064,9 @@ SP_API sp_status sp_active_columns(sp_handle* h, uint32_t* out, uint32_t cap, ui
   if (!h || !n || (!out && cap)) return fail(SP_EINVAL, "NULL argument");
   if (h->batch) return fail(SP_EBUSY, "the handle is a member of a batch");
   DeviceGuard g(h->device);
-  SP_CUDA(cudaMemcpyAsync(h->h_result, h->d_result, ((size_t)h->max_active + 1) * 4,
-                          cudaMemcpyDeviceToHost, h->stream));
+  if (!h->host_result)
+    SP_CUDA(cudaMemcpyAsync(h->h_result, h->d_result, ((size_t)h->max_active + 1) * 4,
+                            cudaMemcpyDeviceToHost, h->stream));
   sp_status s = wait_handle(h);
   if (s != SP_OK) return s;
   const uint32_t cnt = h->h_result[0];
@@ -1453,6 +1460,7 @@ void free_batch(sp_batch* b) {
   for (sp_handle* h : b->members) {
     if (h->batch != b) continue;
     h->cur = b->cur;  // the members' buffers follow the batch's parity
+    h->host_result = false;
     h->pending = b->pending;
     h->stream = h->own_stream;
     h->frames += b->frames;

@@ -207,6 +207,7 @@ struct sp_handle {
   bool bimg_stale = true;           // the permanences may have changed since d_bimg was built
   uint32_t run_gen = 0;             // bumped whenever d_run_ov / d_run_masks are reallocated
   bool unit_boost = true;
+  bool host_result = false;      // the last frame wrote its list to h_result itself
   uint32_t* h_result = nullptr;  // pinned [1 + C]; at creation [3][C], the pools' extents
   cudaStream_t own_stream = nullptr;
   cudaStream_t stream = nullptr;  // stream of the last call
