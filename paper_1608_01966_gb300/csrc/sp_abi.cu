@@ -336,6 +336,7 @@ sp::StepArgs base_args(const sp_handle* h) {
   a.boost = h->d_boost;
   a.ov = h->d_ov;
   a.result = h->d_result;
+  a.list = 1u;
   a.counter = h->d_counter;
   a.unit = (h->unit_boost && h->cfg.inhibition == SP_INHIBIT_GLOBAL) ? 1u : 0u;
   a.hist = a.unit && h->S > sp::kStepBins ? h->d_hist : nullptr;

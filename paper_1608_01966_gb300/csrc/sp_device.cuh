@@ -288,12 +288,12 @@ __device__ uint32_t mark_paper_literal(const uint32_t* sv, uint32_t C, uint32_t 
 // The k-th largest of the counts in a histogram (hist[v] columns count v, v >=
 // 1; hist[0] is the largest count), by one warp: 32 bins a step from the
 // largest down.  T = 0 when at most k columns count (all of them win),
-// 0xffffffff when k is 0; else `need` of the columns at T win.
+// 0xffffffff when k is 0; else `need` of the `ties` columns at T win.
 __device__ __forceinline__ void warp_kth_count(const uint32_t* hist, uint32_t k, uint32_t& T,
-                                               uint32_t& need) {
+                                               uint32_t& need, uint32_t& ties) {
   const uint32_t lane = threadIdx.x & 31u;
   T = 0xffffffffu;
-  need = 0u;
+  need = ties = 0u;
   if (k == 0u) return;
   T = 0u;
   uint32_t acc = 0u;
@@ -310,7 +310,8 @@ __device__ __forceinline__ void warp_kth_count(const uint32_t* hist, uint32_t k,
     if (hit) {
       const int src = __ffs(hit) - 1;
       T = b0 - (uint32_t)src;
-      need = k - (acc + __shfl_sync(kFull, inc - h, src));
+      ties = __shfl_sync(kFull, h, src);
+      need = k - (acc + __shfl_sync(kFull, inc, src) - ties);
       return;
     }
     acc += __shfl_sync(kFull, inc, 31);
@@ -318,67 +319,84 @@ __device__ __forceinline__ void warp_kth_count(const uint32_t* hist, uint32_t k,
 }
 
 // Winner mask of global inhibition for all C columns, given (T, need): every
-// warp takes 32 columns a step (a ballot is a mask word); warp 0 then gives
-// the `need` lowest tied columns their bits, 32 words a step, and writes the
-// words to smask and, if list != nullptr, the ascending winner list.  stie
-// holds ceil(C / 32) words.  Returns the number of winners in warp 0's
-// threads.  Every thread of the block must call it; smask is visible to the
-// caller's other warps after its next barrier.
+// warp takes 32 columns a step (a ballot is a mask word), four steps at a time.
+// Where some tied columns win (need != 0) warp 0 gives the `need` lowest their
+// bits, 32 words a step; where a list is wanted it also numbers the words'
+// winners, and every warp writes its words' share of the ascending list.  The
+// words go to smask; stie holds ceil(C / 32) words.  Returns the number of
+// winners in warp 0's threads (0 without a list).  Every thread of the block
+// must call it; smask is complete after the caller's next barrier.
 template <int NTHREADS>
 __device__ uint32_t mark_global(const uint32_t* sv, uint32_t C, uint32_t T, uint32_t need,
                                 uint32_t* smask, uint32_t* stie, uint32_t* list) {
   constexpr uint32_t NW = NTHREADS / 32;
   const uint32_t warp = threadIdx.x >> 5, lane = threadIdx.x & 31u;
   const uint32_t words = (C + 31u) / 32u;
-  for (uint32_t w = warp; w < words; w += NW) {
-    const uint32_t i = 32u * w + lane, v = i < C ? sv[i] : 0u;
-    const uint32_t g = __ballot_sync(kFull, v > T);
-    const uint32_t e = __ballot_sync(kFull, i < C && v == T);
-    if (lane == 0u) {
-      smask[w] = g;
-      stie[w] = e;
+  for (uint32_t w0 = warp; w0 < words; w0 += 4u * NW) {
+    uint32_t v[4];
+#pragma unroll
+    for (uint32_t j = 0; j < 4u; ++j) {
+      const uint32_t i = 32u * (w0 + j * NW) + lane;
+      v[j] = i < C ? sv[i] : 0u;
+    }
+#pragma unroll
+    for (uint32_t j = 0; j < 4u; ++j) {
+      const uint32_t w = w0 + j * NW;
+      const uint32_t g = __ballot_sync(kFull, v[j] > T);
+      const uint32_t e = need ? __ballot_sync(kFull, v[j] == T) : 0u;  // T != 0: padding never ties
+      if (lane == 0u && w < words) {
+        smask[w] = g;
+        stie[w] = e;
+      }
     }
   }
+  if (need == 0u && !list) return 0u;
   group_sync<NTHREADS>();
-  if (warp != 0u) return 0u;
   uint32_t seen = 0u, total = 0u;
-  for (uint32_t b = 0; b < words; b += 32u) {
-    const uint32_t w = b + lane;
-    uint32_t m = w < words ? smask[w] : 0u;
-    if (need != 0u) {
-      uint32_t e = w < words ? stie[w] : 0u;
-      const uint32_t ce = __popc(e);
-      uint32_t inc = ce;
+  if (warp == 0u) {
+    for (uint32_t b = 0; b < words; b += 32u) {
+      const uint32_t w = b + lane;
+      uint32_t m = w < words ? smask[w] : 0u;
+      if (need != 0u) {
+        uint32_t e = w < words ? stie[w] : 0u;
+        const uint32_t ce = __popc(e);
+        uint32_t inc = ce;
 #pragma unroll
-      for (uint32_t o = 1; o < 32u; o <<= 1) {
-        const uint32_t y = __shfl_up_sync(kFull, inc, o);
-        if (lane >= o) inc += y;
-      }
-      const uint32_t before = seen + inc - ce;
-      seen += __shfl_sync(kFull, inc, 31);
-      uint32_t take = need > before ? min(need - before, ce) : 0u;
-      if (take == ce) {
-        m |= e;
-      } else {
-        for (; take != 0u; --take) {  // the lowest tied columns
-          m |= e & (0u - e);
-          e &= e - 1u;
+        for (uint32_t o = 1; o < 32u; o <<= 1) {
+          const uint32_t y = __shfl_up_sync(kFull, inc, o);
+          if (lane >= o) inc += y;
         }
+        const uint32_t before = seen + inc - ce;
+        seen += __shfl_sync(kFull, inc, 31);
+        uint32_t take = need > before ? min(need - before, ce) : 0u;
+        if (take == ce) {
+          m |= e;
+        } else {
+          for (; take != 0u; --take) {  // the lowest tied columns
+            m |= e & (0u - e);
+            e &= e - 1u;
+          }
+        }
+        if (w < words) smask[w] = m;
       }
-      if (w < words) smask[w] = m;
-    }
-    const uint32_t c = __popc(m);
-    uint32_t inc = c;
+      if (list) {
+        const uint32_t c = __popc(m);
+        uint32_t inc = c;
 #pragma unroll
-    for (uint32_t o = 1; o < 32u; o <<= 1) {
-      const uint32_t y = __shfl_up_sync(kFull, inc, o);
-      if (lane >= o) inc += y;
+        for (uint32_t o = 1; o < 32u; o <<= 1) {
+          const uint32_t y = __shfl_up_sync(kFull, inc, o);
+          if (lane >= o) inc += y;
+        }
+        if (w < words) stie[w] = total + inc - c;  // the word's first list slot
+        total += __shfl_sync(kFull, inc, 31);
+      }
     }
-    if (list) {
-      uint32_t pos = total + inc - c;
-      for (uint32_t r = m; r != 0u; r &= r - 1u) list[pos++] = 32u * w + (uint32_t)(__ffs(r) - 1);
-    }
-    total += __shfl_sync(kFull, inc, 31);
+  }
+  if (!list) return 0u;
+  group_sync<NTHREADS>();
+  for (uint32_t w = warp; w < words; w += NW) {
+    const uint32_t m = smask[w];
+    if ((m >> lane) & 1u) list[stie[w] + __popc(m & ((1u << lane) - 1u))] = 32u * w + lane;
   }
   return total;
 }

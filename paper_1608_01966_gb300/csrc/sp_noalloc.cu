@@ -102,6 +102,7 @@ SP_API sp_status sp_step_noalloc(const sp_config* cfg, const uint32_t* d_idx, fl
   a.x = d_input;
   a.mask_out = d_active_mask;
   a.result = d_active_list;
+  a.list = 1u;
   a.counter = counter;
   a.counter_clear = scratch + SP_NOALLOC_MAX_COLUMNS + (turn ^ 1u);
   a.C = C;

@@ -241,16 +241,17 @@ __device__ __forceinline__ uint32_t column_overlap(const StepArgs& a, uint32_t c
 // frame's chain, so it makes one pass over the overlaps in L2 (kSelLoads of a
 // thread's loads in flight).  Where the overlaps are counts (unit boosts, or
 // found to be whole numbers up to S) they are counted into a histogram in
-// shared memory as they arrive, and every warp reads the k-th largest off it:
-// four barriers in all.  dyn: C overlaps, two sets of mask words, and S + 2
-// bins where S <= kStepBins.
-constexpr int kSelLoads = 8;
+// shared memory as they arrive, and every warp reads the k-th largest off it.
+// The ascending list is written only where someone can read it (a.list).  In a
+// full batch launch this takes about a quarter of the SP's chain: a warp gets
+// one issue in ten.  dyn: C overlaps, two sets of mask words, and S + 2 bins
+// where S <= kStepBins.  Returns the mask words (shared memory).
+constexpr int kSelLoads = 16;
 
-__device__ void last_cta_inhibit(const StepArgs& a, uint32_t* dyn) {
+__device__ const uint32_t* last_cta_inhibit(const StepArgs& a, uint32_t* dyn) {
   __shared__ uint32_t shist[256];
   __shared__ uint32_t sh[2 * kStepWarps];
   __shared__ uint32_t s2[2];
-  __shared__ uint32_t s_total;
   const uint32_t C = a.C;
   const uint32_t t = threadIdx.x;
   uint32_t* sv = dyn;
@@ -300,16 +301,21 @@ __device__ void last_cta_inhibit(const StepArgs& a, uint32_t* dyn) {
       counts = a.unit ? (__syncthreads(), true) : __syncthreads_and(whole ? 1 : 0) != 0;
     }
     if (counts) {
-      dev::warp_kth_count(bins, a.k, T, need);
+      uint32_t ties;
+      dev::warp_kth_count(bins, a.k, T, need, ties);
       if (T != 0xffffffffu) T = __float_as_uint(__uint2float_rn(T));
+      if (need != 0u && need == ties) {
+        T -= 1u;  // every tied column wins: all above the pattern below T's
+        need = 0u;
+      }
     } else {
       uint32_t e0, e1, nz_tot, z;
       dev::block_scan2<kStepWarps>(nz, 0u, e0, e1, nz_tot, z, sh);  // also publishes sv
       dev::select_threshold<kStepThreads>(sv, C, a.k, nz_tot, a.hist, a.hist ? a.S : 0u, shist,
                                           sh, s2, T, need);
     }
-    total = dev::mark_global<kStepThreads>(sv, C, T, need, smask, stie, a.result + 1);
-    if (t == 0u) s_total = total;
+    total = dev::mark_global<kStepThreads>(sv, C, T, need, smask, stie,
+                                           a.list ? a.result + 1 : nullptr);
   } else if (a.inhibition == 1u) {
     for (uint32_t i = t; i < a.mask_words; i += kStepThreads) smask[i] = 0u;
     __syncthreads();
@@ -322,19 +328,7 @@ __device__ void last_cta_inhibit(const StepArgs& a, uint32_t* dyn) {
                                                   s2);
   }
   __syncthreads();
-  if (a.inhibition == 0u) total = s_total;
-  if (t == 0u) a.result[0] = total;
-  if (a.learn_next) {
-    // the SP's next frame learns these winners first thing: ask L2 for their
-    // pool indices and permanences now
-    const uint32_t lines = (a.S * 4u + 127u) / 128u;
-    for (uint32_t i = t; i < C; i += kStepThreads)
-      if ((smask[i >> 5] >> (i & 31u)) & 1u)
-        for (uint32_t l = 0; l < lines; ++l) {
-          asm volatile("prefetch.global.L2 [%0];" ::"l"(a.idx + (uint64_t)i * a.S + 32u * l));
-          asm volatile("prefetch.global.L2 [%0];" ::"l"(a.perm + (uint64_t)i * a.S + 32u * l));
-        }
-  }
+  if (t == 0u && a.list) a.result[0] = total;  // thread 0's total is complete in every mode
   if (a.hist)
     for (uint32_t b = t; b <= a.S; b += kStepThreads) a.hist[b] = 0u;
   for (uint32_t i = t; i < a.mask_words; i += kStepThreads) {
@@ -351,10 +345,26 @@ __device__ void last_cta_inhibit(const StepArgs& a, uint32_t* dyn) {
     }
   }
   if (a.result_copy) {
+    __shared__ uint32_t s_total;
+    if (t == 0u) s_total = total;
     __syncthreads();  // the list written above is visible to the whole CTA
+    total = s_total;
     for (uint32_t i = t; i <= total; i += kStepThreads)
       a.result_copy[i] = i == 0u ? total : __ldcg(a.result + i);
   }
+  return smask;
+}
+
+// The SP's next frame learns these winners first thing: ask L2 for their pool
+// indices and permanences now.
+__device__ __forceinline__ void prefetch_winners(const StepArgs& a, const uint32_t* smask) {
+  const uint32_t lines = (a.S * 4u + 127u) / 128u;
+  for (uint32_t i = threadIdx.x; i < a.C; i += kStepThreads)
+    if ((smask[i >> 5] >> (i & 31u)) & 1u)
+      for (uint32_t l = 0; l < lines; ++l) {
+        asm volatile("prefetch.global.L2 [%0];" ::"l"(a.idx + (uint64_t)i * a.S + 32u * l));
+        asm volatile("prefetch.global.L2 [%0];" ::"l"(a.perm + (uint64_t)i * a.S + 32u * l));
+      }
 }
 
 // Columns of one SP given to CTA bid of nb: a contiguous range of
@@ -664,8 +674,14 @@ __device__ __forceinline__ void window_item(const StepArgs& a, uint32_t lo, uint
 
   // ---- the count: this warp's columns, COLS at a time --------------------
   const uint32_t lane_off = (uint32_t)lane * wpr, row32 = 32u * wpr;
-  const bool learners = a.mask_prev && s_nl != 0u;  // s_nl is stable after the barrier
-  for (uint32_t c = c0; c < hi; c += COLS * kStepWarps) {
+  // this warp's learners: bit i for its i-th column (s_nl is stable after the barrier)
+  unsigned long long lm = 0ull;
+  if (a.mask_prev && s_nl != 0u) {
+    const uint32_t i0 = (uint32_t)warp + 4u * lane, i1 = i0 + 128u;
+    lm = __ballot_sync(kFull, i0 < n && s_lmap[i0] != 0u) |
+         (unsigned long long)__ballot_sync(kFull, i1 < n && s_lmap[i1] != 0u) << 32;
+  }
+  for (uint32_t c = c0; c < hi; c += COLS * kStepWarps, lm >>= COLS) {
 #if SP_WIN_PIPE
     uint4 nx[COLS];
     load_group(c + COLS * kStepWarps, nx);
@@ -673,10 +689,12 @@ __device__ __forceinline__ void window_item(const StepArgs& a, uint32_t lo, uint
     uint32_t cnt[COLS];
 #pragma unroll
     for (int j = 0; j < COLS; ++j) {
-      const uint32_t cj = c + j * kStepWarps;
-      const uint32_t li = (learners && cj < hi) ? s_lmap[cj - lo] : 0u;
+      // no branch but for learners: the loads of all COLS columns go out
+      // together (a column past the last repeats it and is not published)
+      const uint32_t cj = min(c + j * kStepWarps, hi - 1u);
       uint4 b = bm[j];
-      if (li != 0u) {  // a learner: its bitmap as rewritten above
+      if ((lm >> j) & 1ull) {  // a learner: its bitmap as rewritten above
+        const uint32_t li = s_lmap[cj - lo];
         if (li != 255u) {
           const uint32_t* s = scr + (li - 1u) * kWinWords;
           b = make_uint4(s[2 * lane], s[2 * lane + 1], s[2 * lane + 64], s[2 * lane + 65]);
@@ -684,7 +702,7 @@ __device__ __forceinline__ void window_item(const StepArgs& a, uint32_t lo, uint
           b = __ldcg(reinterpret_cast<const uint4*>(a.wbits + (uint64_t)cj * kWinWords) + lane);
         }
       }
-      cnt[j] = (ok && cj < hi) ? window_count(band, b, s_org[cj - lo], lane_off, row32) : 0u;
+      cnt[j] = window_count(band, b, s_org[cj - lo], lane_off, row32);
     }
     // lane j publishes the group's column j
     uint32_t mine = 0u;
@@ -694,7 +712,7 @@ __device__ __forceinline__ void window_item(const StepArgs& a, uint32_t lo, uint
       mine = lane == j ? r : mine;
     }
     if (lane < COLS && c + (uint32_t)lane * kStepWarps < hi)
-      publish_overlap(a, c + (uint32_t)lane * kStepWarps, mine);
+      publish_overlap(a, c + (uint32_t)lane * kStepWarps, ok ? mine : 0u);
 #if SP_WIN_PIPE
 #pragma unroll
     for (int j = 0; j < COLS; ++j) bm[j] = nx[j];
@@ -932,7 +950,7 @@ __device__ __forceinline__ void step_body(const StepArgs& a, uint32_t bid, uint3
   __syncthreads();
   if (s_ticket != nb - 1u) return;
   __threadfence();
-  last_cta_inhibit(a, dyn_smem);
+  const uint32_t* smask = last_cta_inhibit(a, dyn_smem);
   if (threadIdx.x == 0) atomicExch(a.counter, 0u);
   if (done) {
     // release this frame's results (mask, list, reset counter and
@@ -943,6 +961,8 @@ __device__ __forceinline__ void step_body(const StepArgs& a, uint32_t bid, uint3
       atomicExch(done, done_value);
     }
   }
+  // after the release: the next frame's items need not wait for it
+  if (a.learn_next) prefetch_winners(a, smask);
 }
 
 template <int VEC>
@@ -974,6 +994,7 @@ __global__ void __launch_bounds__(kStepThreads, SP_BATCH_MIN_BLOCKS) sp_batch_st
   const BatchDesc& d = ba.desc[inst];
   StepArgs a;
   a.learn_next = 0u;
+  a.list = 1u;
   a.idx = d.idx;
   a.perm = d.perm;
   a.boost = d.boost;
@@ -1129,6 +1150,7 @@ __global__ void __launch_bounds__(kStepThreads, MINB) sp_batch_run_kernel(const 
     StepArgs a;
     a.learn_next = r.learn;
     a.unit = d.unit;
+    a.list = t + 1u == r.n_frames ? 1u : 0u;  // only the last frame's list can be read
     const uint32_t cur = r.cur0 ^ (t & 1u);
     const uint32_t pending = t > 0u ? r.learn : r.pending0;
     const uint32_t save = t + 1u == r.n_frames ? 1u : 0u;
