@@ -420,6 +420,15 @@ sp_status enqueue_sequence(sp_handle* h, cudaStream_t st, const uint32_t* x_base
   return SP_OK;
 }
 
+// Whether n frames run in one cluster launch.
+bool use_cluster(const sp_handle* h, uint32_t n) {
+  const uint32_t least =
+      h->cfg.inhibition == SP_INHIBIT_LOCAL && h->C >= kSeqLocalColumns
+          ? 1u
+          : (h->seq_form == sp::kSeqWindowL2 ? kSeqMinFramesL2 : kSeqMinFrames);
+  return h->seq_ok && n >= least && seq_enabled();
+}
+
 // Run a frame sequence on the handle's stream: replay its recorded graph if
 // this exact sequence was seen before, else record it on the private capture
 // stream first.  Short sequences, or SP_DISABLE_GRAPHS=1, launch directly.
@@ -524,7 +533,7 @@ sp_status run_sequence(sp_handle* h, const uint32_t* x_base, uint32_t n, uint64_
   if (learn) h->bimg_stale = true;
   if (!learn && h->dense && n >= kDenseMinFrames && dense_enabled())
     return run_dense(h, x_base, n, stride, masks, ovs);
-  if (h->seq_ok && n >= kSeqMinFrames && seq_enabled()) {
+  if (use_cluster(h, n)) {
     sp::SeqArgs a{};
     a.idx = h->d_idx;
     a.perm = h->d_perm;
@@ -967,6 +976,7 @@ SP_API sp_status sp_compute(sp_handle* h, const uint32_t* input_bits, int learn)
   uint32_t* dst = h->d_xsave[h->cur];
   SP_CUDA(cudaMemcpyAsync(dst, input_bits, (size_t)h->n_words * 4, cudaMemcpyHostToDevice,
                           h->stream));
+  if (use_cluster(h, 1)) return run_sequence(h, dst, 1, h->n_words, learn, nullptr);
   return enqueue_frame(h, h->stream, dst, h->d_xsave[h->cur ^ 1], nullptr, learn, nullptr, nullptr,
                        true);
 }
@@ -978,6 +988,7 @@ SP_API sp_status sp_compute_device(sp_handle* h, const uint32_t* d_bits, int lea
   DeviceGuard g(h->device);
   sp_status s = use_stream(h, static_cast<cudaStream_t>(stream));
   if (s != SP_OK) return s;
+  if (use_cluster(h, 1)) return run_sequence(h, d_bits, 1, h->n_words, learn, nullptr);
   return enqueue_frame(h, h->stream, d_bits, h->d_xsave[h->cur ^ 1],
                        learn ? h->d_xsave[h->cur] : nullptr, learn, nullptr);
 }

@@ -85,7 +85,15 @@ uint32_t batch_xspan_cap();
 constexpr uint32_t kChunkFrames = 32;  // frames per staged chunk in sp_compute_frames
 constexpr int kSlots = 2;
 constexpr uint32_t kGraphMinFrames = 4;  // shorter sequences are launched directly
-constexpr uint32_t kSeqMinFrames = 8;    // shorter sequences use the per-frame kernel
+// Sequences of at least so many frames run in one cluster launch, fewer as one
+// kernel per frame (us, cluster / per frame: 1024 x 256 1 frame 19.7 / 10.4, 2
+// 22.7 / 20.7, 3 24.8 / 30.9; 256 x 16 2 16.4 / 15.5, 3 17.9 / 23.8).  With local
+// inhibition a single frame already: the per-frame kernel ranks all columns in
+// its last CTA (4096 x 64: 20.6 / 63.7).  Building the bitmaps of an SP that
+// large takes longer (4096 x 256 4 57.8 / 54.9, 6 68.2 / 80.9).
+constexpr uint32_t kSeqMinFrames = 3;
+constexpr uint32_t kSeqMinFramesL2 = 5;
+constexpr uint32_t kSeqLocalColumns = 512;  // fewer are ranked fast enough by one CTA
 // Sequences of SPs of at most so many synapses, on frames of at most so many
 // words, run in one CTA instead of a cluster, us per frame: 256 x 16 2.02
 // against 2.56, 512 x 16 2.51 / 2.65, 256 x 32 2.62 / 2.74, but 256 x 64 3.66 /

@@ -317,32 +317,87 @@ __global__ void __launch_bounds__(kSeqThreads + kSeqHelpers, 1) sp_seq_cluster_k
     const uint32_t r = __umulhi(id, inv_w);
     return r * a.win_w > id ? r - 1u : r;
   };
-  // boxes of the columns, and the smallest and largest value that the CTA's
-  // band must cover (input indices; window forms: box rows)
+  // position of synapse id in its column's box: (bitmap word << 5) | bit
+  auto box_pos = [&](uint32_t id, uint32_t org) {
+    const uint32_t d = id - (org >> 16) * a.win_w;
+    const uint32_t r = row_of(d), jx = d - r * a.win_w - (org & 0xffffu);
+    return ((4u * (r & 31u) + 2u * (r >> 5) + (jx >> 5)) << 5) | (jx & 31u);
+  };
+  // learning left pending by the previous call; the columns' boxes and bitmaps;
+  // the smallest and largest value that the CTA's band must cover (input
+  // indices; window forms: box rows)
   if (!helper) {
     uint32_t mn = 0xffffffffu, mx = 0u;
     for (uint32_t i = 0; i < own; ++i) {
       const uint32_t lc = own_col(i);
       if (lc >= nc) continue;
-      const uint32_t* row = kWindow ? a.idx + g0 + (uint64_t)lc * S : s_idx + lc * S;
+      const uint32_t c = c0 + lc;
+      const bool pend = a.pend_mask && ((__ldg(a.pend_mask + (c >> 5)) >> (c & 31u)) & 1u);
       if (kWindow) {
+        // kBatch synapses a lane at a time, loaded before the first is used (a
+        // pool of up to 256 is read once)
+        constexpr int kBatch = 8;
+        const uint64_t e0 = g0 + (uint64_t)lc * S;
+        uint32_t id[kBatch];
+        float pm[kBatch];
+        auto load_batch = [&](uint32_t s0) {
+#pragma unroll
+          for (int j = 0; j < kBatch; ++j) {
+            const uint32_t s = min(s0 + 32u * j, S - 1u);
+            id[j] = __ldg(a.idx + e0 + s);
+            pm[j] = a.perm[e0 + s];
+          }
+        };
         uint32_t x0 = 0xffffffffu, y0 = 0xffffffffu;
-        for (uint32_t s = lane; s < S; s += 32u) {
-          const uint32_t id = __ldg(row + s), y = row_of(id);
-          x0 = min(x0, id - y * a.win_w);
-          y0 = min(y0, y);
+        for (uint32_t s0 = lane; s0 < S; s0 += 32u * kBatch) {
+          load_batch(s0);
+#pragma unroll
+          for (int j = 0; j < kBatch; ++j) {
+            const uint32_t y = row_of(id[j]);
+            x0 = min(x0, id[j] - y * a.win_w);
+            y0 = min(y0, y);
+          }
         }
         x0 = __reduce_min_sync(kFull, x0);
         y0 = __reduce_min_sync(kFull, y0);
-        if (lane == 0u) s_org[lc] = (y0 << 16) | x0;
+        const uint32_t org = (y0 << 16) | x0;
+        if (lane == 0u) s_org[lc] = org;
         mn = min(mn, y0);
         mx = max(mx, y0 + 63u);
+        uint32_t* wb = s_bits + lc * kBoxWords;
+        reinterpret_cast<uint4*>(wb)[lane] = make_uint4(0u, 0u, 0u, 0u);
+        __syncwarp();
+        for (uint32_t s0 = lane; s0 < S; s0 += 32u * kBatch) {
+          if (S > 32u * kBatch) load_batch(s0);
+#pragma unroll
+          for (int j = 0; j < kBatch; ++j) {
+            const uint32_t s = s0 + 32u * j;
+            if (s < S) {
+              const uint32_t pos = box_pos(id[j], org);
+              float p = pm[j];
+              if (pend) p = learn_one(p, dev::input_bit(a.pend_x, id[j]), a.inc, a.dec);
+              if (kPermSmem) {
+                s_pos[lc * S + s] = (uint16_t)pos;
+                s_perm[lc * S + s] = p;
+              } else if (pend) {
+                a.perm[e0 + s] = p;
+              }
+              if (p >= a.thr) atomicOr(wb + (pos >> 5), 1u << (pos & 31u));
+            }
+          }
+        }
       } else {
+        const uint32_t* row = s_idx + lc * S;
         for (uint32_t s = lane; s < S; s += 32u) {
-          mn = min(mn, row[s]);
-          mx = max(mx, row[s]);
+          const uint32_t id = row[s];
+          mn = min(mn, id);
+          mx = max(mx, id);
+          if (pend)
+            s_perm[lc * S + s] =
+                learn_one(s_perm[lc * S + s], dev::input_bit(a.pend_x, id), a.inc, a.dec);
         }
       }
+      if (pend && kPermSmem && lane == 0u) atomicOr(s_dirty + (lc >> 5), 1u << (lc & 31u));
     }
     mn = __reduce_min_sync(kFull, mn);
     mx = __reduce_max_sync(kFull, mx);
@@ -372,48 +427,12 @@ __global__ void __launch_bounds__(kSeqThreads + kSeqHelpers, 1) sp_seq_cluster_k
       blen = (m1 >> 5) + 1u - w_lo;
     }
   }
-  // position of synapse id in its column's box: (bitmap word << 5) | bit
-  auto box_pos = [&](uint32_t id, uint32_t org) {
-    const uint32_t d = id - (org >> 16) * a.win_w;
-    const uint32_t r = row_of(d), jx = d - r * a.win_w - (org & 0xffffu);
-    return ((4u * (r & 31u) + 2u * (r >> 5) + (jx >> 5)) << 5) | (jx & 31u);
-  };
-  // ---- learning left pending by the previous call, then the bitmaps ----------
   if (helper) {
     copy_band(s_band, a.frames + w_lo, brows, blen, pitch, &s_band_bar[0]);
-  } else {
-    for (uint32_t i = 0; i < own; ++i) {
-      const uint32_t lc = own_col(i);
-      if (lc >= nc) continue;
-      const uint32_t c = c0 + lc;
-      const bool pend = a.pend_mask && ((__ldg(a.pend_mask + (c >> 5)) >> (c & 31u)) & 1u);
-      if (kWindow) {
-        const uint32_t org = s_org[lc];
-        uint32_t* wb = s_bits + lc * kBoxWords;
-        reinterpret_cast<uint4*>(wb)[lane] = make_uint4(0u, 0u, 0u, 0u);
-        if (lane == 0u)
-          s_at[lc] = ((((org >> 16) - y_lo) * pitch + ((org & 0xffffu) >> 5)) << 5) | (org & 31u);
-        __syncwarp();
-        for (uint32_t s = lane; s < S; s += 32u) {
-          const uint64_t e = g0 + (uint64_t)lc * S + s;
-          const uint32_t id = __ldg(a.idx + e), pos = box_pos(id, org);
-          float p = a.perm[e];
-          if (pend) p = learn_one(p, dev::input_bit(a.pend_x, id), a.inc, a.dec);
-          if (kPermSmem) {
-            s_pos[lc * S + s] = (uint16_t)pos;
-            s_perm[lc * S + s] = p;
-          } else if (pend) {
-            a.perm[e] = p;
-          }
-          if (p >= a.thr) atomicOr(wb + (pos >> 5), 1u << (pos & 31u));
-        }
-      } else if (pend) {
-        for (uint32_t s = lane; s < S; s += 32u) {
-          const uint32_t e = lc * S + s;
-          s_perm[e] = learn_one(s_perm[e], dev::input_bit(a.pend_x, s_idx[e]), a.inc, a.dec);
-        }
-      }
-      if (pend && kPermSmem && lane == 0u) atomicOr(s_dirty + (lc >> 5), 1u << (lc & 31u));
+  } else if (kWindow) {
+    for (uint32_t lc = t; lc < nc; lc += kSeqThreads) {
+      const uint32_t org = s_org[lc];
+      s_at[lc] = ((((org >> 16) - y_lo) * pitch + ((org & 0xffffu) >> 5)) << 5) | (org & 31u);
     }
   }
   // barriers initialized, counts cleared and bitmaps built in every CTA

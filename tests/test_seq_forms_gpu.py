@@ -146,3 +146,31 @@ def test_all_columns_tie():
     np.testing.assert_array_equal(spg.masks_to_dense(masks.cpu().numpy().view(np.uint32), 777), act)
     assert (act.sum(axis=1) == 333).all()
     spg.sp_destroy(h)
+
+
+@pytest.mark.parametrize("n", [1, 2, 3, 5, 7])
+@pytest.mark.parametrize("inh", [0, 1])
+def test_short_sequences_and_single_frames(n, inh):
+    """Runs of every short length from the two frame APIs in turn, learning on
+    and off, so that each launch form takes over pending learning from the
+    others."""
+    C, W, H, S = 32 * 17, 96, 80, 100
+    idx = _box_pools(np.random.default_rng(12), C, S, W, H, 64)
+    perm = synth.perm_uniform(78, (C, S), 0.1, 0.3)
+    case = wl.Case("short", W, H, C, S, idx, perm, np.ones(C, np.float32), min_overlap=3, k=9,
+                   inhibition=inh, gw=32, gh=17, radius=3)
+    fr = (np.random.default_rng(6).random((4 * (n + 2), W * H)) < 0.3).astype(np.uint8)
+    packed = wl.pack(fr)
+    d = torch.from_numpy(packed.view(np.int32)).cuda()
+    h = spg.sp_create_from_state(case.config(), idx, perm, case.boost)
+    p, t, st = perm, 0, torch.cuda.current_stream()
+    for turn in range(4):
+        learn = turn != 2
+        spg.sp_compute_frames_device(h, d[t], n, packed.shape[1], learn, None, st)
+        spg.sp_compute_device(h, d[t + n], learn, st)
+        spg.sp_compute(h, packed[t + n + 1], learn)
+        act, p, _ = oracle_run(case, fr[t:t + n + 2], learn, perm=p)
+        np.testing.assert_array_equal(spg.sp_active_columns(h), np.flatnonzero(act[-1]))
+        t += n + 2
+    np.testing.assert_array_equal(spg.sp_get_permanences(h), p)
+    spg.sp_destroy(h)
