@@ -318,8 +318,9 @@ SP_API sp_status sp_batch_get_info(const sp_batch* b, sp_batch_info* out);
 SP_API sp_status sp_batch_autotune(sp_batch* b, const uint32_t* d_frames, uint32_t n_frames,
                                    uint64_t stride, uint32_t* cols_per_warp);
 
-/* The batch's schedule as set by sp_batch_autotune (before tuning: the
- * default): resident CTAs per SM and columns per warp in flight of the
+/* The batch's schedule as set by sp_batch_autotune (before tuning: 8 x 4 for
+ * batches whose members' default splits give at most 18 CTAs per SM, 10 x 4
+ * for larger ones): resident CTAs per SM and columns per warp in flight of the
  * persistent pass, and each member's columns per warp (an array of
  * `members` entries, 0 for the member's default).  Any output may be NULL.
  * Tuning machinery: the paper has no counterpart. */
@@ -329,7 +330,7 @@ SP_API sp_status sp_batch_schedule(const sp_batch* b, uint32_t* ctas_per_sm,
 /* The compiled schedules of the persistent pass (needs no device): *count
  * (nullable) receives how many; ctas_per_sm[i] and cols_in_flight[i]
  * (either nullable, room for cap entries, else SP_EINVAL) receive each.
- * Entry 0 is the default.  Tuning machinery: the paper has no counterpart. */
+ * Entry 0 is the default of large batches.  Tuning machinery: the paper has no counterpart. */
 SP_API sp_status sp_batch_schedule_list(uint32_t* ctas_per_sm, uint32_t* cols_in_flight,
                                         uint32_t cap, uint32_t* count);
 

@@ -482,7 +482,7 @@ def sp_batch_schedule(b, members):
 
 def sp_batch_schedule_list():
     """[(ctas_per_sm, cols_in_flight)] of the compiled schedules; the first is
-    the default."""
+    the default of large batches."""
     n = ct.c_uint32(0)
     _check(lib().sp_batch_schedule_list(None, None, 0, ct.byref(n)), "sp_batch_schedule_list")
     cps = (ct.c_uint32 * max(1, n.value))()

@@ -1279,7 +1279,8 @@ struct sp_batch {
   void* d_sync = nullptr;             // persistent launches: work counter, abort, done[n]
   std::vector<uint32_t> member_cpw;   // columns per warp of each member (0: the default)
   uint32_t default_cpw = 0;           // the batch's default columns per warp (default_split)
-  uint32_t sched = 0;                 // compiled schedule of the persistent pass (0: default)
+  uint32_t default_sched = 0;         // the batch's default schedule (batch_default_schedule)
+  uint32_t sched = 0;                 // compiled schedule of the persistent pass
   uint32_t stage_cap = 0;             // shared memory for staging state by bulk copy
   uint32_t xspan_cap = 0;             // shared memory for each CTA's input words
   uint32_t win_cap = 0;               // shared memory of the widest window-form CTA
@@ -1337,12 +1338,10 @@ uint32_t batch_ctas(uint32_t C, uint32_t S, uint32_t cols_per_warp) {
 // more, each takes its ticket for too little work.  us per frame by columns per
 // warp 2 / 4 / 8 / 16 / 32: 8 SPs of 1024 x 256 16.5 16.4 17.6 19.9 25.5; 32: 19.6
 // 18.6 20.2 24.1 31.3; 64: 38 22.2 21.8 26.7 34.1; 128: 75 43 29.0 27.0 35.2; 200: 120
-// 70 46 34.6 39.2; 256: 159 93 61 44.9 43.3.  Where sizes are uneven the largest
-// SP's chain is the longest, and half as many items again pay: 64 SPs of 128 to
-// 4096 columns 91 54 41.9 45.5 59.7 (60.5 with 32, 16 or 8 by the synapses).
-uint32_t default_split(uint64_t columns, uint32_t members, uint32_t largest, int sms) {
-  uint64_t items = 22ull * (uint64_t)sms;  // 10 CTAs resident per SM
-  if ((uint64_t)largest * members * 2u >= columns * 3u) items += items / 2u;
+// 70 46 34.6 39.2; 256: 159 93 61 44.9 43.3; 64 SPs of 128 to 4096 columns, each
+// count with the better schedule (batch_default_schedule): - 55 41.2 38.6 52.3.
+uint32_t default_split(uint64_t columns, int sms) {
+  const uint64_t items = 22ull * (uint64_t)sms;
   uint32_t cpw = 2u;
   while (cpw < 32u && columns > items * (uint64_t)(sp::kStepWarps * cpw)) cpw *= 2u;
   return cpw;
@@ -1646,16 +1645,12 @@ SP_API sp_status sp_batch_create(sp_handle* const* members, uint32_t n, sp_batch
     }
   }
   uint64_t columns = 0;
-  uint32_t largest = 0;
-  for (uint32_t i = 0; i < n; ++i) {
-    columns += members[i]->C;
-    largest = std::max(largest, members[i]->C);
-  }
+  for (uint32_t i = 0; i < n; ++i) columns += members[i]->C;
   int sms = 0;
   if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, b->device) != cudaSuccess || sms < 1)
     sms = 1;
   if (!std::getenv("SP_BATCH_COLS_PER_WARP"))
-    b->default_cpw = default_split(columns, n, largest, sms);
+    b->default_cpw = default_split(columns, sms);
   std::vector<sp::BatchDesc> desc(n);
   std::vector<uint32_t> cta_inst;
   uint64_t foff = 0, moff = 0, ooff = 0;
@@ -1686,6 +1681,7 @@ SP_API sp_status sp_batch_create(sp_handle* const* members, uint32_t n, sp_batch
   b->mask_words = moff;
   b->ov_words = ooff;
   b->n_ctas = (uint32_t)cta_inst.size();
+  b->sched = b->default_sched = sp::batch_default_schedule(b->n_ctas, sms);
   b->h_desc = desc;
   const size_t desc_bytes = align256(sizeof(sp::BatchDesc) * n);
   cudaError_t e = device_malloc((void**)&b->d_block, desc_bytes + cta_inst.size() * 4);
@@ -2258,7 +2254,7 @@ SP_API sp_status sp_batch_autotune(sp_batch* b, const uint32_t* d_frames, uint32
   constexpr float kGain = 1.03f;
   const size_t n = b->members.size();
   std::vector<uint32_t> cpw(n, 0u);
-  b->sched = 0u;
+  b->sched = b->default_sched;
   s = batch_relayout(b, cpw);
   float best_ms = 0.0f;
   if (s == SP_OK) s = time_layout(&best_ms);
@@ -2278,8 +2274,9 @@ SP_API sp_status sp_batch_autotune(sp_batch* b, const uint32_t* d_frames, uint32
   std::fill(cpw.begin(), cpw.end(), uniform);
   if (s == SP_OK) s = batch_relayout(b, cpw);
   // 2. the compiled schedule (resident CTAs per SM x columns in flight)
-  uint32_t best_sched = 0u;
-  for (uint32_t i = 1; persistent && s == SP_OK && i < sp::batch_schedule_count(); ++i) {
+  uint32_t best_sched = b->default_sched;
+  for (uint32_t i = 0; persistent && s == SP_OK && i < sp::batch_schedule_count(); ++i) {
+    if (i == b->default_sched) continue;
     b->sched = i;
     float ms = 0.0f;
     s = time_layout(&ms);

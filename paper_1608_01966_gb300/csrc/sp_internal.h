@@ -70,7 +70,7 @@ bool all_ones(const float* v, size_t n);
 sp_status handle_wait(sp_handle* h);
 sp_status handle_flush_learning(sp_handle* h);
 uint32_t batch_ctas(uint32_t C, uint32_t S, uint32_t cols_per_warp = 0);
-uint32_t default_split(uint64_t columns, uint32_t members, uint32_t largest, int sms);
+uint32_t default_split(uint64_t columns, int sms);
 uint32_t batch_stage_cap(uint32_t need);
 // The descriptor of one SP inside a multi-SP launch, in the best form it
 // qualifies for (window, compact, else full); *win_bytes (nullable) receives

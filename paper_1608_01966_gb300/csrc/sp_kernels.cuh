@@ -177,6 +177,7 @@ cudaError_t launch_batch_run(const BatchRunArgs& r, uint32_t max_C, uint32_t max
 // resident CTAs per SM and columns per warp in flight of schedule i (false
 // when i is out of range).
 uint32_t batch_schedule_count();
+uint32_t batch_default_schedule(uint32_t items, int sms);
 bool batch_schedule(uint32_t i, uint32_t* ctas_per_sm, uint32_t* cols_in_flight);
 // Compact form of an SP's pools and connectivity (S <= 256), rows padded to
 // cS = S rounded up to a multiple of 32 synapses and laid out lane-strided

@@ -1208,7 +1208,7 @@ __global__ void __launch_bounds__(kStepThreads, MINB) sp_batch_run_kernel(const 
 
 namespace {
 
-// The compiled schedules of the persistent batch pass; entry 0 is the default.
+// The compiled schedules of the persistent batch pass.
 struct RunSchedule {
   void (*kernel)(const BatchRunArgs);
   uint32_t ctas_per_sm, cols_in_flight;
@@ -1225,6 +1225,27 @@ constexpr uint32_t kNumRunSchedules = sizeof(kRunSchedules) / sizeof(kRunSchedul
 }  // namespace
 
 uint32_t batch_schedule_count() { return kNumRunSchedules; }
+
+// The schedule of a batch that nothing has tuned.  With 8 CTAs per SM a thread
+// has 64 registers instead of 48: more of a column group's loads and of a
+// learner's synapses are in flight, and a frame's items, each a chain of its
+// own, end sooner.  With many more items than that fit at once the two further
+// CTAs hide more.  us per frame, 10 x 4 / 8 x 4, by a frame's items per SM: 6.7
+// (16 SPs of 1024 x 256) 19.4 / 17.5; 10.5 (200 of 256 x 64) 29.9 / 28.4; 13.5 (64
+// of 1024 x 256) 25.3 / 22.2, (32 of 4096 x 256) 33.1 / 29.9, (256 of 1024 x 256)
+// 50.2 / 48.8; 16.0 (64 of 128 to 4096 columns) 41.0 / 38.6; 18.1 (32 of 4096 x
+// 256, 48 columns to a CTA) 32.7 / 28.9; 21 (100 of 2025 x 128) 60.5 / 69.7, (200
+// of 256 x 64) 28.9 / 33.5, (64 of 128 to 4096) 38.4 / 41.7: between the last
+// uneven points the two cross at 18.
+constexpr uint32_t kWideItemsPerSm = 18;
+
+uint32_t batch_default_schedule(uint32_t items, int sms) {
+  if ((uint64_t)items > (uint64_t)kWideItemsPerSm * (uint64_t)std::max(1, sms)) return 0u;
+  for (uint32_t i = 0; i < kNumRunSchedules; ++i)
+    if (kRunSchedules[i].ctas_per_sm == 8u && kRunSchedules[i].cols_in_flight == (uint32_t)kCompactCols)
+      return i;
+  return 0u;
+}
 
 bool batch_schedule(uint32_t i, uint32_t* ctas_per_sm, uint32_t* cols_in_flight) {
   if (i >= kNumRunSchedules) return false;
