@@ -1331,15 +1331,14 @@ uint32_t batch_ctas(uint32_t C, uint32_t S, uint32_t cols_per_warp) {
   return (C + per_cta - 1u) / per_cta;
 }
 
-// Columns per warp of a batch whose members together have `columns` columns,
-// the largest `largest`.  A frame of an SP is a chain (band or pools, count,
-// ticket, Alg. 2), and a warp's columns a chain inside it, so a warp gets the
-// fewest that keep a frame's items at most about twice the resident CTAs: with
-// more, each takes its ticket for too little work.  us per frame by columns per
-// warp 2 / 4 / 8 / 16 / 32: 8 SPs of 1024 x 256 16.5 16.4 17.6 19.9 25.5; 32: 19.6
-// 18.6 20.2 24.1 31.3; 64: 38 22.2 21.8 26.7 34.1; 128: 75 43 29.0 27.0 35.2; 200: 120
-// 70 46 34.6 39.2; 256: 159 93 61 44.9 43.3; 64 SPs of 128 to 4096 columns, each
-// count with the better schedule (batch_default_schedule): - 55 41.2 38.6 52.3.
+// Columns per warp of a batch whose members together have `columns` columns.
+// A frame of an SP is a chain (band or pools, count, ticket, Alg. 2), and a
+// warp's columns a chain inside it, so a warp gets the fewest that keep a
+// frame's items at most about 22 per SM: with more, each takes its ticket for
+// too little work.  us per frame by columns per warp 4 / 8 / 16 / 32: 16 SPs of
+// 1024 x 256 15.5 16.9 19.3 23.5; 64 of them 21.8 20.5 24.9 30.3; 256 90 57.8 41.6
+// 40.3; 100 SPs of 2025 x 128 72.6 56.4 48.5 52.2; 64 of 128 to 4096 columns 54.9
+// 41.2 41.0 55.3 (all with 10 CTAs per SM; the last with 8: 38.6 at 16).
 uint32_t default_split(uint64_t columns, int sms) {
   const uint64_t items = 22ull * (uint64_t)sms;
   uint32_t cpw = 2u;

@@ -1231,11 +1231,11 @@ uint32_t batch_schedule_count() { return kNumRunSchedules; }
 // learner's synapses are in flight, and a frame's items, each a chain of its
 // own, end sooner.  With many more items than that fit at once the two further
 // CTAs hide more.  us per frame, 10 x 4 / 8 x 4, by a frame's items per SM: 6.7
-// (16 SPs of 1024 x 256) 19.4 / 17.5; 10.5 (200 of 256 x 64) 29.9 / 28.4; 13.5 (64
-// of 1024 x 256) 25.3 / 22.2, (32 of 4096 x 256) 33.1 / 29.9, (256 of 1024 x 256)
-// 50.2 / 48.8; 16.0 (64 of 128 to 4096 columns) 41.0 / 38.6; 18.1 (32 of 4096 x
-// 256, 48 columns to a CTA) 32.7 / 28.9; 21 (100 of 2025 x 128) 60.5 / 69.7, (200
-// of 256 x 64) 28.9 / 33.5, (64 of 128 to 4096) 38.4 / 41.7: between the last
+// (16 SPs of 1024 x 256) 15.5 / 14.0; 10.5 (200 of 256 x 64) 24.0 / 22.7; 13.5 (64
+// of 1024 x 256) 20.2 / 17.7, (32 of 4096 x 256) 26.5 / 23.9, (256 of 1024 x 256)
+// 40.2 / 39.0; 16.0 (64 of 128 to 4096 columns) 41.0 / 38.6; 18.1 (32 of 4096 x
+// 256, 48 columns to a CTA) 26.2 / 23.1; 21 (100 of 2025 x 128) 48.4 / 55.7, (200
+// of 256 x 64) 23.1 / 26.8, (64 of 128 to 4096) 38.4 / 41.7: between the last
 // uneven points the two cross at 18.
 constexpr uint32_t kWideItemsPerSm = 18;
 
