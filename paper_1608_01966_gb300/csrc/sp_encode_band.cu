@@ -53,6 +53,7 @@ struct BandArgs {
   uint32_t g_pitch;     // bytes per gray row in shared memory
   uint32_t g_bytes;     // bytes of the gray area (16-byte multiple)
   uint32_t v_pitch;     // words per V row: >= Wr + block + 2, a multiple of 4
+  uint32_t vec4;        // f == 1 and 4-byte aligned rows: four pixels per load
   uint32_t vecf;        // f % 4 == 0 and 4-byte aligned rows: whole words per block row
 };
 
@@ -111,6 +112,17 @@ __device__ __forceinline__ uint32_t reduced_gray_words(const BandArgs& a, const 
   return (77u * r + 150u * g + 29u * b + 128u) >> 8;
 }
 
+// Luma of four RGB pixels held in three little-endian words
+// (R0 G0 B0 R1 | G1 B1 R2 G2 | B2 R3 G3 B3), packed as four bytes.
+__device__ __forceinline__ uint32_t luma4(uint32_t w0, uint32_t w1, uint32_t w2) {
+  constexpr uint32_t kW = 77u | (150u << 8) | (29u << 16);  // byte 3 weighs 0
+  const uint32_t g0 = __dp4a(w0, kW, 128u) >> 8;
+  const uint32_t g1 = __dp4a(__byte_perm(w0, w1, 0x0543), kW, 128u) >> 8;
+  const uint32_t g2 = __dp4a(__byte_perm(w1, w2, 0x0432), kW, 128u) >> 8;
+  const uint32_t g3 = __dp4a(w2 >> 8, kW, 128u) >> 8;
+  return g0 | (g1 << 8) | (g2 << 16) | (g3 << 24);
+}
+
 // Binomial-weighted sum of B values v[0..B-1]: the weights are symmetric,
 // so pairs are added first and multiplied once (half the multiplies).
 template <int B, typename F>
@@ -164,7 +176,41 @@ __global__ void __launch_bounds__(kEncThreads, 2) sp_encode_band_kernel(const Ba
     return (uint32_t)(gy < 0 ? 0 : (gy >= (int)a.Hr ? (int)a.Hr - 1 : gy));
   };
   const uint32_t* fw = reinterpret_cast<const uint32_t*>(fs);
-  if (a.vecf && a.f == 4u) {
+  if (a.vec4) {
+    // four pixels per item from aligned words (f == 1, W % 4 == 0)
+    const uint32_t q = a.Wr >> 2;
+    uint32_t r = tid / q, k = tid - r * q;
+    const uint32_t sr = kEncThreads / q, sk = kEncThreads - sr * q;
+    while (r < nG) {
+      uint32_t ru[kUnroll], ku[kUnroll], w0[kUnroll], w1[kUnroll], w2[kUnroll];
+#pragma unroll
+      for (int u = 0; u < kUnroll; ++u) {
+        ru[u] = r;
+        ku[u] = k;
+        advance(r, k, sr, sk, q);
+      }
+#pragma unroll
+      for (int u = 0; u < kUnroll; ++u) {
+        w0[u] = w1[u] = w2[u] = 0u;
+        if (ru[u] < nG) {
+          const uint32_t gy = clamp_row(ru[u]);
+          if (a.ch == 3u) {
+            const uint32_t* w = fw + (uint64_t)gy * q * 3u + 3u * ku[u];
+            w0[u] = __ldg(w);
+            w1[u] = __ldg(w + 1);
+            w2[u] = __ldg(w + 2);
+          } else {
+            w0[u] = __ldg(fw + (uint64_t)gy * q + ku[u]);
+          }
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < kUnroll; ++u)
+        if (ru[u] < nG)
+          *reinterpret_cast<uint32_t*>(G + ru[u] * a.g_pitch + 4u * ku[u]) =
+              a.ch == 3u ? luma4(w0[u], w1[u], w2[u]) : w0[u];
+    }
+  } else if (a.vecf && a.f == 4u) {
     // 4 x 4 blocks from aligned words: 3 words (RGB) or 1 word (gray) per block row
     const uint32_t wpr = a.W * a.ch / 4u;
     uint32_t r = tid / a.Wr, x = tid - r * a.Wr;
@@ -367,6 +413,10 @@ cudaError_t launch_encode_band(const EncodeArgs& e, uint32_t block, cudaStream_t
   a.out = e.out;
   a.out_stride = e.out_stride;
   a.n_words = e.n_words;
+  a.vec4 = (e.f == 1u && e.W % 4u == 0u && e.src_stride % 4u == 0u &&
+            reinterpret_cast<uintptr_t>(e.src) % 4u == 0u)
+               ? 1u
+               : 0u;
   a.vecf = (e.f % 4u == 0u && e.W % 4u == 0u && e.src_stride % 4u == 0u &&
             reinterpret_cast<uintptr_t>(e.src) % 4u == 0u) ? 1u : 0u;
   uint32_t th = 32;

@@ -37,8 +37,8 @@ cudaError_t launch_encode(EncodeArgs a, uint32_t block, cudaStream_t st) {
     else
       need = tall && image_rows < 25000u ? 85u : (a.ch == 1u ? 50u : 60u);
   } else if (a.ch == 1u) {
-    if (a.strips > 1u)
-      need = 50u;
+    if (a.strips > 1u)  // f 2, 252 b 11: n 30 h 200 33 / 29, n 128 h 400 97 / 142
+      need = tall && a.f == 2u && image_rows < 25000u ? 65u : 50u;
     else
       need = a.f == 1u ? (tall ? 101u : 95u) : (tall ? 95u : 60u);
   } else if (a.f == 1u) {
@@ -47,6 +47,13 @@ cudaError_t launch_encode(EncodeArgs a, uint32_t block, cudaStream_t st) {
     // at most 304 warps of 4 rows: two per SM
     const uint64_t warps = (uint64_t)a.n_frames * a.strips * ((a.Hr + 3u) / 4u);
     need = tall || warps > 304u ? 101u : (a.strips > 1u ? 65u : 85u);
+  }
+  if (!a8 && a.f == 1u && a.W % 4u == 0u && a.src_stride % 4u == 0u &&
+      reinterpret_cast<uintptr_t>(a.src) % 4u == 0u) {
+    // rows of whole words: the band kernel reads four pixels at a time (us,
+    // strip / band, b 7: gray 300 n 12 h 100 9.6 / 8.8, n 60 h 270 19 / 21, RGB
+    // 27 / 23, 404 n 40 19 / 23, 644 n 40 h 360 27 / 37)
+    need = std::max(need, image_rows < 4096u ? 101u : (a.ch == 1u ? 60u : 80u));
   }
   if (a.f >= 3u || a.Wr < 8u || filled < need) return launch_encode_band(a, block, st);
   // Rows per chunk: every chunk reads block - 1 rows besides its own, a chunk
