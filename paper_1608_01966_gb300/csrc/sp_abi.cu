@@ -798,19 +798,39 @@ bool handle_window(sp_handle* h, uint32_t n_ctas, uint32_t* win_bytes) {
   return true;
 }
 
-bool window_rebands(sp_handle* h, sp::BatchDesc* d, uint32_t* win_bytes) {
-  if (!d->worg) return false;
+// The bands of a member that is in the window form, for its split.
+static bool window_rebands(sp_handle* h, const sp::BatchDesc* d, uint32_t* win_bytes) {
   DeviceGuard g(h->device);
   const uint32_t need = (h->C + d->n_ctas - 1u) / d->n_ctas > 256u ? 0u : window_bands(h, d->n_ctas);
-  if (need == 0u || need > window_cap_bytes()) {
-    d->worg = nullptr;
-    d->wbits = nullptr;
-    d->wband = nullptr;
-    return false;
-  }
-  d->wband = h->d_wband;
+  if (need == 0u || need > window_cap_bytes()) return false;
   if (win_bytes) *win_bytes = need;
   return true;
+}
+
+// The form of a member for its split (d->n_ctas): window, else compact, else
+// full.  The form in use stays current by itself (learning writes it); a form
+// taken up here, and with `derive` the one in use too, is derived from the
+// permanences as they are now.
+static void choose_form(sp_handle* h, sp::BatchDesc* d, bool derive, uint32_t* win_bytes) {
+  const bool in_window = d->worg && !derive, in_compact = d->cidx && !derive;
+  d->worg = nullptr;
+  d->wbits = nullptr;
+  d->wband = nullptr;
+  d->cidx = nullptr;
+  d->cbase = nullptr;
+  d->conn = nullptr;
+  if (win_bytes) *win_bytes = 0u;
+  if (in_window ? window_rebands(h, d, win_bytes) : handle_window(h, d->n_ctas, win_bytes)) {
+    d->worg = h->d_worg;
+    d->wbits = h->d_wbits;
+    d->wband = h->d_wband;
+    d->wpr = h->cfg.input_w / 32u;
+    d->win_w = h->cfg.input_w;
+  } else if (in_compact || handle_compact(h)) {
+    d->cidx = h->d_cidx;
+    d->cbase = h->d_cbase;
+    d->conn = h->d_cconn;
+  }
 }
 
 void fill_desc(sp_handle* h, sp::BatchDesc* d, uint32_t cols_per_warp, uint32_t* win_bytes) {
@@ -844,18 +864,7 @@ void fill_desc(sp_handle* h, sp::BatchDesc* d, uint32_t cols_per_warp, uint32_t*
   d->radius = h->cfg.local_radius;
   d->n_ctas = batch_ctas(h->C, h->S, cols_per_warp);
   d->xspan = batch_xspan_cap() > 0u ? handle_xspan(h, d->n_ctas) : nullptr;
-  if (win_bytes) *win_bytes = 0u;
-  if (handle_window(h, d->n_ctas, win_bytes)) {
-    d->worg = h->d_worg;
-    d->wbits = h->d_wbits;
-    d->wband = h->d_wband;
-    d->wpr = h->cfg.input_w / 32u;
-    d->win_w = h->cfg.input_w;
-  } else if (handle_compact(h)) {
-    d->cidx = h->d_cidx;
-    d->cbase = h->d_cbase;
-    d->conn = h->d_cconn;
-  }
+  choose_form(h, d, true, win_bytes);
 }
 
 }  // namespace rt
@@ -2088,8 +2097,10 @@ namespace {
 
 // Re-split member i into CTAs of 4 * cols_per_warp[i] columns (0: the
 // member's default) and upload the descriptors and CTA map.  The batch must
-// be idle.
-sp_status batch_relayout(sp_batch* b, const std::vector<uint32_t>& cols_per_warp) {
+// be idle, with no learning pending.  derive: the permanences were written by
+// other means than the batch's own frames since the last layout.
+sp_status batch_relayout(sp_batch* b, const std::vector<uint32_t>& cols_per_warp,
+                         bool derive = false) {
   std::vector<uint32_t> cta_inst;
   uint32_t win_cap = 0;
   for (size_t i = 0; i < b->members.size(); ++i) {
@@ -2099,13 +2110,7 @@ sp_status batch_relayout(sp_batch* b, const std::vector<uint32_t>& cols_per_warp
     d.cta_first = (uint32_t)cta_inst.size();
     d.xspan = batch_xspan_cap() > 0u ? handle_xspan(h, d.n_ctas) : nullptr;
     uint32_t wb = 0;
-    if (d.worg && !window_rebands(h, &d, &wb) && handle_compact(h)) {
-      // the bands of this split do not fit: the compact form, derived from
-      // the permanences as they are now (the window form kept them current)
-      d.cidx = h->d_cidx;
-      d.cbase = h->d_cbase;
-      d.conn = h->d_cconn;
-    }
+    choose_form(h, &d, derive, &wb);
     win_cap = std::max(win_cap, wb);
     for (uint32_t c = 0; c < d.n_ctas; ++c) cta_inst.push_back((uint32_t)i);
   }
@@ -2320,9 +2325,10 @@ SP_API sp_status sp_batch_autotune(sp_batch* b, const uint32_t* d_frames, uint32
   }
   cudaStreamSynchronize(b->stream);
   if (d_keep) cudaFree(d_keep);
-  // the final split after the state is back, so that forms derived from the
-  // permanences (a compact form a split needs) derive from the kept ones
-  if (s == SP_OK) s = batch_relayout(b, cpw);
+  // the final split after the state is back, every form derived from it: a
+  // form that only a trial split took up follows what the tuning frames learnt
+  const sp_status sl = batch_relayout(b, cpw, true);
+  if (s == SP_OK) s = sl;
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
   if (s == SP_OK && cols_per_warp) {

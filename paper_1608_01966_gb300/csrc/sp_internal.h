@@ -77,9 +77,6 @@ uint32_t batch_stage_cap(uint32_t need);
 // the shared memory a CTA of this SP needs in the window form, 0 otherwise.
 void fill_desc(sp_handle* h, sp::BatchDesc* d, uint32_t cols_per_warp = 0,
                uint32_t* win_bytes = nullptr);
-// Recompute the window form's per-CTA frame bands for a new CTA split; false
-// (the descriptor then leaves the window form) if they no longer fit.
-bool window_rebands(sp_handle* h, sp::BatchDesc* d, uint32_t* win_bytes);
 uint32_t batch_xspan_cap();
 
 constexpr uint32_t kChunkFrames = 32;  // frames per staged chunk in sp_compute_frames
