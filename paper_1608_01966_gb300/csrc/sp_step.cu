@@ -238,16 +238,19 @@ __device__ __forceinline__ uint32_t column_overlap(const StepArgs& a, uint32_t c
 }
 
 // Alg. 2 over all overlaps, run by the last CTA.  This is the tail of every
-// frame's chain, so it makes one pass over the overlaps in L2 (kSelLoads of a
-// thread's loads in flight).  Where the overlaps are counts (unit boosts, or
-// found to be whole numbers up to S) they are counted into a histogram in
-// shared memory as they arrive, and every warp reads the k-th largest off it.
-// The ascending list is written only where someone can read it (a.list).  In a
-// full batch launch this takes about a quarter of the SP's chain: a warp gets
-// one issue in ten.  dyn: C overlaps, two sets of mask words, and S + 2 bins
+// frame's chain, so it makes one pass over the overlaps in L2, all of them in
+// flight to shared memory at once (a.ov is 16-byte aligned and padded to 16
+// bytes).  Where the overlaps are counts (unit boosts, or found to be whole
+// numbers up to S) they are counted into a histogram in shared memory, and
+// every warp reads the k-th largest off it.  The ascending list is written
+// only where someone can read it (a.list).  In a full batch launch this takes
+// about a quarter of the SP's chain: a warp gets one issue in ten.
+// us per frame of a kernel per frame, 256 x 148 / 1024 x 148 / 2116 x 148 / 4096 x
+// 256: 16 loads of a thread in registers at a time, each counted behind a
+// branch 6.7 / 7.4 / 10.0 / 12.4; as here 6.3 / 7.0 / 9.1 / 11.3.  Few loads and
+// little code matter: the code is cold in the last CTA of every frame.
+// dyn: C overlaps (rounded up to 4), two sets of mask words, and S + 2 bins
 // where S <= kStepBins.  Returns the mask words (shared memory).
-constexpr int kSelLoads = 16;
-
 __device__ const uint32_t* last_cta_inhibit(const StepArgs& a, uint32_t* dyn) {
   __shared__ uint32_t shist[256];
   __shared__ uint32_t sh[2 * kStepWarps];
@@ -255,41 +258,39 @@ __device__ const uint32_t* last_cta_inhibit(const StepArgs& a, uint32_t* dyn) {
   const uint32_t C = a.C;
   const uint32_t t = threadIdx.x;
   uint32_t* sv = dyn;
-  uint32_t* smask = sv + C;
+  uint32_t* smask = sv + ((C + 3u) & ~3u);
   uint32_t* stie = smask + a.mask_words;
   uint32_t* bins = stie + a.mask_words;
   const bool binned = a.inhibition == 0u && a.S <= kStepBins && !a.hist;
-  if (binned) {
+  for (uint32_t i = 4u * t; i < C; i += 4u * kStepThreads)
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(
+                     (uint32_t)__cvta_generic_to_shared(sv + i)),
+                 "l"(a.ov + i)
+                 : "memory");
+  if (binned)
     for (uint32_t b = t; b <= a.S; b += kStepThreads) bins[b] = 0u;
-    __syncthreads();
-  }
+  __syncthreads();
+  asm volatile("cp.async.wait_all;\n" ::: "memory");
   uint32_t nz = 0u, top = 0u;
   bool whole = true;  // every overlap of this thread is a count of at most S
-  for (uint32_t i0 = t; i0 < C; i0 += kStepThreads * kSelLoads) {
-    uint32_t v[kSelLoads];
+  // a thread reads what it copied, four overlaps before the first is counted
+  // (a load cannot pass the atomic before it)
+  for (uint32_t i = 4u * t; i < C; i += 4u * kStepThreads) {
+    const uint4 q = *reinterpret_cast<const uint4*>(sv + i);
+    const uint32_t v[4] = {q.x, i + 1u < C ? q.y : 0u, i + 2u < C ? q.z : 0u, i + 3u < C ? q.w : 0u};
+    uint32_t n[4];
 #pragma unroll
-    for (int j = 0; j < kSelLoads; ++j) {
-      const uint32_t i = i0 + (uint32_t)j * kStepThreads;
-      v[j] = i < C ? __float_as_uint(__ldcg(a.ov + i)) : 0u;
+    for (int j = 0; j < 4; ++j) {
+      const float f = __uint_as_float(v[j]);
+      n[j] = f <= (float)a.S ? __float2uint_rz(f) : 0u;
+      nz += v[j] != 0u;
+      whole = whole && __float_as_uint(__uint2float_rn(n[j])) == v[j];
+      top = max(top, n[j]);
     }
+    if (binned)
 #pragma unroll
-    for (int j = 0; j < kSelLoads; ++j) {
-      const uint32_t i = i0 + (uint32_t)j * kStepThreads;
-      if (i < C) sv[i] = v[j];
-      if (v[j] != 0u) {
-        ++nz;
-        if (binned) {
-          const float f = __uint_as_float(v[j]);
-          const uint32_t n = f <= (float)a.S ? __float2uint_rz(f) : 0u;
-          if (n != 0u && __uint2float_rn(n) == f) {
-            atomicAdd(bins + n, 1u);
-            top = max(top, n);
-          } else {
-            whole = false;
-          }
-        }
-      }
-    }
+      for (int j = 0; j < 4; ++j)
+        if (n[j] != 0u) atomicAdd(bins + n[j], 1u);
   }
   uint32_t total;
   if (a.inhibition == 0u) {
@@ -1078,7 +1079,7 @@ __global__ void __launch_bounds__(kStepThreads) sp_learn_kernel(const LearnArgs 
 
 size_t step_smem_bytes(uint32_t C, uint32_t S) {
   const uint32_t bins = S <= kStepBins ? S + 2u : 0u;
-  return ((size_t)C + 2u * ((C + 31u) / 32u) + bins) * sizeof(uint32_t);
+  return (((size_t)C + 3u) / 4u * 4u + 2u * ((C + 31u) / 32u) + bins) * sizeof(uint32_t);
 }
 
 int step_grid(uint32_t C) { return (int)((C + kStepWarps - 1) / kStepWarps); }
