@@ -318,6 +318,15 @@ sp_status wait_handle(sp_handle* h) {
   }
 }
 
+// A call on a capturing stream is recorded into the caller's graph: from then
+// on a replay that the handle does not see may have written the last frame's
+// list, so it is read from the device.
+void note_capture(sp_handle* h) {
+  cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
+  if (!h->captured && cudaStreamIsCapturing(h->stream, &status) == cudaSuccess)
+    h->captured = status != cudaStreamCaptureStatusNone;
+}
+
 // Order the handle's work on stream s after everything enqueued before.
 sp_status use_stream(sp_handle* h, cudaStream_t s) {
   if (!s) s = h->own_stream;
@@ -326,6 +335,7 @@ sp_status use_stream(sp_handle* h, cudaStream_t s) {
     SP_CUDA(cudaStreamWaitEvent(s, h->ev_switch, 0));
     h->stream = s;
   }
+  note_capture(h);
   return SP_OK;
 }
 
@@ -1085,7 +1095,7 @@ SP_API sp_status sp_active_columns(sp_handle* h, uint32_t* out, uint32_t cap, ui
   if (!h || !n || (!out && cap)) return fail(SP_EINVAL, "NULL argument");
   if (h->batch) return fail(SP_EBUSY, "the handle is a member of a batch");
   DeviceGuard g(h->device);
-  if (!h->host_result)
+  if (!h->host_result || h->captured)
     SP_CUDA(cudaMemcpyAsync(h->h_result, h->d_result, ((size_t)h->max_active + 1) * 4,
                             cudaMemcpyDeviceToHost, h->stream));
   sp_status s = wait_handle(h);

@@ -213,6 +213,7 @@ struct sp_handle {
   uint32_t run_gen = 0;             // bumped whenever d_run_ov / d_run_masks are reallocated
   bool unit_boost = true;
   bool host_result = false;      // the last frame wrote its list to h_result itself
+  bool captured = false;         // a call was recorded into a caller's graph
   uint32_t* h_result = nullptr;  // pinned [1 + C]; at creation [3][C], the pools' extents
   cudaStream_t own_stream = nullptr;
   cudaStream_t stream = nullptr;  // stream of the last call
