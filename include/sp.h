@@ -249,6 +249,16 @@ SP_API sp_status sp_sync(sp_handle* h);
  * the work running. */
 SP_API sp_status sp_set_timeout_ms(sp_handle* h, uint32_t ms);
 
+/* Bound, in nanoseconds of the GPU's global timer, of the waits inside a
+ * sequence launch (a CTA's wait for its part of a frame and for the other
+ * CTAs' counts of a frame): they end by themselves; if one has not ended
+ * within the bound, the launch stops early and the next waiting call returns
+ * SP_ETIMEOUT.  The frames from there on have no results, and the CTAs may
+ * have learnt one frame more or less than each other: restore the state or
+ * destroy the handle.  A bound below 1000 expires where there is anything to
+ * wait for.  0 restores the default of 1 s. */
+SP_API sp_status sp_set_device_wait_ns(sp_handle* h, uint64_t ns);
+
 /* ---- Batches of SPs ------------------------------------------------------
  *
  * The paper's 'Multiple HTMs' setup (Section 3, "Outer Structure") runs one

@@ -146,6 +146,7 @@ def lib():
         L.sp_set_boost.argtypes = [vp, _f32p]
         L.sp_sync.argtypes = [vp]
         L.sp_set_timeout_ms.argtypes = [vp, ct.c_uint32]
+        L.sp_set_device_wait_ns.argtypes = [vp, ct.c_uint64]
         L.sp_status_str.argtypes = [ct.c_int]
         L.sp_step_noalloc.argtypes = [ct.POINTER(SpConfig), vp, vp, vp, vp, ct.c_int, vp, vp, vp]
         L.sp_batch_create.argtypes = [ct.POINTER(vp), ct.c_uint32, ct.POINTER(vp)]
@@ -372,6 +373,10 @@ def sp_sync(h):
 
 def sp_set_timeout_ms(h, ms):
     _check(lib().sp_set_timeout_ms(h, ms), "sp_set_timeout_ms")
+
+
+def sp_set_device_wait_ns(h, ns):
+    _check(lib().sp_set_device_wait_ns(h, ns), "sp_set_device_wait_ns")
 
 
 def sp_step_noalloc(cfg, d_idx, d_perm, d_boost, d_input, learn, d_active_mask, d_active_list,

@@ -581,6 +581,7 @@ sp_status run_sequence(sp_handle* h, const uint32_t* x_base, uint32_t n, uint64_
     a.duty_period = h->cfg.duty_period;
     a.win_w = h->cfg.input_w;
     a.wpr = h->cfg.input_w / 32u;
+    a.wait_ns = h->wait_ns;
     a.err = h->h_err + 1;  // pinned host memory, written by the device as it is
     SP_CUDA(sp::launch_seq(a, h->seq_form, h->seq_Q, h->seq_smem, h->stream));
     h->pending = false;  // learning of every frame is already applied
@@ -1257,6 +1258,12 @@ SP_API sp_status sp_sync(sp_handle* h) {
 SP_API sp_status sp_set_timeout_ms(sp_handle* h, uint32_t ms) {
   if (!h) return fail(SP_EINVAL, "NULL handle");
   h->timeout_ms = ms ? ms : default_timeout_ms();
+  return SP_OK;
+}
+
+SP_API sp_status sp_set_device_wait_ns(sp_handle* h, uint64_t ns) {
+  if (!h) return fail(SP_EINVAL, "NULL handle");
+  h->wait_ns = ns ? ns : kDeviceWaitNs;
   return SP_OK;
 }
 

@@ -238,4 +238,5 @@ struct sp_handle {
   bool seq_ok = false;
   uint32_t seq_form = 0, seq_Q = 0, seq_Cq = 0, seq_band_max = 0;
   size_t seq_smem = 0;
+  uint64_t wait_ns = sp::rt::kDeviceWaitNs;  // bound of a sequence launch's waits
 };

@@ -263,6 +263,7 @@ struct SeqArgs {
   float* duty;                // [C] active-duty cycles, or nullptr
   float duty_period;
   uint32_t win_w, wpr;        // window forms: input_w and its words per row
+  uint64_t wait_ns;           // bound of every wait for a frame's band or counts
   uint32_t* err;              // mapped host word, set to 1 if a bounded wait expired
 };
 

@@ -57,10 +57,12 @@
 // only after it has received frame t+1's from everyone, and those are sent
 // after the sender is done with frame t's.
 //
-// Waits are bounded (1 s of %globaltimer): when one expires, the CTA records
-// it, the loop ends at the next CTA barrier, and every CTA reaches the cluster
-// barrier at the end (the others after their own limit), so no CTA leaves
-// while another may still write to its shared memory.
+// Waits are bounded (a.wait_ns of %globaltimer, 1 s by default): when one
+// expires, the CTA learns nothing from that frame and its loop ends at the next
+// B1.  Every CTA reaches the cluster barrier at the end (the others after their
+// own limit).  There each CTA tells how many frames' counts it has sent, so one
+// that gave up knows what is still on its way to its shared memory and waits
+// for just that before it leaves.
 #include <cooperative_groups.h>
 
 #include <algorithm>
@@ -84,7 +86,7 @@ using dev::learn_one;
 constexpr uint32_t kSeqWarps = kSeqThreads / 32;   // compute warps
 constexpr uint32_t kSeqHelpers = 128;              // threads of the helper warps
 constexpr int kSeqCols = 4;   // window forms: columns a warp counts side by side
-constexpr unsigned long long kSeqWaitNs = 1000000000ull;
+constexpr unsigned long long kSeqDrainNs = 1000000000ull;  // bound of drain_counts' waits
 constexpr uint32_t kBoxWords = 128;  // bitmap words of a 64 x 64 box
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) {
@@ -108,13 +110,23 @@ __device__ __forceinline__ void mbar_expect(uint64_t* bar, uint32_t bytes) {
                : "memory");
 }
 
-// Wait (bounded) for the phase with this parity; with CLUSTER, what other CTAs
-// of the cluster sent with it is visible after.
-template <bool CLUSTER>
-__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity) {
+// Wait (at most about `ns`; ONCE: only look) for the phase with this parity;
+// with CLUSTER, what other CTAs of the cluster sent with it is visible after.
+template <bool CLUSTER, bool ONCE = false>
+__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, unsigned long long ns) {
+  uint32_t ok;
+  if (ONCE) {
+    asm volatile(
+        "{\n.reg .pred p;\n"
+        "mbarrier.test_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n"
+        "selp.b32 %0, 1, 0, p;\n}\n"
+        : "=r"(ok)
+        : "r"(smem_u32(bar)), "r"(parity)
+        : "memory");
+    return ok != 0u;
+  }
   unsigned long long t0 = 0;
   for (uint32_t i = 0;; ++i) {
-    uint32_t ok;
     if (CLUSTER)
       asm volatile(
           "{\n.reg .pred p;\n"
@@ -136,7 +148,7 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity) {
       const unsigned long long t = now_ns();
       if (i == 0u)
         t0 = t;
-      else if (t - t0 > kSeqWaitNs)
+      else if (t - t0 > ns)
         return false;
     }
   }
@@ -185,6 +197,49 @@ __device__ __forceinline__ void compute_sync() {
   asm volatile("bar.sync 2, %0;\n" ::"n"(kSeqThreads) : "memory");
 }
 
+// What the other CTAs of the cluster still send to a CTA whose wait for counts
+// gave up, by one of its warps: it sent *sent frames' counts (`bytes` each to
+// every other CTA), and its barriers expect as many from every other; those
+// were waited for but the last.  A CTA sends a frame's counts after it has
+// everyone's of the frame before, so the others sent one frame less, as many,
+// or one more.  (Shared-memory addresses and a loop over the two barriers: as
+// pointers and straight code this cost the loop over the frames 2 %.)
+__device__ __forceinline__ void drain_counts(uint32_t cnt_bar, uint32_t sent, uint32_t bytes) {
+  uint32_t n, m, Q;
+  asm volatile("ld.shared.u32 %0, [%1];\n" : "=r"(n) : "r"(sent) : "memory");
+  asm volatile("mov.u32 %0, %%cluster_nctaid.x;\n" : "=r"(Q));
+  const uint32_t lane = threadIdx.x & 31u;
+  const bool peer = lane < Q;  // at most kSeqMaxCluster
+  asm volatile("ld.shared::cluster.u32 %0, [%1];\n"
+               : "=r"(m)
+               : "r"(peer_addr(sent, peer ? lane : 0u))
+               : "memory");
+  const uint32_t fewer = __popc(__ballot_sync(kFull, peer && m < n));
+  const uint32_t more = __popc(__ballot_sync(kFull, peer && m > n));
+  if (lane != 0u) return;
+  for (uint32_t k = 0; k < 2u; ++k) {  // frames n - 1 and n
+    if (k ? more == 0u : n == 0u) continue;
+    const uint32_t f = n + k - 1u, bar = cnt_bar + 8u * (f & 1u), miss = (k ? more : fewer) * bytes;
+    if (k)  // not armed yet: what is on its way
+      asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(bar), "r"(miss)
+                   : "memory");
+    else if (miss)  // armed for everyone's: less what nobody will send
+      asm volatile("mbarrier.complete_tx.relaxed.cluster.shared::cta.b64 [%0], %1;\n" ::"r"(bar),
+                   "r"(miss)
+                   : "memory");
+    const unsigned long long t0 = now_ns();
+    uint32_t ok = 0u;
+    while (!ok && now_ns() - t0 < kSeqDrainNs)
+      asm volatile(
+          "{\n.reg .pred p;\n"
+          "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n"
+          "selp.b32 %0, 1, 0, p;\n}\n"
+          : "=r"(ok)
+          : "r"(bar), "r"((f >> 1) & 1u)
+          : "memory");
+  }
+}
+
 // Words of one frame's histogram: bins 0..S, bin 0 the largest count.
 __host__ __device__ __forceinline__ uint32_t hist_words(uint32_t S) { return (S + 4u) & ~3u; }
 
@@ -230,7 +285,10 @@ struct IntC {
   static constexpr int value = N;
 };
 
-template <uint32_t FORM>
+// ONCE: a bound of less than a microsecond, which the clock may not resolve, is
+// no wait at all; its own instance, since a choice between two mbarrier
+// instructions in the chain of a frame took 3 % (1024 x 256).
+template <uint32_t FORM, bool ONCE>
 __global__ void __launch_bounds__(kSeqThreads + kSeqHelpers, 1) sp_seq_cluster_kernel(const SeqArgs a) {
   constexpr bool kWindow = FORM != kSeqPools;
   constexpr bool kPermSmem = FORM != kSeqWindowL2;
@@ -238,6 +296,8 @@ __global__ void __launch_bounds__(kSeqThreads + kSeqHelpers, 1) sp_seq_cluster_k
   cg::cluster_group cluster = cg::this_cluster();
   extern __shared__ __align__(16) uint32_t sm[];
   __shared__ uint32_t sh[2 * kSeqWarps];
+  // non-unit boosts: select_threshold's; else [0] is set once a wait has given
+  // up, [1] is the number of frames whose counts this CTA has sent
   __shared__ uint32_t s2[2];
   __shared__ uint32_t s_n;                 // winners listed in this frame
   __shared__ uint16_t s_list[kSeqThreads];  // their columns in this CTA
@@ -285,6 +345,7 @@ __global__ void __launch_bounds__(kSeqThreads + kSeqHelpers, 1) sp_seq_cluster_k
   // ---- prologue: barriers, this CTA's state and input band -------------------
   if (t == 0) {
     s_n = 0u;
+    s2[0] = s2[1] = 0u;
     mbar_init(&s_band_bar[0], kSeqHelpers);
     mbar_init(&s_band_bar[1], kSeqHelpers);
     mbar_init(&s_cnt_bar[0], 1);
@@ -455,7 +516,10 @@ __global__ void __launch_bounds__(kSeqThreads + kSeqHelpers, 1) sp_seq_cluster_k
         if (fast) break;
       }
       const uint32_t h = t - kSeqThreads;
-      if (fast && Q > 1u && h == 0u) mbar_expect(&s_cnt_bar[par], (Q - 1u) * Cq * 2u);
+      if (fast && Q > 1u && h == 0u) {
+        mbar_expect(&s_cnt_bar[par], (Q - 1u) * Cq * 2u);
+        s2[1] = f + 1u;
+      }
       if (f + 1u < a.n_frames)
         copy_band(s_band + (par ^ 1u) * a.band_max, a.frames + (uint64_t)(f + 1u) * a.stride + w_lo,
                   brows, blen, pitch, &s_band_bar[par ^ 1u]);
@@ -530,7 +594,7 @@ __global__ void __launch_bounds__(kSeqThreads + kSeqHelpers, 1) sp_seq_cluster_k
       uint32_t* hist = sm + L.hist + slot * hw;
       uint32_t* smask_f = sm + L.mask + slot * mw;
       float* ov_pub = reinterpret_cast<float*>(sm + L.ov) + par * Cq;
-      if (ok) ok = mbar_wait<false>(&s_band_bar[par], phase);
+      if (ok) ok = mbar_wait<false, ONCE>(&s_band_bar[par], phase, a.wait_ns);
 
       // ---- Alg. 1 for this warp's columns ---------------------------------------
       // every load of a step is issued before its first use: no branch
@@ -678,7 +742,8 @@ __global__ void __launch_bounds__(kSeqThreads + kSeqHelpers, 1) sp_seq_cluster_k
             for (uint32_t u = lane; u < Cq / 8u; u += 32u)
               send16(dst + u * 16u, reinterpret_cast<const uint4*>(s_cnt + c0)[u], bar);
           }
-          if (ok) ok = mbar_wait<true>(&s_cnt_bar[par], phase);
+          if (ok) ok = mbar_wait<true, ONCE>(&s_cnt_bar[par], phase, a.wait_ns);
+          if (!ok) atomicSub(&s_n, 1u << 20);  // read as below 0: nothing is learnt from it
         }
         if (global) {
           if (Q > 1u) {
@@ -832,7 +897,7 @@ __global__ void __launch_bounds__(kSeqThreads + kSeqHelpers, 1) sp_seq_cluster_k
           uint32_t at = 0u;
           if (lane == 0u) at = atomicAdd(&s_n, (uint32_t)__popc(w));
           at = __shfl_sync(kFull, at, 0) + __popc(w & ((1u << lane) - 1u));
-          if ((w >> lane) & 1u) s_list[at] = (uint16_t)lc;
+          if ((w >> lane) & 1u) s_list[at & (kSeqThreads - 1u)] = (uint16_t)lc;
         }
       }
       if (!a.learn) continue;
@@ -840,7 +905,7 @@ __global__ void __launch_bounds__(kSeqThreads + kSeqHelpers, 1) sp_seq_cluster_k
       // ---- learning: the listed winners' synapses, 32 J of one column a unit,
       // units dealt to the warps; a unit's loads are issued before the first is
       // used.  Few winners: small units, so that their chains are short
-      const uint32_t n_win = s_n;
+      const uint32_t n_win = (uint32_t)max((int)s_n, 0);
       auto learn = [&](auto jc, uint32_t parts, float inv_parts) {
         constexpr int J = decltype(jc)::value;
         const uint32_t units = n_win * parts;
@@ -912,13 +977,8 @@ __global__ void __launch_bounds__(kSeqThreads + kSeqHelpers, 1) sp_seq_cluster_k
     }
   }
   if (!ok) {
-    // a wait gave up: report it, and wait (bounded) for what may still be on
-    // its way into this CTA's shared memory
+    s2[0] = 1u;
     if (a.err) atomicExch(a.err, 1u);
-    if (!helper && fast && Q > 1u && f < a.n_frames) {
-      if (t == 0) mbar_expect(&s_cnt_bar[f & 1u], (Q - 1u) * Cq * 2u);
-      mbar_wait<true>(&s_cnt_bar[f & 1u], (f >> 1) & 1u);
-    }
   }
   asm volatile("cp.async.wait_all;\n" ::: "memory");
   __syncthreads();
@@ -945,7 +1005,8 @@ __global__ void __launch_bounds__(kSeqThreads + kSeqHelpers, 1) sp_seq_cluster_k
       for (uint32_t s = lane; s < S; s += 32) gp[s] = s_perm[lc * S + s];
     }
   }
-  cluster.sync();  // every CTA's mask of the last frame is final
+  cluster.sync();  // every CTA's mask of the last frame is final, and its last counts are sent
+  if (warp == kSeqWarps && s2[0] && fast) drain_counts(smem_u32(s_cnt_bar), smem_u32(&s2[1]), Cq * 2u);
   if (q == 0u && warp == 0u) {
     // ascending list of the last frame's winners, 32 mask words at a time
     uint32_t total = 0u;
@@ -1007,10 +1068,11 @@ __global__ void __launch_bounds__(256) sp_pool_scan_kernel(const uint32_t* idx, 
 
 using SeqKernel = void (*)(const SeqArgs);
 
+template <bool ONCE>
 SeqKernel seq_kernel(uint32_t form) {
-  return form == kSeqPools ? sp_seq_cluster_kernel<kSeqPools>
-                           : (form == kSeqWindow ? sp_seq_cluster_kernel<kSeqWindow>
-                                                 : sp_seq_cluster_kernel<kSeqWindowL2>);
+  return form == kSeqPools ? sp_seq_cluster_kernel<kSeqPools, ONCE>
+                           : (form == kSeqWindow ? sp_seq_cluster_kernel<kSeqWindow, ONCE>
+                                                 : sp_seq_cluster_kernel<kSeqWindowL2, ONCE>);
 }
 
 }  // namespace
@@ -1028,10 +1090,13 @@ size_t seq_smem_bytes(uint32_t form, uint32_t Q, uint32_t C, uint32_t S, uint32_
 }
 
 cudaError_t seq_kernel_init(uint32_t form, size_t smem_bytes) {
-  const SeqKernel k = seq_kernel(form);
-  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-  if (e != cudaSuccess) return e;
-  return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes);
+  for (const SeqKernel k : {seq_kernel<false>(form), seq_kernel<true>(form)}) {
+    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes);
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
 }
 
 cudaError_t seq_max_active_clusters(uint32_t form, uint32_t Q, size_t smem_bytes, int* out) {
@@ -1046,7 +1111,7 @@ cudaError_t seq_max_active_clusters(uint32_t form, uint32_t Q, size_t smem_bytes
   attr[0].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaOccupancyMaxActiveClusters(out, seq_kernel(form), &cfg);
+  return cudaOccupancyMaxActiveClusters(out, seq_kernel<false>(form), &cfg);
 }
 
 cudaError_t launch_seq(const SeqArgs& a, uint32_t form, uint32_t Q, size_t smem_bytes,
@@ -1063,7 +1128,7 @@ cudaError_t launch_seq(const SeqArgs& a, uint32_t form, uint32_t Q, size_t smem_
   attr[0].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  const cudaError_t e = cudaLaunchKernelEx(&cfg, seq_kernel(form), a);
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, a.wait_ns < 1000u ? seq_kernel<true>(form) : seq_kernel<false>(form), a);
   g_launches.fetch_add(1, std::memory_order_relaxed);
   return e;
 }
