@@ -154,9 +154,18 @@ void plan_cluster_path(sp_handle* h, const uint32_t* scan) {
   const uint32_t *lo = scan, *hi = scan + h->C, *row = scan + 2u * h->C;
   const bool boxes = std::find(row, row + h->C, 0xffffffffu) == row + h->C;
   uint32_t Q = std::min((h->C + 31u) / 32u, sp::kSeqMaxCluster);
-  // small SPs: one CTA counts them in less time than a cluster exchanges counts
-  if (h->C <= (uint32_t)sp::kSeqThreads && (uint64_t)h->C * h->S <= kSeqOneCtaSynapses &&
-      h->n_words <= kSeqOneCtaWords)
+  // small SPs: one CTA counts them in less time than a cluster exchanges
+  // counts, as long as its warps pass over their columns no more than twice, or
+  // the cluster would have two CTAs.  us per frame, one CTA / cluster (passes of
+  // the one CTA in parentheses): 64 x 26 (4) 2.14 / 2.48, 64 x 90 (4) 2.44 / 2.63,
+  // 100 x 16 (2) 2.40 / 2.69, 100 x 48 (4) 2.86 / 2.65, 128 x 32 (2) 2.44 / 2.67, 160 x
+  // 26 (10) 3.10 / 2.58, 185 x 32 (3) 2.91 / 2.71, 256 x 16 (2) 2.54 / 2.76, 256 x 32
+  // (4) 2.97 / 2.71, 320 x 8 (3) 2.74 / 2.70, 400 x 20 (7) 4.22 / 2.83, 512 x 16 (4)
+  // 3.36 / 2.87; of 12 frames 185 x 32 45.7 / 40.4 in all, 256 x 16 41.6 / 39.6.
+  const uint32_t all = (h->C + 31u) & ~31u;
+  const uint32_t step = (uint32_t)sp::kSeqThreads / 32u << sp::seq_pool_groups(h->S, all);
+  if (all <= (uint32_t)sp::kSeqThreads && (uint64_t)h->C * h->S <= kSeqOneCtaSynapses &&
+      h->n_words <= kSeqOneCtaWords && (Q <= 2u || (all + step - 1u) / step <= 2u))
     Q = 1u;
   const uint32_t Cq = (((h->C + Q - 1u) / Q) + 31u) & ~31u;
   if (Cq > (uint32_t)sp::kSeqThreads) return;  // a warp's columns are a 32-bit mask

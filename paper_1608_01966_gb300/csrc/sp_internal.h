@@ -92,10 +92,9 @@ constexpr uint32_t kSeqMinFrames = 3;
 constexpr uint32_t kSeqMinFramesL2 = 5;
 constexpr uint32_t kSeqLocalColumns = 512;  // fewer are ranked fast enough by one CTA
 // Sequences of SPs of at most so many synapses, on frames of at most so many
-// words, run in one CTA instead of a cluster, us per frame: 256 x 16 2.02
-// against 2.56, 512 x 16 2.51 / 2.65, 256 x 32 2.62 / 2.74, but 256 x 64 3.66 /
-// 2.75; and a lone CTA that must copy all 16,200 words of a 960 x 540 frame
-// takes 4.2 where a cluster, a band each, takes 2.8 (256 x 32).
+// words, may run in one CTA instead of a cluster (plan_cluster_path); a lone
+// CTA that must copy all 16,200 words of a 960 x 540 frame takes 4.2 us a frame
+// where a cluster, a band each, takes 2.8 (256 x 32).
 constexpr uint64_t kSeqOneCtaSynapses = 8192;
 constexpr uint32_t kSeqOneCtaWords = 2048;
 // Pools of at least so many synapses count faster as bitmaps (the pools' cost

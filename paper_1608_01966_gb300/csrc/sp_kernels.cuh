@@ -239,6 +239,21 @@ constexpr uint32_t kSeqMaxCluster = 16;
 // permanences stay in global memory).
 enum : uint32_t { kSeqPools = 0u, kSeqWindow = 1u, kSeqWindowL2 = 2u };
 
+// log2 of the columns that a warp counts side by side in the pools form, of a
+// CTA's Cq columns of S synapses.  More than one share the warp's lanes where
+// a pool has few loads to give, so that a warp needs fewer passes over its
+// columns; but their sums take shuffles where a column of the whole warp takes
+// one reduction, so only until two passes remain: us per frame with as many as
+// fit / as here, cluster of 256 x 32 2.79 / 2.70, 128 x 48 2.74 / 2.63, 32 x 16 2.29 /
+// 2.17; equal where passes remain (2000 x 16 3.37 / 3.42).
+__host__ __device__ inline uint32_t seq_pool_groups(uint32_t S, uint32_t Cq) {
+  const uint32_t warps = (uint32_t)kSeqThreads / 32u;
+  const uint32_t units = (S & 3u) == 0u ? S >> 2 : S;  // lane loads of one pool
+  uint32_t lp = 0u;
+  while (lp < 3u && Cq > (2u * warps << lp) && (units << (lp + 1u)) <= 32u) ++lp;
+  return lp;
+}
+
 struct SeqArgs {
   const uint32_t* idx;        // [C][S]
   float* perm;                // [C][S], rows that learned are written back at the end

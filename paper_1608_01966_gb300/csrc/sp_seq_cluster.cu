@@ -330,11 +330,7 @@ __global__ void __launch_bounds__(kSeqThreads + kSeqHelpers, 1) sp_seq_cluster_k
   // Column ownership of the count.  A warp counts P columns side by side,
   // L32 = 32 / P lanes each (pools of a few synapses); its i-th own column is
   //   lc = ((i / P) * kSeqWarps + warp) * P + i % P,   i < own.
-  uint32_t lp = 0u;  // log2 P
-  if (!kWindow) {
-    const uint32_t units = (S & 3u) == 0u ? S >> 2 : S;  // lane loads of one pool
-    while (lp < 3u && (units << (lp + 1u)) <= 32u && (kSeqWarps << (lp + 1u)) <= Cq) ++lp;
-  }
+  const uint32_t lp = kWindow ? 0u : seq_pool_groups(S, Cq);  // log2 P
   const uint32_t P = 1u << lp, ll = 5u - lp, L32 = 1u << ll;
   const uint32_t passes = (Cq + (kSeqWarps << lp) - 1u) / (kSeqWarps << lp);
   const uint32_t own = passes << lp;  // at most 32 (Cq <= kSeqThreads)
