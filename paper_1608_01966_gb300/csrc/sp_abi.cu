@@ -441,10 +441,9 @@ sp_status enqueue_sequence(sp_handle* h, cudaStream_t st, const uint32_t* x_base
 
 // Whether n frames run in one cluster launch.
 bool use_cluster(const sp_handle* h, uint32_t n) {
-  const uint32_t least =
-      h->cfg.inhibition == SP_INHIBIT_LOCAL && h->C >= kSeqLocalColumns
-          ? 1u
-          : (h->seq_form == sp::kSeqWindowL2 ? kSeqMinFramesL2 : kSeqMinFrames);
+  uint32_t least = h->seq_form == sp::kSeqWindowL2 ? kSeqMinFramesL2 : kSeqMinFrames;
+  if (h->cfg.inhibition == SP_INHIBIT_LOCAL && h->C >= kSeqLocalColumns)
+    least = local_frame_in_cluster(h->C, h->S, h->cfg.min_overlap) ? 1u : 2u;
   return h->seq_ok && n >= least && seq_enabled();
 }
 

@@ -84,13 +84,29 @@ constexpr int kSlots = 2;
 constexpr uint32_t kGraphMinFrames = 4;  // shorter sequences are launched directly
 // Sequences of at least so many frames run in one cluster launch, fewer as one
 // kernel per frame (us, cluster / per frame: 1024 x 256 1 frame 19.7 / 10.4, 2
-// 22.7 / 20.7, 3 24.8 / 30.9; 256 x 16 2 16.4 / 15.5, 3 17.9 / 23.8).  With local
-// inhibition a single frame already: the per-frame kernel ranks all columns in
-// its last CTA (4096 x 64: 20.6 / 63.7).  Building the bitmaps of an SP that
-// large takes longer (4096 x 256 4 57.8 / 54.9, 6 68.2 / 80.9).
+// 22.7 / 20.7, 3 24.8 / 30.9; 256 x 16 2 16.4 / 15.5, 3 17.9 / 23.8).  Building the
+// bitmaps of an SP that does not fit otherwise takes longer (4096 x 256 4 57.8 /
+// 54.9, 6 68.2 / 80.9).  With local inhibition two frames already, and often one
+// (local_frame_in_cluster): the per-frame kernel ranks all columns in its last
+// CTA.
 constexpr uint32_t kSeqMinFrames = 3;
 constexpr uint32_t kSeqMinFramesL2 = 5;
 constexpr uint32_t kSeqLocalColumns = 512;  // fewer are ranked fast enough by one CTA
+
+// Whether a single frame with local inhibition runs in the cluster kernel.  The
+// per-frame kernel ranks only columns that reach the minimum overlap m, so what
+// it takes depends on how many do, and on C.  us per sp_compute, cluster / per
+// frame, blobbed frames of 5-20 % density: 529 x 16 m 1 37.7 / 40.1, m 2 37.4 / 38.6,
+// m 4 35.7 / 28.0; 529 x 32 m 4 37.6 / 35.3, 529 x 64 m 4 37.4 / 39.6, m 8 37.7 / 32.1;
+// 1024 x 16 m 4 37.6 / 30.9, 1024 x 32 m 4 37.5 / 40.2, 1024 x 64 m 8 37.5 / 35.5, 1024
+// x 128 m 8 38.2 / 44.2; 2025 x 16 m 4 37.7 / 38.1, 2025 x 40 m 8 38.0 / 31.6, 2025 x 64
+// m 8 38.2 / 46.5; 4096 x 16 m 4 38.5 / 52.4, m 8 39.0 / 28.5, 4096 x 40 m 8 40.4 / 36.8,
+// 4096 x 64 m 8 43.1 / 66.2, 4096 x 128 m 16 58.7 / 49.7, 4096 x 256 m 16 70.9 / 94.3:
+// the line lies near S = m^2, and higher where there are fewer columns to rank.
+inline bool local_frame_in_cluster(uint32_t C, uint32_t S, uint32_t m) {
+  return S >= 16u && S >= (C < 1024u ? 3u : (C < 1536u ? 2u : 1u)) * (uint64_t)m * m;
+}
+
 // Sequences of SPs of at most so many synapses, on frames of at most so many
 // words, may run in one CTA instead of a cluster (plan_cluster_path); a lone
 // CTA that must copy all 16,200 words of a 960 x 540 frame takes 4.2 us a frame
