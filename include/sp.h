@@ -638,12 +638,13 @@ SP_API sp_status sp_encode_compute(sp_encoder* e, sp_handle* h, const uint8_t* h
  * against a fixed device-memory budget, or owns every allocation itself, and
  * so cannot let the library grow its footprint.
  *
- * The kernel's scratch (C boosted overlaps and ticket counters) lives in a
+ * The kernel's scratch (C boosted overlaps and a ticket counter) lives in a
  * static device array of SP_NOALLOC_SCRATCH_BYTES inside the library, which
  * every GPU that loads the library holds until the process exits.  Every call
- * shares that array and it keeps the last call's contents, so calls whose work overlaps on a GPU
- * -- different streams, or different threads without ordering -- race and
- * give wrong results: order them, e.g. all on one stream.
+ * shares that array and it keeps the last call's contents (the counter starts
+ * anew in every call and every replay of a recorded one), so calls whose work
+ * overlaps on a GPU -- different streams, or different threads without
+ * ordering -- race and give wrong results: order them, e.g. all on one stream.
  *
  * Every call looks up the array's device address in the current device's
  * context (a lookup that allocates nothing), so a device reset between calls

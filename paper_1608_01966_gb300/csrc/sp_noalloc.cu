@@ -26,13 +26,15 @@
 namespace {
 
 // [0, SP_NOALLOC_MAX_COLUMNS): boosted overlaps of the current call;
-// [SP_NOALLOC_MAX_COLUMNS .. + 1]: two last-CTA ticket counters, used by calls
-// in turn.  A call leaves its own at zero and its kernel clears the other one
-// first, so that a counter left wrong by calls that raced does not last; with
-// one counter, clearing it took a memset node of 1.5 us before every kernel.
+// [SP_NOALLOC_MAX_COLUMNS .. + 1]: the last-CTA ticket word.  Each call counts its
+// tickets from a base above every earlier call's, so whatever calls that raced
+// left there does not matter to the next one; clearing a plain counter took a
+// memset of 1.5 us before every kernel.  A call recorded into a graph carries
+// one base for all its replays and has the memset.
 constexpr uint32_t kScratchWords = SP_NOALLOC_MAX_COLUMNS + 64u;
 static __device__ __align__(256) uint32_t g_noalloc_scratch[kScratchWords];
-std::atomic<uint32_t> g_turn{0};
+constexpr uint32_t kTicketBits = 16;  // a grid has at most SP_NOALLOC_MAX_COLUMNS / 4 CTAs
+std::atomic<uint64_t> g_calls{0};
 
 constexpr size_t kPlainSmem = 44u << 10;  // less the step kernel's static shared memory
 
@@ -91,8 +93,11 @@ SP_API sp_status sp_step_noalloc(const sp_config* cfg, const uint32_t* d_idx, fl
   sp_status s = scratch_address(&scratch, sp::step_smem_bytes(C, S));
   if (s != SP_OK) return s;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  const uint32_t turn = g_turn.fetch_add(1, std::memory_order_relaxed) & 1u;
-  uint32_t* counter = scratch + SP_NOALLOC_MAX_COLUMNS + turn;
+  auto* ticket = reinterpret_cast<unsigned long long*>(scratch + SP_NOALLOC_MAX_COLUMNS);
+  cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(st, &capture) != cudaSuccess || capture != cudaStreamCaptureStatusNone)
+    if (cudaMemsetAsync(ticket, 0, sizeof(*ticket), st) != cudaSuccess)
+      return noalloc_fail(SP_ECUDA, "clearing the scratch counter failed");
 
   sp::StepArgs a{};
   a.idx = d_idx;
@@ -103,8 +108,8 @@ SP_API sp_status sp_step_noalloc(const sp_config* cfg, const uint32_t* d_idx, fl
   a.mask_out = d_active_mask;
   a.result = d_active_list;
   a.list = 1u;
-  a.counter = counter;
-  a.counter_clear = scratch + SP_NOALLOC_MAX_COLUMNS + (turn ^ 1u);
+  a.ticket = ticket;
+  a.ticket_base = (g_calls.fetch_add(1, std::memory_order_relaxed) + 1u) << kTicketBits;
   a.C = C;
   a.S = S;
   a.n_words = (uint32_t)((n_in + 31) / 32);

@@ -946,13 +946,24 @@ __device__ __forceinline__ void step_body(const StepArgs& a, uint32_t bid, uint3
   __syncthreads();
   if (threadIdx.x == 0) {
     __threadfence();
-    s_ticket = atomicAdd(a.counter, 1u);
+    if (a.ticket) {
+      // both by this thread on one word, so in this order
+      atomicMax(a.ticket, a.ticket_base);
+      s_ticket = (uint32_t)(atomicAdd(a.ticket, 1ull) - a.ticket_base);
+    } else {
+      s_ticket = atomicAdd(a.counter, 1u);
+    }
   }
   __syncthreads();
   if (s_ticket != nb - 1u) return;
   __threadfence();
   const uint32_t* smask = last_cta_inhibit(a, dyn_smem);
-  if (threadIdx.x == 0) atomicExch(a.counter, 0u);
+  if (threadIdx.x == 0) {
+    if (a.ticket)
+      atomicExch(a.ticket, 0ull);
+    else
+      atomicExch(a.counter, 0u);
+  }
   if (done) {
     // release this frame's results (mask, list, reset counter and
     // histogram) to the CTAs of the SP's next frame in the same launch
@@ -969,7 +980,6 @@ __device__ __forceinline__ void step_body(const StepArgs& a, uint32_t bid, uint3
 template <int VEC>
 __global__ void __launch_bounds__(kStepThreads) sp_step_kernel(const StepArgs a) {
   extern __shared__ __align__(128) uint32_t dyn_smem[];
-  if (a.counter_clear && blockIdx.x == 0u && threadIdx.x == 0u) *a.counter_clear = 0u;
   step_body<VEC, false>(a, blockIdx.x, gridDim.x, dyn_smem);
 }
 
@@ -1030,6 +1040,7 @@ __global__ void __launch_bounds__(kStepThreads, SP_BATCH_MIN_BLOCKS) sp_batch_st
   a.ov_copy = (ba.ov_out && !ba.tick) ? ba.ov_out + d.ov_off : nullptr;
   a.result = d.result;
   a.counter = d.counter;
+  a.ticket = nullptr;
   a.hist = d.hist;
   a.duty = d.duty;
   a.duty_period = d.duty_period;
@@ -1171,6 +1182,7 @@ __global__ void __launch_bounds__(kStepThreads, MINB) sp_batch_run_kernel(const 
     a.ov_copy = r.ov_out ? r.ov_out + (uint64_t)t * r.ov_stride + d.ov_off : nullptr;
     a.result = d.result;
     a.counter = d.counter;
+    a.ticket = nullptr;
     a.hist = d.hist;
     a.duty = d.duty;
     a.duty_period = d.duty_period;
