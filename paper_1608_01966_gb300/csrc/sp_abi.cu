@@ -2001,6 +2001,16 @@ SP_API sp_status sp_batch_infer_overlaps_device(sp_batch* b, const uint32_t* d_f
     max_S = std::max(max_S, f.unit_S);
     all_global = all_global && f.inhibition == 0u;
   }
+  // a launch has room for the most columns and the largest histogram of any
+  // member: members whose histogram is too large for that go without one
+  while (max_S != 0u && sp::frame_inhibit_smem(max_C, max_S) > sp::frame_inhibit_smem_limit()) {
+    uint32_t next = 0u;
+    for (sp::FrameInhibitArgs& f : fargs) {
+      if (f.unit_S == max_S) f.unit_S = 0u;
+      next = std::max(next, f.unit_S);
+    }
+    max_S = next;
+  }
   if (sp::frame_inhibit_smem(max_C, max_S) > sp::frame_inhibit_smem_limit())
     return fail(SP_ENOTSUP, "members too large for one per-frame inhibition launch");
   const size_t arg_bytes = (sizeof(sp::DenseArgs) + sizeof(sp::FrameInhibitArgs)) * n;
