@@ -303,7 +303,7 @@ SP_API sp_status sp_batch_get_info(const sp_batch* b, sp_batch_info* out);
  * as for sp_batch_compute_device, stride in words) three times per candidate
  * and keep the fastest, in three steps:
  *   1. one CTA split for every member: each member's default, or 4 warps x
- *      {2, 4, 8, 16} columns per warp;
+ *      {2, 4, 8, 16, 32} columns per warp;
  *   2. the compiled schedule of the persistent pass (resident CTAs per SM,
  *      which sets each thread's register budget, x columns per warp in
  *      flight; sp_batch_schedule reports the choice);

@@ -2297,7 +2297,7 @@ SP_API sp_status sp_batch_autotune(sp_batch* b, const uint32_t* d_frames, uint32
   s = batch_relayout(b, cpw);
   float best_ms = 0.0f;
   if (s == SP_OK) s = time_layout(&best_ms);
-  const uint32_t candidates[] = {2u, 4u, 8u, 16u};
+  const uint32_t candidates[] = {2u, 4u, 8u, 16u, 32u};
   // 1. one split for every member
   uint32_t uniform = 0u;
   for (uint32_t c : candidates) {
@@ -2337,7 +2337,7 @@ SP_API sp_status sp_batch_autotune(sp_batch* b, const uint32_t* d_frames, uint32
   for (uint32_t k : order) {
     if (order.size() < 2u) break;  // one bucket: step 1 has tried its splits
     uint32_t keep = uniform;
-    for (uint32_t c : {0u, 2u, 4u, 8u, 16u}) {
+    for (uint32_t c : {0u, 2u, 4u, 8u, 16u, 32u}) {
       if (s != SP_OK || c == uniform) continue;
       std::vector<uint32_t> trial = cpw;
       for (size_t i = 0; i < n; ++i)
