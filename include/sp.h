@@ -539,7 +539,9 @@ SP_API sp_status sp_server_submit_many_device(sp_server* s, uint32_t n, const ui
                                               void* stream);
 
 /* Take up to max_results finished frames (oldest first), their active lists
- * copied into active[0..active_cap); waits up to wait_ms for the first one.
+ * copied into active[0..active_cap); waits up to wait_ms for the first one
+ * (while frames are outstanding, one of the waiting threads yields for up to
+ * 0.1 ms before it sleeps, as the server's worker does after every request).
  * *n_results may be 0.  Results whose lists do not fit stay queued. */
 SP_API sp_status sp_server_poll(sp_server* s, sp_server_result* results, uint32_t max_results,
                                 uint32_t* active, uint32_t active_cap, uint32_t* n_results,

@@ -94,6 +94,7 @@ struct sp_server {
   // requests published and results delivered so far: what the worker and a
   // waiting poll watch for a moment before they sleep
   std::atomic<uint64_t> published{0}, delivered{0};
+  std::atomic<bool> poll_spins{false};  // one waiting poll at a time
   std::vector<Stream> streams;
   sp::BatchDesc* d_desc = nullptr;
   cudaStream_t copy_stream = nullptr;
@@ -247,6 +248,7 @@ void worker_main(sp_server* s) {
   cudaSetDevice(s->device);
   std::unique_lock<std::mutex> lk(s->mu);
   uint32_t idle_spins = 0;
+  uint64_t slept_on = UINT64_MAX;  // `published` when the worker last went to sleep
   while (!s->stop.load()) {
     bool progress = false;
     // deliver finished launches oldest first: a stream's frames can be in both
@@ -294,12 +296,17 @@ void worker_main(sp_server* s) {
       lk.lock();
     } else {
       idle_spins = 0;
+      // watch for the next request once after every one, then sleep
       const uint64_t seen = s->published.load(std::memory_order_acquire);
-      lk.unlock();
-      spin_while(s->published, seen);
-      lk.lock();
-      if (s->published.load(std::memory_order_acquire) == seen)
+      if (seen != slept_on) {
+        lk.unlock();
+        spin_while(s->published, seen);
+        lk.lock();
+      }
+      if (s->published.load(std::memory_order_acquire) == seen) {
+        slept_on = seen;
         s->cv_work.wait_for(lk, std::chrono::milliseconds(5));
+      }
     }
   }
 }
@@ -643,11 +650,13 @@ SP_API sp_status sp_server_poll(sp_server* s, sp_server_result* results, uint32_
   if (!s || !n_results || (!results && max_results)) return fail(SP_EINVAL, "NULL argument");
   *n_results = 0;
   std::unique_lock<std::mutex> lk(s->mu);
-  if (s->done.empty() && wait_ms) {
+  // only where a result is on its way, and only one of the waiting threads
+  if (s->done.empty() && wait_ms && s->submitted != s->completed && !s->poll_spins.exchange(true)) {
     const uint64_t seen = s->delivered.load(std::memory_order_acquire);
     lk.unlock();
     spin_while(s->delivered, seen);
     lk.lock();
+    s->poll_spins.store(false);
   }
   if (s->done.empty() && wait_ms)
     s->cv_done.wait_for(lk, std::chrono::milliseconds(wait_ms), [&] { return !s->done.empty(); });
