@@ -32,13 +32,14 @@
 // registers; at 96 registers (5 warps) the cascade spills: 105 and 204 us.
 #pragma once
 
+#include "sp_encode_rule.h"
 #include "sp_encode_strip.cuh"
 
 namespace sp {
 namespace enc {
 
 constexpr uint32_t kWarps = 2;     // independent warps of a CTA
-constexpr uint32_t kStrip = 240;   // output columns of a strip: lanes 1..30
+constexpr uint32_t kStrip = kEncodeStrip;  // output columns of a strip: lanes 1..30
 constexpr uint32_t kAll = 0xffffffffu;
 
 __host__ __device__ constexpr uint32_t binom(uint32_t n, uint32_t k) {
@@ -368,20 +369,25 @@ __global__ void __launch_bounds__(kWarps * 32, 8) sp_encode_kernel(const EncodeA
       reinterpret_cast<uint8_t*>(out)[b] = 0u;
 }
 
-// f is 1 or 2; a8: see the kernel.
+// f is 1 or 2; a8: see the kernel.  Unaligned RGB rows take the strip kernel up
+// to window 7 only (encode_in_strips).
 template <int B>
 cudaError_t launch_block(const EncodeArgs& a, bool a8, cudaStream_t st) {
   const uint32_t grid = (a.units + kWarps - 1u) / kWarps, threads = kWarps * 32;
-  if (a.ch == 3u && a.f == 1u) {
-    if (a8)
+  if (a.ch == 3u && a8) {
+    if (a.f == 1u)
       sp_encode_kernel<B, 3, 1, true><<<grid, threads, 0, st>>>(a);
     else
-      sp_encode_kernel<B, 3, 1, false><<<grid, threads, 0, st>>>(a);
-  } else if (a.ch == 3u) {
-    if (a8)
       sp_encode_kernel<B, 3, 2, true><<<grid, threads, 0, st>>>(a);
-    else
-      sp_encode_kernel<B, 3, 2, false><<<grid, threads, 0, st>>>(a);
+  } else if (a.ch == 3u) {
+    if constexpr (B <= 7) {
+      if (a.f == 1u)
+        sp_encode_kernel<B, 3, 1, false><<<grid, threads, 0, st>>>(a);
+      else
+        sp_encode_kernel<B, 3, 2, false><<<grid, threads, 0, st>>>(a);
+    } else {
+      return cudaErrorNotSupported;
+    }
   } else if (a.f == 1u) {
     if (a8)
       sp_encode_kernel<B, 1, 1, true><<<grid, threads, 0, st>>>(a);
