@@ -34,12 +34,6 @@ constexpr int kEncThreads = 512;
 constexpr uint32_t kEncSmemTarget = 100u << 10;  // two CTAs per SM
 constexpr uint32_t kEncSmemMax = 200u << 10;
 
-__host__ __device__ constexpr uint32_t binom(uint32_t n, uint32_t k) {
-  uint64_t r = 1;
-  for (uint32_t i = 1; i <= k; ++i) r = r * (n - k + i) / i;
-  return (uint32_t)r;
-}
-
 struct BandArgs {
   const uint8_t* src;
   uint64_t src_stride;  // bytes between frames

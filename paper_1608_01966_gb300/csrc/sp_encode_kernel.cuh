@@ -42,12 +42,6 @@ constexpr uint32_t kWarps = 2;     // independent warps of a CTA
 constexpr uint32_t kStrip = kEncodeStrip;  // output columns of a strip: lanes 1..30
 constexpr uint32_t kAll = 0xffffffffu;
 
-__host__ __device__ constexpr uint32_t binom(uint32_t n, uint32_t k) {
-  uint64_t r = 1;
-  for (uint32_t i = 1; i <= k; ++i) r = r * (n - k + i) / i;
-  return (uint32_t)r;
-}
-
 // Luma (77 R + 150 G + 29 B + 128) >> 8 of four pixels, given the sums before
 // the shift (16 bits each): their second bytes.
 __device__ __forceinline__ uint32_t pack_luma(uint32_t l0, uint32_t l1, uint32_t l2, uint32_t l3) {

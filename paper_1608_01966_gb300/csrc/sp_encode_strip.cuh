@@ -8,6 +8,13 @@
 
 namespace sp {
 
+// Weights of the encoder's window: row n of Pascal's triangle.
+__host__ __device__ constexpr uint32_t binom(uint32_t n, uint32_t k) {
+  uint64_t r = 1;
+  for (uint32_t i = 1; i <= k; ++i) r = r * (n - k + i) / i;
+  return (uint32_t)r;
+}
+
 struct EncodeArgs {
   const uint8_t* src;
   uint64_t src_stride;   // bytes between frames

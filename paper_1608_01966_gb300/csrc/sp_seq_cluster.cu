@@ -757,31 +757,9 @@ __global__ void __launch_bounds__(kSeqThreads + kSeqHelpers, 1) sp_seq_cluster_k
           if (warp < mw) {
             // T = the k-th largest count (0 when at most k columns count);
             // `need` of the `ties` columns at it win, in column order
-            uint32_t T = 0xffffffffu, need = 0u, ties = 0u;
-            const uint32_t k = a.k, c = c0 + 32u * warp + lane, v = s_cnt[c];
-            if (k != 0u) {
-              T = 0u;
-              uint32_t acc = 0u;
-              for (uint32_t b0 = hist[0]; b0 >= 1u; b0 = b0 > 32u ? b0 - 32u : 0u) {
-                const uint32_t bin = b0 > lane ? b0 - lane : 0u;
-                const uint32_t h = bin ? hist[bin] : 0u;
-                uint32_t inc = h;
-#pragma unroll
-                for (uint32_t o = 1; o < 32u; o <<= 1) {
-                  const uint32_t y = __shfl_up_sync(kFull, inc, o);
-                  if (lane >= o) inc += y;
-                }
-                const uint32_t hit = __ballot_sync(kFull, acc + inc >= k);
-                if (hit) {
-                  const int src = __ffs(hit) - 1;
-                  T = b0 - (uint32_t)src;
-                  ties = __shfl_sync(kFull, h, src);
-                  need = k - (acc + __shfl_sync(kFull, inc, src) - ties);
-                  break;
-                }
-                acc += __shfl_sync(kFull, inc, 31);
-              }
-            }
+            uint32_t T, need, ties;
+            const uint32_t v = s_cnt[c0 + 32u * warp + lane];
+            dev::warp_kth_count(hist, a.k, T, need, ties);
             const bool tie = T != 0u && v == T;
             bool win = T != 0xffffffffu && v > T;
             const uint32_t tw = __ballot_sync(kFull, tie);

@@ -444,12 +444,11 @@ __device__ __forceinline__ void publish_overlap(const StepArgs& a, uint32_t c, u
 // their boxes cover a band of consecutive frame rows: the band is copied to
 // shared memory once per item (one bulk copy).  Every warp then counts its
 // columns kWinCols at a time, their bitmaps loaded into registers (16 bytes
-// per lane and column, one coalesced request per column) -- with
-// SP_WIN_PIPE the next group's loads are issued before the current group is
-// counted.  Lane l of a column's warp counts rows l and l + 32 of its box: a
-// funnel shift aligns each 64-pixel row segment of the band to the box, an
-// AND with the bitmap row and a population count give the row's share of
-// Alg. 1's count.  No gather leaves shared memory.
+// per lane and column, one coalesced request per column).  Lane l of a
+// column's warp counts rows l and l + 32 of its box: a funnel shift aligns
+// each 64-pixel row segment of the band to the box, an AND with the bitmap
+// row and a population count give the row's share of Alg. 1's count.  No
+// gather leaves shared memory.
 //
 // Learning (the previous frame's winners, rare) runs first, CTA-wide: all
 // synapses of up to kWinLearn columns at once, a pass's indices and
@@ -462,9 +461,6 @@ __device__ __forceinline__ void publish_overlap(const StepArgs& a, uint32_t c, u
 
 #ifndef SP_WINDOW_COLS
 #define SP_WINDOW_COLS 4
-#endif
-#ifndef SP_WIN_PIPE
-#define SP_WIN_PIPE 0
 #endif
 constexpr int kWinCols = SP_WINDOW_COLS;  // columns per warp in flight
 constexpr uint32_t kWinLearn = 8;         // learners kept in shared memory
@@ -683,10 +679,6 @@ __device__ __forceinline__ void window_item(const StepArgs& a, uint32_t lo, uint
          (unsigned long long)__ballot_sync(kFull, i1 < n && s_lmap[i1] != 0u) << 32;
   }
   for (uint32_t c = c0; c < hi; c += COLS * kStepWarps, lm >>= COLS) {
-#if SP_WIN_PIPE
-    uint4 nx[COLS];
-    load_group(c + COLS * kStepWarps, nx);
-#endif
     uint32_t cnt[COLS];
 #pragma unroll
     for (int j = 0; j < COLS; ++j) {
@@ -714,12 +706,7 @@ __device__ __forceinline__ void window_item(const StepArgs& a, uint32_t lo, uint
     }
     if (lane < COLS && c + (uint32_t)lane * kStepWarps < hi)
       publish_overlap(a, c + (uint32_t)lane * kStepWarps, ok ? mine : 0u);
-#if SP_WIN_PIPE
-#pragma unroll
-    for (int j = 0; j < COLS; ++j) bm[j] = nx[j];
-#else
     load_group(c + COLS * kStepWarps, bm);
-#endif
   }
   __syncthreads();  // the band becomes the last CTA's working memory
   if (t == 0) mbar_inval(&s_bar_band);
