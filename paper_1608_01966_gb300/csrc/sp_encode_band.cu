@@ -1,6 +1,7 @@
 // Frame encoder, band kernel: colour frames -> reduction -> gray -> adaptive
-// Gaussian threshold -> packed input bits, for reductions by 3 and more and for
-// outputs narrower than a strip kernel's lane.
+// Gaussian threshold -> packed input bits, for the calls that strips are slower
+// on (sp_encode_rule.h): reductions by 3 and more, strips filled badly or with
+// rows slow to read, and outputs narrower than a strip kernel's lane.
 //
 // One CTA encodes a band of output rows of one frame.  It owns the output
 // words whose first pixel lies in the band; the last of them may run into

@@ -25,7 +25,7 @@
 // The weighted sum, its rounding and the comparison are exact integers as in
 // the definition: g + offset > floor((s + h) / 2^k) iff (g + offset) 2^k > s + h.
 //
-// 128 frames of 960 x 540 RGB, window 11: 84 us, 26 warp instructions per 32
+// 128 frames of 960 x 540 RGB, window 11: 86 us, 26 warp instructions per 32
 // pixels at 1.15 times the rows (halo); gray and vertical sums of a band in shared
 // memory, three barriers apart (sp_encode_band.cu), 211 us and 101.  64 frames of
 // 1920 x 1080 halved: 94 us (4.3 TB/s) against 529.  4 warps a scheduler at 128

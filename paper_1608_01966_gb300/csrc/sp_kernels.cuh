@@ -24,7 +24,7 @@ struct StepArgs {
   const uint32_t* idx;       // [C][S] input indices
   float* perm;               // [C][S] permanences (updated for pending learning)
   const float* boost;        // [C]
-  float* ov;                 // [C] boosted overlaps (out)
+  float* ov;                 // [C] boosted overlaps (out), on and padded to 16 bytes
   const uint32_t* x;         // this frame, packed bits
   const uint32_t* x_prev;    // previous frame (pending learning), or nullptr
   const uint32_t* mask_prev; // previous frame's winners (pending learning), or nullptr
@@ -170,8 +170,8 @@ cudaError_t launch_tick_gather(const TickItem* items, uint32_t count, TickMember
 cudaError_t launch_batch_step(const BatchArgs& a, uint32_t n_ctas, uint32_t max_C, uint32_t max_S,
                               cudaStream_t stream);
 // One persistent launch over r.n_frames batch frames (grid sized to the
-// resident CTAs) with compiled schedule `schedule` (0: the default; out of
-// range: the default); r.work and r.abort must be 0.
+// resident CTAs) with compiled schedule `schedule` (out of range: schedule 0);
+// r.work and r.abort must be 0.
 cudaError_t launch_batch_run(const BatchRunArgs& r, uint32_t max_C, uint32_t max_S,
                              uint32_t schedule, cudaStream_t stream);
 // The compiled schedules of the persistent batch pass: how many, and the
