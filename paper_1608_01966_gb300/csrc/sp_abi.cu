@@ -329,10 +329,12 @@ sp_status wait_handle(sp_handle* h) {
 
 // A call on a capturing stream is recorded into the caller's graph: from then
 // on a replay that the handle does not see may have written the last frame's
-// list, so it is read from the device.
+// list, so it is read from the device.  (The legacy stream cannot be captured,
+// and the handle's own only after a call on one that is.)
 void note_capture(sp_handle* h) {
+  if (h->captured || h->stream == h->own_stream || h->stream == cudaStreamLegacy) return;
   cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
-  if (!h->captured && cudaStreamIsCapturing(h->stream, &status) == cudaSuccess)
+  if (cudaStreamIsCapturing(h->stream, &status) == cudaSuccess)
     h->captured = status != cudaStreamCaptureStatusNone;
 }
 

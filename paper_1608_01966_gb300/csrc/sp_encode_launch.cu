@@ -13,13 +13,19 @@ cudaError_t launch_encode(EncodeArgs a, uint32_t block, cudaStream_t st) {
   const bool a8 = reinterpret_cast<uintptr_t>(a.src) % 8u == 0u && a.src_stride % 8u == 0u &&
                   (uint64_t)a.W * a.ch % 8u == 0u && a.Wr % 8u == 0u;
   a.strips = (a.Wr + kEncodeStrip - 1u) / kEncodeStrip;
-  int dev = 0, sms = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  if (e != cudaSuccess) return e;
+  // asked for where it is needed: the two calls take half a microsecond
+  int sms = 0;
+  auto ask_sms = [&]() {
+    int dev = 0;
+    const cudaError_t e = cudaGetDevice(&dev);
+    return e != cudaSuccess ? e : cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  };
+  cudaError_t e = cudaSuccess;
+  if (!a8 && a.ch == 3u && a.f == 2u && (e = ask_sms()) != cudaSuccess) return e;
   const bool words = a.src_stride % 4u == 0u && reinterpret_cast<uintptr_t>(a.src) % 4u == 0u;
   if (!encode_in_strips({a.W, a.ch, a.f, a.Wr, a.Hr, block, a.n_frames, a8, words, (uint32_t)sms}))
     return launch_encode_band(a, block, st);
+  if (sms == 0 && (e = ask_sms()) != cudaSuccess) return e;
   // Rows per chunk: every chunk reads block - 1 rows besides its own, a chunk
   // per warp; the fewest rows walked by the warps of a full machine in whole
   // waves (16 warps resident per SM, at 128 registers a thread)

@@ -16,7 +16,7 @@ struct EncodeShape {
   uint32_t n_frames;
   bool a8;              // rows, frames and strips on 8-byte boundaries, output rows whole bytes
   bool words;           // rows and frames on 4-byte boundaries
-  uint32_t sms;
+  uint32_t sms;         // of unaligned RGB halved; else it may be 0
 };
 
 // Whether the strip kernel takes the call (else the band kernel).  Blocks of 3 x

@@ -94,10 +94,12 @@ SP_API sp_status sp_step_noalloc(const sp_config* cfg, const uint32_t* d_idx, fl
   if (s != SP_OK) return s;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   auto* ticket = reinterpret_cast<unsigned long long*>(scratch + SP_NOALLOC_MAX_COLUMNS);
-  cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
-  if (cudaStreamIsCapturing(st, &capture) != cudaSuccess || capture != cudaStreamCaptureStatusNone)
-    if (cudaMemsetAsync(ticket, 0, sizeof(*ticket), st) != cudaSuccess)
-      return noalloc_fail(SP_ECUDA, "clearing the scratch counter failed");
+  if (st && st != cudaStreamLegacy) {  // the legacy stream cannot be captured
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &capture) != cudaSuccess || capture != cudaStreamCaptureStatusNone)
+      if (cudaMemsetAsync(ticket, 0, sizeof(*ticket), st) != cudaSuccess)
+        return noalloc_fail(SP_ECUDA, "clearing the scratch counter failed");
+  }
 
   sp::StepArgs a{};
   a.idx = d_idx;
