@@ -715,7 +715,7 @@ __device__ __forceinline__ void window_item(const StepArgs& a, uint32_t lo, uint
 // One frame of one SP, run by nb CTAs of which this is number bid.  With
 // STAGE, a CTA whose columns' state fits in stage_cap bytes of dynamic
 // shared memory stages it there by bulk copy first.
-template <int VEC, bool STREAM, bool STAGE = false, int COLS = kCompactCols>
+template <int VEC, bool STREAM, bool STAGE = false, int COLS = kCompactCols, bool TICKET = false>
 __device__ __forceinline__ void step_body(const StepArgs& a, uint32_t bid, uint32_t nb,
                                           uint32_t* dyn_smem, uint32_t stage_cap = 0u,
                                           uint32_t* err = nullptr, uint32_t xspan_cap = 0u,
@@ -933,7 +933,7 @@ __device__ __forceinline__ void step_body(const StepArgs& a, uint32_t bid, uint3
   __syncthreads();
   if (threadIdx.x == 0) {
     __threadfence();
-    if (a.ticket) {
+    if (TICKET) {
       // both by this thread on one word, so in this order
       atomicMax(a.ticket, a.ticket_base);
       s_ticket = (uint32_t)(atomicAdd(a.ticket, 1ull) - a.ticket_base);
@@ -946,7 +946,7 @@ __device__ __forceinline__ void step_body(const StepArgs& a, uint32_t bid, uint3
   __threadfence();
   const uint32_t* smask = last_cta_inhibit(a, dyn_smem);
   if (threadIdx.x == 0) {
-    if (a.ticket)
+    if (TICKET)
       atomicExch(a.ticket, 0ull);
     else
       atomicExch(a.counter, 0u);
@@ -964,10 +964,12 @@ __device__ __forceinline__ void step_body(const StepArgs& a, uint32_t bid, uint3
   if (a.learn_next) prefetch_winners(a, smask);
 }
 
-template <int VEC>
+// TICKET: the CTAs' tickets come from a.ticket (its own instance: the choice in
+// the kernel cost a frame of 900 x 143 0.3 us).
+template <int VEC, bool TICKET>
 __global__ void __launch_bounds__(kStepThreads) sp_step_kernel(const StepArgs a) {
   extern __shared__ __align__(128) uint32_t dyn_smem[];
-  step_body<VEC, false>(a, blockIdx.x, gridDim.x, dyn_smem);
+  step_body<VEC, false, false, kCompactCols, TICKET>(a, blockIdx.x, gridDim.x, dyn_smem);
 }
 
 // Resident CTAs per SM the batch kernel is compiled for (register budget).
@@ -1027,7 +1029,6 @@ __global__ void __launch_bounds__(kStepThreads, SP_BATCH_MIN_BLOCKS) sp_batch_st
   a.ov_copy = (ba.ov_out && !ba.tick) ? ba.ov_out + d.ov_off : nullptr;
   a.result = d.result;
   a.counter = d.counter;
-  a.ticket = nullptr;
   a.hist = d.hist;
   a.duty = d.duty;
   a.duty_period = d.duty_period;
@@ -1169,7 +1170,6 @@ __global__ void __launch_bounds__(kStepThreads, MINB) sp_batch_run_kernel(const 
     a.ov_copy = r.ov_out ? r.ov_out + (uint64_t)t * r.ov_stride + d.ov_off : nullptr;
     a.result = d.result;
     a.counter = d.counter;
-    a.ticket = nullptr;
     a.hist = d.hist;
     a.duty = d.duty;
     a.duty_period = d.duty_period;
@@ -1256,18 +1256,16 @@ bool batch_schedule(uint32_t i, uint32_t* ctas_per_sm, uint32_t* cols_in_flight)
 
 cudaError_t kernels_init() {
   const int bytes = (int)step_smem_bytes(SP_MAX_COLUMNS, kStepBins);
-  cudaError_t e = cudaFuncSetAttribute(sp_step_kernel<4>,
+  cudaError_t e = cudaFuncSetAttribute(sp_batch_step_kernel,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-  if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(sp_batch_step_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           bytes);
-  if (e != cudaSuccess) return e;
+  for (auto k : {sp_step_kernel<4, false>, sp_step_kernel<4, true>, sp_step_kernel<1, false>,
+                 sp_step_kernel<1, true>})
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
   for (uint32_t i = 0; i < kNumRunSchedules && e == cudaSuccess; ++i)
     e = cudaFuncSetAttribute(kRunSchedules[i].kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              bytes);
-  if (e != cudaSuccess) return e;
-  return cudaFuncSetAttribute(sp_step_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              bytes);
+  return e;
 }
 
 // One warp per column: base, 16-bit offsets and connected bits.
@@ -1524,9 +1522,11 @@ cudaError_t launch_batch_step(const BatchArgs& a, uint32_t n_ctas, uint32_t max_
 cudaError_t launch_step(const StepArgs& a, int grid, cudaStream_t stream) {
   const size_t smem = step_smem_bytes(a.C, a.S);
   if (a.S % 4u == 0u)
-    sp_step_kernel<4><<<grid, kStepThreads, smem, stream>>>(a);
+    (a.ticket ? sp_step_kernel<4, true> : sp_step_kernel<4, false>)<<<grid, kStepThreads, smem,
+                                                                      stream>>>(a);
   else
-    sp_step_kernel<1><<<grid, kStepThreads, smem, stream>>>(a);
+    (a.ticket ? sp_step_kernel<1, true> : sp_step_kernel<1, false>)<<<grid, kStepThreads, smem,
+                                                                      stream>>>(a);
   g_launches.fetch_add(1, std::memory_order_relaxed);
   return cudaGetLastError();
 }
