@@ -33,7 +33,7 @@ struct StepArgs {
   uint32_t* mask_copy;       // optional second copy of the mask (caller array), or nullptr
   uint32_t* result;          // [0] = number of winners, [1..] ascending winners
   uint32_t* counter;         // last-CTA ticket, 0 between launches
-  unsigned long long* ticket;  // or, where the word may hold anything below
+  unsigned long long* ticket;  // or nullptr; a word that may hold anything below
   unsigned long long ticket_base;  // ticket_base: counted from there, then left 0
   uint32_t* hist;            // [S + 1] counts of surviving raw overlaps, 0 between
                              // launches; used (global inhibition) when every boost
